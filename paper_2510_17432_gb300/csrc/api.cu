@@ -353,11 +353,60 @@ __global__ void k_make_diag(int64_t n, const double* v64, double H0, double half
 }
 
 // ------------------------------------------------------------------ initial states
+// exp(2 pi i u / 2^32) * (sh + sl) in FP32 with an error below 0.5 ulp + 2^-10 ulp: the draw is reduced
+// exactly to a quarter turn (an integer below 2^29, split exactly into two floats), sin and cos
+// of the remainder |x| <= 1/4 (in units of pi) come from their Taylor series, whose first three
+// (sine) and four (cosine) terms are summed in float pairs (h + l) and the rest in FP32, where their
+// weight keeps the error below 2^-36, and the scale is applied to the pair before the one rounding.
+struct F2 {
+  float h, l;
+};
+// c + z s for float pairs with |c| >= |z s|
+__host__ __device__ __forceinline__ F2 pair_step(F2 c, F2 z, F2 s) {
+  const float p = z.h * s.h;
+  const float e = fmaf(z.h, s.h, -p) + fmaf(z.l, s.h, z.h * s.l);
+  const float h = c.h + p;
+  return {h, (c.h - h) + p + (c.l + e)};
+}
+__host__ __device__ __forceinline__ float2 unit_phase(uint32_t u, float sh, float sl) {
+  const uint32_t q = (u + 0x20000000u) >> 30;
+  const int r = (int)(u - (q << 30));  // [-2^29, 2^29)
+  const float xi = (float)r;
+  const F2 x = {xi * 0x1p-31f, (float)(r - (int)xi) * 0x1p-31f};
+  F2 z;
+  z.h = x.h * x.h;
+  z.l = fmaf(x.h, x.h, -z.h) + 2.f * x.h * x.l;
+  // pi^(2k+1)/(2k+1)! and pi^(2k)/(2k)!, alternating
+  float t = fmaf(z.h, -2.19153535e-05f, 4.66302794e-04f);
+  t = fmaf(z.h, t, -7.37043098e-03f);
+  t = fmaf(z.h, t, 8.21458846e-02f);
+  t = fmaf(z.h, t, -5.99264503e-01f);
+  F2 s = pair_step({2.55016398f, 5.55786386e-08f}, z, {t, 0.f});
+  s = pair_step({-5.16771269f, -9.16039227e-08f}, z, s);
+  s = pair_step({3.14159274f, -8.74227766e-08f}, z, s);
+  const float ph = x.h * s.h;  // sin = x s
+  s = {ph, fmaf(x.h, s.h, -ph) + fmaf(x.l, s.h, x.h * s.l)};
+  t = fmaf(z.h, -1.04638108e-04f, 1.9295743e-03f);
+  t = fmaf(z.h, t, -2.58068908e-02f);
+  t = fmaf(z.h, t, 2.35330626e-01f);
+  F2 c = pair_step({-1.33526278f, 6.56655308e-09f}, z, {t, 0.f});
+  c = pair_step({4.05871201f, 1.20801531e-07f}, z, c);
+  c = pair_step({-4.93480206f, -1.45185794e-07f}, z, c);
+  c = pair_step({1.f, 0.f}, z, c);
+  const float cs = fmaf(c.h, sh, fmaf(c.h, sl, c.l * sh));
+  const float sn = fmaf(s.h, sh, fmaf(s.h, sl, s.l * sh));
+  const float a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;  // quarter turns: (c, s), (-s, c), (-c, -s), (s, -c)
+  return make_float2((q == 1 || q == 2) ? -a : a, q >= 2 && q < 4 ? -b : b);
+}
+
 // Random phases psi_i = exp(2 pi i u / 2^32) / sqrt(N), u = Philox(state_seed; i, 2, s).
+// complex64 is bound by the draw (integer multiplies) and FP32 issue: 537M states take 3.2 ms against 31.1 ms
+// with FP64 sincospi (GB300 issues two FP64 operations per clock and SM), which complex128 keeps.
 template <typename R>
 __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint64_t seed, const int64_t* full_of,
                               double inv_sqrt_n, R* out, uint32_t* draws) {
   const int64_t total = n * Spad;
+  const float sh = (float)inv_sqrt_n, sl = (float)(inv_sqrt_n - (double)sh);
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t k = e >> logS;
@@ -366,14 +415,23 @@ __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint
     if (s < S) {
       const int64_t f = full_of ? full_of[k] : k;
       const uint32_t u = draw_u32(seed, (uint64_t)f, STREAM_PHASE, (uint32_t)(s0 + s));
-      double sn, cs;
-      sincospi((double)u * 0x1p-31, &sn, &cs);
-      re = (R)(cs * inv_sqrt_n);
-      im = (R)(sn * inv_sqrt_n);
+      if constexpr (sizeof(R) == 4) {
+        const float2 v = unit_phase(u, sh, sl);
+        re = v.x;
+        im = v.y;
+      } else {
+        double sn, cs;
+        sincospi((double)u * 0x1p-31, &sn, &cs);
+        re = (R)(cs * inv_sqrt_n);
+        im = (R)(sn * inv_sqrt_n);
+      }
       if (draws) draws[(int64_t)s * n + k] = u;
     }
-    out[2 * e] = re;
-    out[2 * e + 1] = im;
+    if constexpr (sizeof(R) == 4) {
+      reinterpret_cast<float2*>(out)[e] = make_float2(re, im);
+    } else {
+      reinterpret_cast<double2*>(out)[e] = make_double2(re, im);
+    }
   }
 }
 
