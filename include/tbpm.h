@@ -165,7 +165,11 @@ int tbpm_sync(tbpm_ctx* ctx);
 int64_t tbpm_launch_count(const tbpm_ctx* ctx);
 /* Temporal fusion of the moment pass (several Chebyshev steps per pass, so each state vector
  * crosses HBM twice per pass instead of three times per step), used where a fused kernel exists
- * (honeycomb stencil, complex64, S >= 2, lattice at least 48 x 32 cells).
+ * (complex64; honeycomb stencil with S >= 2, lattice at least 48 x 32 cells; in modes 8 to 10 also the
+ * honeycomb with one state and at least 128 cells per row, square lattices of at least 96 rows and 96
+ * sites per row and one 128-thread band wide, and, on the automatic path, honeycomb and square
+ * lattices with at most half their sites vacant: there the vacant sites keep their place in the state
+ * blocks with amplitude zero).
  * mode: 0 = one step per pass; 1 = 4 steps per pass (2-D tiles); 2 = 2 steps per pass (2-D tiles);
  * 3, 4 = 2 steps per pass by a row sweep (bands of cells, rows of phi_n streamed through a
  * shared-memory ring one row ahead, each further step one row behind the previous; 128- and

@@ -404,7 +404,7 @@ __host__ __device__ __forceinline__ float2 unit_phase(uint32_t u, float sh, floa
 // with FP64 sincospi (GB300 issues two FP64 operations per clock and SM), which complex128 keeps.
 template <typename R>
 __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint64_t seed, const int64_t* full_of,
-                              double inv_sqrt_n, R* out, uint32_t* draws) {
+                              const float* masked, double inv_sqrt_n, R* out, uint32_t* draws) {
   const int64_t total = n * Spad;
   const float sh = (float)inv_sqrt_n, sl = (float)(inv_sqrt_n - (double)sh);
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -412,7 +412,7 @@ __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint
     const int64_t k = e >> logS;
     const int s = (int)(e & (Spad - 1));
     R re = R(0), im = R(0);
-    if (s < S) {
+    if (s < S && !(masked && isnan(masked[k]))) {  // vacant sites of the full layout stay zero
       const int64_t f = full_of ? full_of[k] : k;
       const uint32_t u = draw_u32(seed, (uint64_t)f, STREAM_PHASE, (uint32_t)(s0 + s));
       if constexpr (sizeof(R) == 4) {
@@ -436,10 +436,28 @@ __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint
 }
 
 template <typename R>
-__global__ void k_init_sites(int64_t n, int Spad, int S, const int64_t* sites, R* out) {
+__global__ void k_init_sites(int64_t n, int Spad, int S, const int64_t* sites, const int64_t* full_of, R* out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
-  out[2 * (sites[s] * Spad + s)] = R(1);
+  const int64_t i = full_of ? full_of[sites[s]] : sites[s];
+  out[2 * (i * Spad + s)] = R(1);
+}
+
+// D_i by full site index for the masked stencil, NaN at vacant sites.
+__global__ void k_make_dfull(int64_t n_full, const int64_t* compact, const float* d32, float dconst, float* out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_full; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t c = compact[i];
+    out[i] = c < 0 ? __int_as_float(0x7fc00000) : (d32 ? d32[c] : dconst);
+  }
+}
+
+// State blocks of a full-layout pass back in the compact order of the active sites (16- or 8-byte units).
+template <typename T>
+__global__ void k_compact_states(int64_t n, int P, const int64_t* full_of, const T* in, T* out) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n * P; u += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = u / P;
+    out[u] = in[full_of[k] * P + (u - k * P)];
+  }
 }
 
 }  // namespace tbpm
@@ -878,10 +896,20 @@ static int ensure_d64(tbpm_lattice* lat) {
   return TBPM_OK;
 }
 
+static int ensure_dfull(tbpm_lattice* lat) {
+  if (lat->dfull) return TBPM_OK;
+  tbpm_ctx* ctx = lat->ctx;
+  TBPM_TRY(dev_alloc(ctx, &lat->dfull, lat->geom.n_full));
+  k_make_dfull<<<grid_for(ctx, lat->geom.n_full, kT), kT, 0, ctx->stream>>>(
+      lat->geom.n_full, lat->compact, lat->d32, (float)((0.0 - lat->H0) / lat->half), lat->dfull);
+  TBPM_CK_LAUNCH(ctx);
+  return TBPM_OK;
+}
+
 static void free_lattice_mem(tbpm_lattice* lat) {
   tbpm_ctx* ctx = lat->ctx;
   void* ps[] = {lat->d32, lat->d64, lat->v64, lat->ell, lat->compact, lat->full_of, lat->wrel32, lat->wrel64,
-                lat->chunks, lat->jw};
+                lat->chunks, lat->jw, lat->dfull};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, ctx->stream);
 }
@@ -1073,7 +1101,29 @@ struct Plan {
   size_t state_bytes; // one block of Spad states
   double tau;
   int s0;             // index of the block's first state among the request's states (Philox sub-stream)
+  int64_t n;          // sites of a state block: the active sites, or all of them in the full layout
+  bool full;          // vacancy lattice on the masked stencil: blocks by full site index, vacant sites zero
 };
+
+void set_layout(const tbpm_lattice* lat, Plan* pl, bool full) {
+  pl->full = full;
+  pl->n = full ? lat->geom.n_full : lat->n_sites;
+  pl->state_bytes = (size_t)pl->n * pl->Spad * pl->elem;
+}
+
+// Whether a nearest-neighbour vacancy lattice takes the masked register sweep: automatic path, a shape
+// the sweep takes, and at most half the sites vacant.  In the full layout a step costs 8 B per
+// (site + vacancy) and 4 / S B of D_i where the index lists cost 24 + (4 z + 4) / S B per site, so the
+// sweep would win beyond half as well; the rule keeps the extra state memory below the lists' own scale.
+bool masked_sweep_ok(const tbpm_lattice* lat, const Plan& pl) {
+  return lat->path == TBPM_PATH_CSR && lat->desc.path == TBPM_PATH_AUTO && lat->desc.vacancy_frac > 0.0 &&
+         2 * lat->n_sites >= lat->geom.n_full && sweep_shape_ok(lat, pl.precision, pl.Spad);
+}
+
+// The register sweep carries this plan's recurrence.
+bool sweep_ok(const tbpm_lattice* lat, const Plan& pl) {
+  return (lat->path == TBPM_PATH_STENCIL || pl.full) && sweep_shape_ok(lat, pl.precision, pl.Spad);
+}
 
 int ilog2(int v) {
   int r = 0;
@@ -1116,7 +1166,7 @@ int make_plan(const tbpm_lattice* lat, const tbpm_request* req, Plan* pl) {
   pl->P = pl->Spad / pl->spt;
   pl->logP = ilog2(pl->P);
   pl->elem = req->precision == TBPM_C64 ? 8 : 16;
-  pl->state_bytes = (size_t)lat->n_sites * pl->Spad * pl->elem;
+  set_layout(lat, pl, false);
   pl->tau = req->tau == 0.0 ? M_PI : req->tau;
   pl->s0 = 0;
   if (!(pl->tau > 0.0) || !isfinite(pl->tau)) {
@@ -1128,39 +1178,43 @@ int make_plan(const tbpm_lattice* lat, const tbpm_request* req, Plan* pl) {
 
 int init_states(tbpm_ctx* ctx, const tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, void* dst,
                 uint32_t* draws) {
-  const int64_t n = lat->n_sites;
+  const int64_t n = pl.n;
+  const int64_t* full_of = pl.full ? nullptr : lat->full_of;
+  const float* masked = pl.full ? lat->dfull : nullptr;
   if (req->states == TBPM_STATES_RANDOM) {
-    const double inv = 1.0 / sqrt((double)n);
+    const double inv = 1.0 / sqrt((double)lat->n_sites);
     const int nb = grid_for(ctx, n * pl.Spad, kT, 32);
     if (pl.precision == TBPM_C64)
-      k_init_random<float><<<nb, kT, 0, ctx->stream>>>(n, pl.Spad, pl.logS, pl.S, pl.s0, req->state_seed, lat->full_of,
-                                                       inv, (float*)dst, draws);
+      k_init_random<float><<<nb, kT, 0, ctx->stream>>>(n, pl.Spad, pl.logS, pl.S, pl.s0, req->state_seed, full_of,
+                                                       masked, inv, (float*)dst, draws);
     else
-      k_init_random<double><<<nb, kT, 0, ctx->stream>>>(n, pl.Spad, pl.logS, pl.S, pl.s0, req->state_seed, lat->full_of,
-                                                        inv, (double*)dst, draws);
+      k_init_random<double><<<nb, kT, 0, ctx->stream>>>(n, pl.Spad, pl.logS, pl.S, pl.s0, req->state_seed, full_of,
+                                                        masked, inv, (double*)dst, draws);
     TBPM_CK_LAUNCH(ctx);
   } else {
     TBPM_CK(cudaMemsetAsync(dst, 0, pl.state_bytes, ctx->stream));
     TBPM_TRY(ensure(ctx, ctx->ws_aux, sizeof(int64_t) * 32));
     TBPM_CK(cudaMemcpyAsync(ctx->ws_aux.p, req->sites, sizeof(int64_t) * pl.S, cudaMemcpyHostToDevice, ctx->stream));
     if (pl.precision == TBPM_C64)
-      k_init_sites<float><<<1, 32, 0, ctx->stream>>>(n, pl.Spad, pl.S, (const int64_t*)ctx->ws_aux.p, (float*)dst);
+      k_init_sites<float><<<1, 32, 0, ctx->stream>>>(n, pl.Spad, pl.S, (const int64_t*)ctx->ws_aux.p,
+                                                     pl.full ? lat->full_of : nullptr, (float*)dst);
     else
-      k_init_sites<double><<<1, 32, 0, ctx->stream>>>(n, pl.Spad, pl.S, (const int64_t*)ctx->ws_aux.p, (double*)dst);
+      k_init_sites<double><<<1, 32, 0, ctx->stream>>>(n, pl.Spad, pl.S, (const int64_t*)ctx->ws_aux.p, nullptr,
+                                                      (double*)dst);
     TBPM_CK_LAUNCH(ctx);
   }
   return TBPM_OK;
 }
 
 int64_t tiles_of(const tbpm_lattice* lat, const Plan& pl) {
-  if (lat->path == TBPM_PATH_CSR) return (lat->n_sites * pl.P + 255) / 256;
+  if (lat->path == TBPM_PATH_CSR && !pl.full) return (lat->n_sites * pl.P + 255) / 256;
   return lat->geom.n_rows * ((lat->geom.row_sites * pl.P + 255) / 256);
 }
 
 int base_args(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pl, RecurrenceArgs* a, int comps) {
   memset(a, 0, sizeof(*a));
   a->geom = lat->geom;
-  a->path = lat->path;
+  a->path = pl.full ? TBPM_PATH_STENCIL : lat->path;
   a->wrel = lat->wrel64 ? (pl.precision == TBPM_C128 ? (const void*)lat->wrel64 : (const void*)lat->wrel32) : nullptr;
   if (lat->chunks && pl.precision == TBPM_C64 && pl.Spad >= 2) {
     a->taps = lat->chunks;
@@ -1172,7 +1226,11 @@ int base_args(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pl, RecurrenceArgs* 
   }
   if (!a->taps) TBPM_TRY(ensure_ell(ctx, lat));
   a->ell = lat->ell;
-  if (lat->has_v) {
+  if (pl.full) {
+    TBPM_TRY(ensure_dfull(lat));
+    a->diag = lat->dfull;
+    a->masked = 1;
+  } else if (lat->has_v) {
     if (pl.precision == TBPM_C128) TBPM_TRY(ensure_d64(lat));
     a->diag = pl.precision == TBPM_C128 ? (const void*)lat->d64 : (const void*)lat->d32;
   } else {
@@ -1181,7 +1239,7 @@ int base_args(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pl, RecurrenceArgs* 
   a->diag_const = (0.0 - lat->H0) / lat->half;
   a->thop = lat->desc.t / lat->half;
   set_float_coefficients(a);
-  a->n_sites = lat->n_sites;
+  a->n_sites = pl.n;
   a->S = pl.Spad;
   a->P = pl.P;
   a->logP = pl.logP;
@@ -1209,7 +1267,11 @@ int choose_fusion(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, con
     return TBPM_OK;
   }
   *mode = 0;
-  if (!fused_applicable(lat, pl.precision, pl.Spad) || M / 2 < 64) return TBPM_OK;
+  if (!fused_applicable(lat, pl.precision, pl.Spad)) {  // square, vacancy and one-state sweeps: no other fused pass
+    *mode = 8;
+    return TBPM_OK;
+  }
+  if (M / 2 < 64) return TBPM_OK;
   const Geom& g = lat->geom;
   const std::vector<int64_t> key = {g.kind, g.Lx, g.Ly, g.Lz, g.pbc_x | (g.pbc_y << 1) | (g.pbc_z << 2), lat->path,
                                     pl.Spad, pl.precision, lat->has_v ? 1 : 0};
@@ -1288,33 +1350,63 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
 }
 
 // Moments of all Spad states into d_mu [Spad][M][2].
-int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int64_t M,
+int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl_in, int64_t M,
                 double* d_mu) {
   if (M < 2 || (M & 1)) {
     set_error("n_moments must be even and >= 2 (got %lld)", (long long)M);
     return TBPM_EINVAL;
   }
+  Plan pl = pl_in;
+  int fmode = 0;
+  TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));
+  const int64_t steps = M / 2;
+  const int K = fused_steps(fmode);
+  if (fmode >= 8 && steps - 1 >= K && masked_sweep_ok(lat, pl)) {
+    set_layout(lat, &pl, true);
+    TBPM_TRY(ensure_dfull(lat));
+  }
+  const int band = (fmode == 9 ? 192 : fmode == 10 ? 256 : 128) / std::max(1, pl.Spad / 2);
+  const bool wide_ok = fmode == 8 || lat->geom.kind != TBPM_HONEYCOMB || pl.Spad < 2 || lat->geom.Lx >= band;
+  const bool sweep = fmode >= 8 && steps - 1 >= K && wide_ok && sweep_ok(lat, pl);
+  const bool fuse = !sweep && fmode > 0 && fused_applicable(lat, pl.precision, pl.Spad) && steps - 1 >= K;
   TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
+  if (fuse || sweep) {
+    TBPM_TRY(ensure(ctx, ctx->ws_phi2[0], pl.state_bytes));
+    TBPM_TRY(ensure(ctx, ctx->ws_phi2[1], pl.state_bytes));
+  }
   TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
   RecurrenceArgs a;
   TBPM_TRY(base_args(ctx, lat, pl, &a, 3));
   a.mu = d_mu;
   a.M = (int)M;
-  int fmode = 0;
-  TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));
-  const int K = fused_steps(fmode);
-  const bool fuse = fmode > 0 && fused_applicable(lat, pl.precision, pl.Spad) && M / 2 - 1 >= K;
-  if (fuse) {
-    TBPM_TRY(ensure(ctx, ctx->ws_phi2[0], pl.state_bytes));
-    TBPM_TRY(ensure(ctx, ctx->ws_phi2[1], pl.state_bytes));
-  }
   // the pass sequence: step n reads cur = phi_n and overwrites prev (phi_{n-1}) with phi_{n+1}
   bool capturing = false;
   auto body = [&]() -> int {
     void* cur = ctx->ws_phi[0].p;
     void* prev = ctx->ws_phi[1].p;
+    void* pair_out[2] = {ctx->ws_phi2[0].p, ctx->ws_phi2[1].p};
     int64_t n = 0;
+    auto advance = [&](int steps_done) {
+      std::swap(prev, pair_out[0]);
+      std::swap(cur, pair_out[1]);
+      n += steps_done;
+    };
+    if (sweep) {
+      // every step through the register sweep: the first pass starts from phi_0 alone, the last
+      // one may need fewer steps and stores no state
+      const int ftok = phase_begin(ctx, 2);
+      while (n < steps) {
+        const int nk = (int)std::min<int64_t>(K, steps - n);
+        const bool last = n + K >= steps;
+        TBPM_TRY(launch_sweep_pass(ctx, lat, a, prev, cur, last ? nullptr : pair_out[0], last ? nullptr : pair_out[1],
+                                   (int)n, nk, fmode));
+        throttle_queue(ctx, capturing);
+        advance(K);
+      }
+      phase_end(ctx, ftok);
+      return TBPM_OK;
+    }
     auto unfused = [&]() -> int {
       a.cur = cur;
       a.prev_out = prev;
@@ -1328,21 +1420,14 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     TBPM_TRY(unfused());  // phi_1 = H~ phi_0, m_0, m_1
     if (fuse) {
       const int ftok = phase_begin(ctx, 2);
-      void* pair_out[2] = {ctx->ws_phi2[0].p, ctx->ws_phi2[1].p};
-      while (n + K <= M / 2) {
+      while (n + K <= steps) {
         TBPM_TRY(launch_fused_pass(ctx, lat, a, prev, cur, pair_out[0], pair_out[1], (int)n, fmode));
         throttle_queue(ctx, capturing);
-        void* old_prev = prev;
-        void* old_cur = cur;
-        prev = pair_out[0];
-        cur = pair_out[1];
-        pair_out[0] = old_prev;
-        pair_out[1] = old_cur;
-        n += K;
+        advance(K);
       }
       phase_end(ctx, ftok);
     }
-    while (n < M / 2) TBPM_TRY(unfused());
+    while (n < steps) TBPM_TRY(unfused());
     return TBPM_OK;
   };
   const int tok = phase_begin(ctx, 0);
@@ -1361,10 +1446,10 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     const std::vector<uint64_t> key = {
         (uint64_t)ctx->ws_phi[0].p, (uint64_t)ctx->ws_phi[1].p, (uint64_t)ctx->ws_phi2[0].p,
         (uint64_t)ctx->ws_phi2[1].p, (uint64_t)d_mu, (uint64_t)lat, (uint64_t)lat->d32, (uint64_t)lat->d64,
-        (uint64_t)lat->ell, (uint64_t)a.partials, (uint64_t)a.counter, (uint64_t)ctx->ws_fused_partials.p,
+        (uint64_t)lat->ell, (uint64_t)lat->dfull, (uint64_t)pl.full, (uint64_t)a.partials, (uint64_t)a.counter, (uint64_t)ctx->ws_fused_partials.p,
         (uint64_t)M, (uint64_t)fmode, (uint64_t)pl.precision, (uint64_t)pl.Spad, bits(a.thop), bits(a.diag_const),
         (uint64_t)g.Lx, (uint64_t)g.Ly, (uint64_t)g.Lz, (uint64_t)g.kind,
-        (uint64_t)(g.pbc_x | (g.pbc_y << 1) | (g.pbc_z << 2)), (uint64_t)lat->path, (uint64_t)lat->n_sites,
+        (uint64_t)(g.pbc_x | (g.pbc_y << 1) | (g.pbc_z << 2)), (uint64_t)lat->path, (uint64_t)pl.n,
         (uint64_t)lat->chunks, (uint64_t)a.taps_rx, (uint64_t)a.taps_ry, (uint64_t)a.taps_n0, (uint64_t)a.taps_n1,
         (uint64_t)a.taps_exact,
         (uint64_t)lat->wrel32, (uint64_t)lat->wrel64};
@@ -1469,7 +1554,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
   memset(&g, 0, sizeof(g));
   TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
   g.acc = ctx->ws_acc.p;
-  g.acc_stride = lat->n_sites * (int64_t)pl.Spad;
+  g.acc_stride = pl.n * (int64_t)pl.Spad;
   g.coef = (const double*)ctx->ws_table.p;
   g.psi = ctx->ws_psi.p;
   g.j_done = -1;
@@ -1499,6 +1584,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
   // buffered blocks: a step is the recurrence into a buffer slot plus its share of the flush's
   // slot reads; an accumulator update is the flush's extra cost per accumulator and term
   const int Tm = 8;
+  const bool sweep = sweep_ok(lat, pl);
   if (r == TBPM_OK && ctx->buffer_blocks && k_acc >= 2 &&
       ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)Tm) == TBPM_OK &&
       ensure(ctx, ctx->ws_blk_coef, sizeof(double) * 2 * (size_t)Tm * k_acc) == TBPM_OK) {
@@ -1514,7 +1600,15 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
       g.j_lo = 0;
       g.r.next = ctx->ws_blk.p;
       cudaEventRecord(e[0], ctx->stream);
-      for (int i = 0; i < reps && r == TBPM_OK; ++i) r = launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
+      for (int i = 0; i < reps && r == TBPM_OK; ++i) {
+        if (sweep) {  // four terms per window pass
+          char* w0 = (char*)ctx->ws_blk.p;
+          void* const w[4] = {w0, w0 + pl.state_bytes, w0 + 2 * pl.state_bytes, w0 + 3 * pl.state_bytes};
+          r = launch_sweep_window(ctx, lat, g.r, ctx->ws_phi[1].p, ctx->ws_phi[0].p, w, false);
+        } else {
+          r = launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
+        }
+      }
       cudaEventRecord(e[1], ctx->stream);
       // both flushes in the 16-accumulator tile of the block sizes being chosen between, so that
       // the difference is the cost of the extra accumulators, not of another kernel
@@ -1537,7 +1631,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
     }
     g.r.next = nullptr;
     if (r == TBPM_OK) {
-      const double rec = m[0] / reps, f1 = m[1] / reps, fk = m[2] / reps;
+      const double rec = m[0] / reps / (sweep ? 4 : 1), f1 = m[1] / reps, fk = m[2] / reps;
       *t_amxsy = rec + f1 / Tm;
       *t_axpy = std::max(1e-6, (fk - f1) / ((double)(k_acc - 1) * Tm));
     }
@@ -1567,6 +1661,57 @@ int choose_block(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
 // psi(t_{start+bb}) as bb consecutive state blocks.  init (device, optional) replaces the
 // request's initial states.
 using BlockHook = std::function<int(int64_t /*start*/, int /*bb*/, const void* /*first state block*/)>;
+
+// The Chebyshev vectors phi_0 .. phi_{n_terms-1} in windows of T buffer slots: slot 2 holds phi_0 on
+// entry, slot 2 + k holds term n0 + k, slots 0 and 1 carry the two latest vectors of the previous
+// window; flush(n0, nt) takes the nt terms from n0 on out of slot 2 ....  Where the register sweep
+// applies, four terms at a time come from one window pass (phi_n and phi_{n-1} read once for four
+// slots), else one term per pass.
+using WindowFlush = std::function<int(int64_t /*n0*/, int /*nt*/)>;
+
+int walk_windows(tbpm_ctx* ctx, tbpm_lattice* lat, const RecurrenceArgs& r, const Plan& pl, char* slots, int T,
+                 int64_t n_terms, const WindowFlush& flush) {
+  const bool sweep = sweep_ok(lat, pl);
+  AccumArgs g;
+  memset(&g, 0, sizeof(g));
+  g.r = r;
+  g.j_done = -1;
+  auto slot = [&](int64_t k) { return (void*)(slots + (size_t)k * pl.state_bytes); };
+  int64_t n0 = 0;
+  auto slot_of = [&](int64_t m) { return m >= n0 ? slot(2 + (m - n0)) : (m == n0 - 1 ? slot(1) : slot(0)); };
+  for (int64_t n = 1; n < n_terms;) {
+    if (n - n0 == T) {
+      TBPM_TRY(flush(n0, T));
+      TBPM_CK(cudaMemcpyAsync(slot(0), slot(T), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+      TBPM_CK(cudaMemcpyAsync(slot(1), slot(T + 1), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+      n0 = n;
+    }
+    void* const cur = slot_of(n - 1);
+    void* const prev = n >= 2 ? slot_of(n - 2) : cur;  // not read by the first step
+    if (sweep) {
+      const int cnt = (int)std::min<int64_t>(4, std::min<int64_t>(n_terms - n, T - (n - n0)));
+      void* w[4] = {nullptr, nullptr, nullptr, nullptr};
+      for (int l = 0; l < cnt; ++l) w[l] = slot_of(n + l);
+      TBPM_TRY(launch_sweep_window(ctx, lat, r, prev, cur, w, n == 1));
+      n += cnt;
+      continue;
+    }
+    g.r.cur = cur;
+    g.r.prev_out = prev;
+    g.r.next = slot_of(n);
+    TBPM_TRY(launch_accum_step(ctx, g, pl.precision, n == 1 ? ACC_FIRST : ACC_REGULAR));
+    ++n;
+  }
+  return flush(n0, (int)(n_terms - n0));
+}
+
+// Slots of a window: at most n_terms and 32, and the buffer at most half the free memory.
+int window_slots(const Plan& pl, int64_t n_terms) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
+  return (int)std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), fit), n_terms);
+}
 
 int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int64_t n_steps,
                int64_t b, double* d_C, double tau_signed = 0.0, const BlockHook& hook = nullptr,
@@ -1618,7 +1763,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   TBPM_CK(cudaStreamSynchronize(ctx->stream));  // host vectors go out of scope below
 
   g.acc = ctx->ws_acc.p;
-  g.acc_stride = lat->n_sites * (int64_t)pl.Spad;
+  g.acc_stride = pl.n * (int64_t)pl.Spad;
   g.psi = corr ? ctx->ws_psi.p : nullptr;
   g.C = corr ? d_C : nullptr;
   g.C_len = C_len;
@@ -1626,20 +1771,12 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   // Buffered accumulation: the recurrence writes phi_n into a window of T buffer slots, and
   // every T terms one flush adds sum_t c_t(j) phi_t to every accumulator of the block (each
   // accumulator crosses HBM once per T terms instead of once per term); C(t_j) = <psi|acc_j>
-  // for the whole block comes from one block inner product at its end.  Slots 0 and 1 carry the
-  // two latest vectors of the previous window, slot 2 + k holds term n0 + k.  Where the register
-  // sweep applies, four terms at a time come from one window pass (phi_n and phi_{n-1} read once
-  // for four slots), which pays even for b = 1: the sequential form then buffers too; otherwise
-  // the sequential form keeps its fused one-accumulator pass.
-  const bool sweep_win = sweep_window_applicable(lat, pl.precision, pl.Spad);
+  // for the whole block comes from one block inner product at its end.  Where the register sweep
+  // applies, this pays even for b = 1: the sequential form then buffers too; otherwise the
+  // sequential form keeps its fused one-accumulator pass.
   int T = 0;
-  if (ctx->buffer_blocks && (b >= 2 || sweep_win)) {
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
-    const int Nb_full = *std::max_element(nper_full.begin(), nper_full.end());
-    T = (int)std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), fit), (int64_t)Nb_full);
-  }
+  if (ctx->buffer_blocks && (b >= 2 || sweep_ok(lat, pl)))
+    T = window_slots(pl, *std::max_element(nper_full.begin(), nper_full.end()));
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
     // coefficient tables with the terms past N(j tau~) set to zero, full block then last block
@@ -1660,12 +1797,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
                             ctx->stream));
     TBPM_CK(cudaStreamSynchronize(ctx->stream));
     char* slots = (char*)ctx->ws_blk.p;
-    auto slot = [&](int k) { return (void*)(slots + (size_t)k * pl.state_bytes); };
-    AccumArgs gr = g;
-    gr.b = 0;
-    gr.j_lo = 0;
-    gr.j_done = -1;
-    gr.first_term = 0;
+    char* const terms = slots + 2 * pl.state_bytes;
     int64_t start = 0;
     while (start < n_steps) {
       const int bb = (int)std::min<int64_t>(b, n_steps - start);
@@ -1673,32 +1805,12 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
       const double* cf = (const double*)ctx->ws_blk_coef.p + ((bb == b) ? off_full : off_last);
       const int Nb = *std::max_element(nper.begin(), nper.end());
       TBPM_CK(cudaMemsetAsync(ctx->ws_acc.p, 0, pl.state_bytes * (size_t)bb, ctx->stream));
-      TBPM_CK(cudaMemcpyAsync(slot(2), ctx->ws_phi[0].p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-      int n0 = 0;
-      auto slot_of = [&](int m) { return m >= n0 ? slot(2 + (m - n0)) : (m == n0 - 1 ? slot(1) : slot(0)); };
-      for (int n = 1; n < Nb; ++n) {
-        if (n - n0 == T) {
-          TBPM_TRY(launch_block_flush(ctx, gr.r, pl.precision, slot(2), T, ctx->ws_acc.p, bb,
-                                      cf + (size_t)n0 * bb * 2));
-          TBPM_CK(cudaMemcpyAsync(slot(0), slot(T), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-          TBPM_CK(cudaMemcpyAsync(slot(1), slot(T + 1), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-          n0 = n;
-        }
-        if (sweep_win && n >= 2 && n + 3 < Nb && n - n0 + 4 <= T) {  // terms n .. n+3 in one pass
-          void* const w[4] = {slot_of(n), slot_of(n + 1), slot_of(n + 2), slot_of(n + 3)};
-          TBPM_TRY(launch_sweep_window(ctx, lat, gr.r, slot_of(n - 2), slot_of(n - 1), w));
-          n += 3;
-          continue;
-        }
-        gr.r.cur = slot_of(n - 1);
-        gr.r.prev_out = n >= 2 ? slot_of(n - 2) : slot_of(n - 1);  // not read by the first step
-        gr.r.next = slot_of(n);
-        TBPM_TRY(launch_accum_step(ctx, gr, pl.precision, n == 1 ? ACC_FIRST : ACC_REGULAR));
-      }
-      TBPM_TRY(launch_block_flush(ctx, gr.r, pl.precision, slot(2), Nb - n0, ctx->ws_acc.p, bb,
-                                  cf + (size_t)n0 * bb * 2));
+      TBPM_CK(cudaMemcpyAsync(terms, ctx->ws_phi[0].p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+      TBPM_TRY(walk_windows(ctx, lat, g.r, pl, slots, T, Nb, [&](int64_t n0, int nt) -> int {
+        return launch_block_flush(ctx, g.r, pl.precision, terms, nt, ctx->ws_acc.p, bb, cf + (size_t)n0 * bb * 2);
+      }));
       if (corr)
-        TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, lat->n_sites, ctx->ws_psi.p, 1, ctx->ws_acc.p, bb, d_C,
+        TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, pl.n, ctx->ws_psi.p, 1, ctx->ws_acc.p, bb, d_C,
                              C_len, 0, 1, start + 1));
       if (hook) TBPM_TRY(hook(start, bb, ctx->ws_acc.p));
       const char* last = (const char*)ctx->ws_acc.p + (size_t)(bb - 1) * pl.state_bytes;
@@ -1746,8 +1858,18 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   return TBPM_OK;
 }
 
+// Time blocks, quasi-eigenstates and the conductivity of a vacancy lattice take the full layout where
+// the masked sweep applies and the buffer's window fits.
+int take_full_layout(tbpm_ctx* ctx, tbpm_lattice* lat, Plan* pl) {
+  if (!ctx->buffer_blocks || !masked_sweep_ok(lat, *pl)) return TBPM_OK;
+  set_layout(lat, pl, true);
+  if (window_slots(*pl, qe_flush_max_terms()) < 8) set_layout(lat, pl, false);
+  return pl->full ? ensure_dfull(lat) : TBPM_OK;
+}
+
 // Correlation of all Spad states into d_C [Spad][n_steps+1][2].
-int run_correlation(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, double* d_C) {
+int run_correlation(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl_in, double* d_C) {
+  Plan pl = pl_in;
   const int64_t n_steps = req->n_steps;
   if (n_steps < 1 || n_steps > (1 << 24)) {
     set_error("n_steps out of range");
@@ -1770,6 +1892,7 @@ int run_correlation(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, c
                                       lat->H0 / lat->half, pl.tau, d_C));
     return TBPM_OK;
   }
+  TBPM_TRY(take_full_layout(ctx, lat, &pl));
   if (req->form == TBPM_SEQUENTIAL) return run_blocks(ctx, lat, req, pl, n_steps, 1, d_C);
   if (req->form == TBPM_CONCURRENT_S) {
     int64_t b = req->time_block;
@@ -1802,16 +1925,28 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     double* coef = phase + 2 * (size_t)nE * (n_steps + 1);
     TBPM_TRY(launch_bessel_table(ctx, pl.tau, (int)n_steps, n_table, table, nper));
     TBPM_TRY(launch_qe_coefficients(ctx, table, (int)n_steps, (int)need, d_E, nE, lat->H0, tphys, phase, coef));
+    // buffered accumulation: the recurrence fills a window of T slots, and every T terms one flush
+    // adds sum_t C_t(E) phi_t to all N_E accumulators
+    const int T = window_slots(pl, need);
+    if (T >= 1) {
+      TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes * (size_t)(T + 2)));
+      char* const terms = (char*)ctx->ws_acc.p + 2 * pl.state_bytes;
+      TBPM_TRY(init_states(ctx, lat, req, pl, terms, nullptr));
+      TBPM_CK(cudaMemsetAsync(ctx->ws_qe.p, 0, pl.state_bytes * (size_t)nE, ctx->stream));
+      RecurrenceArgs ra;
+      TBPM_TRY(base_args(ctx, lat, pl, &ra, 3));
+      const int tok = phase_begin(ctx, 0);
+      TBPM_TRY(walk_windows(ctx, lat, ra, pl, (char*)ctx->ws_acc.p, T, need, [&](int64_t n0, int nt) -> int {
+        return launch_qe_flush(ctx, ra, pl.precision, terms, nt, ctx->ws_qe.p, nE, coef, (int)n0);
+      }));
+      phase_end(ctx, tok);
+      return TBPM_OK;
+    }
+    // memory for one slot only: each pass copies phi_n into it and the flush follows at once
     TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
     TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
     TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
-    // buffered accumulation: each pass also copies phi_n into slot n % T of a buffer of T states,
-    // and every T terms one flush adds sum_t C_t(E) phi_t to all N_E accumulators
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), need),
-                                                               (int64_t)(0.5 * (double)free_b / pl.state_bytes)));
-    TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes * (size_t)T));
+    TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes));
     TBPM_TRY(ensure(ctx, ctx->ws_aux, 2 * sizeof(double)));
     const double one[2] = {1.0, 0.0};
     TBPM_CK(cudaMemcpyAsync(ctx->ws_aux.p, one, sizeof(one), cudaMemcpyHostToDevice, ctx->stream));
@@ -1819,23 +1954,20 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     AccumArgs g;
     memset(&g, 0, sizeof(g));
     TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
-    g.acc_stride = lat->n_sites * (int64_t)pl.Spad;
+    g.acc = ctx->ws_acc.p;
+    g.acc_stride = pl.n * (int64_t)pl.Spad;
     g.b = 1;
     g.j_lo = 0;
     g.j_done = -1;
-    g.first_term = 1;  // the buffer slot is written, not accumulated
+    g.first_term = 1;  // the slot is written, not accumulated
     g.coef = (const double*)ctx->ws_aux.p;
     const int tok = phase_begin(ctx, 0);
     for (int64_t n = 0; n < need; ++n) {
       const int mode = (n == need - 1) ? ACC_NOSPMV : (n == 0 ? ACC_FIRST : ACC_REGULAR);
       g.r.cur = ctx->ws_phi[n & 1].p;
       g.r.prev_out = ctx->ws_phi[(n + 1) & 1].p;
-      g.acc = (char*)ctx->ws_acc.p + (size_t)(n % T) * pl.state_bytes;
       TBPM_TRY(launch_accum_step(ctx, g, pl.precision, mode));
-      if ((n + 1) % T == 0 || n == need - 1) {
-        const int nt = (int)(n % T) + 1;
-        TBPM_TRY(launch_qe_flush(ctx, g.r, pl.precision, ctx->ws_acc.p, nt, ctx->ws_qe.p, nE, coef, (int)(n + 1 - nt)));
-      }
+      TBPM_TRY(launch_qe_flush(ctx, g.r, pl.precision, ctx->ws_acc.p, 1, ctx->ws_qe.p, nE, coef, (int)n));
     }
     phase_end(ctx, tok);
     return TBPM_OK;
@@ -1879,8 +2011,9 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
 // Electronic conductivity (Sec. V) along `direction` for all Spad states and nE energies.
 // Leaves C(t_j, E_k) in ws_out as [Spad][nE][n_steps+1][2] and sigma in ws_ec (after the
 // 2*Spad*nE norms) as [Spad][nE].  Returns the sigma pointer through *d_sigma.
-int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, const double* d_E, int nE,
+int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl_in, const double* d_E, int nE,
            int direction, double** d_C_out, double** d_sigma) {
+  Plan pl = pl_in;
   const int64_t n_steps = req->n_steps;
   const int dims = lat->desc.kind == TBPM_CUBIC ? 3 : 2;
   if (direction < 0 || direction >= dims) {
@@ -1899,6 +2032,7 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
   tbpm_request qreq = *req;
   qreq.form = nE <= 200 ? TBPM_CONCURRENT_E : TBPM_CONCURRENT_S;
   qreq.time_block = 0;
+  TBPM_TRY(take_full_layout(ctx, lat, &pl));
   TBPM_TRY(run_qe(ctx, lat, &qreq, pl, d_E, nE));
   const int rows = pl.Spad * nE;
   const int64_t W = n_steps + 1;
@@ -1910,16 +2044,16 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
   TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
   TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_psi.p, nullptr));
-  const int64_t n = lat->n_sites;
+  const int64_t n = pl.n;
   // <psi|Psi(E)> before the kets are overwritten
   TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, ctx->ws_psi.p, 1, ctx->ws_qe.p, nE, nrm, nE, 0, 1, 0));
   // |psi_2(E)> = J |Psi(E)> in place (through one scratch block), |psi_1> = J |psi>
   for (int k = 0; k < nE; ++k) {
     char* qk = (char*)ctx->ws_qe.p + (size_t)k * pl.state_bytes;
-    TBPM_TRY(launch_current(ctx, lat, pl.precision, pl.Spad, direction, qk, ctx->ws_phi[0].p));
+    TBPM_TRY(launch_current(ctx, lat, pl.precision, pl.Spad, direction, qk, ctx->ws_phi[0].p, pl.full));
     TBPM_CK(cudaMemcpyAsync(qk, ctx->ws_phi[0].p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
   }
-  TBPM_TRY(launch_current(ctx, lat, pl.precision, pl.Spad, direction, ctx->ws_psi.p, ctx->ws_jpsi.p));
+  TBPM_TRY(launch_current(ctx, lat, pl.precision, pl.Spad, direction, ctx->ws_psi.p, ctx->ws_jpsi.p, pl.full));
   const void* kets = ctx->ws_qe.p;
   TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * 2 * (size_t)rows * W));
   double* C = (double*)ctx->ws_out.p;
@@ -1936,44 +2070,15 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     g.b = 0;
     g.j_done = -1;
     // buffered: the recurrence fills a window of up to 32 slots and one block inner product
-    // gives the window's moments against all kets (each ket read once per window, not per term);
-    // slots 0 and 1 carry the previous window's last two vectors, slot 2 + a holds term n0 + a
-    int T = 0;
-    if (ctx->buffer_blocks) {
-      size_t free_b = 0, total_b = 0;
-      cudaMemGetInfo(&free_b, &total_b);
-      const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
-      T = (int)std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), fit), Nn);
-    }
+    // gives the window's moments against all kets (each ket read once per window, not per term)
+    const int T = ctx->buffer_blocks ? window_slots(pl, Nn) : 0;
     if (T >= 4) {
       TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
-      char* slots = (char*)ctx->ws_blk.p;
-      auto slot = [&](int64_t k) { return (void*)(slots + (size_t)k * pl.state_bytes); };
-      int64_t n0 = 0;
-      auto slot_of = [&](int64_t t) { return t >= n0 ? slot(2 + (t - n0)) : (t == n0 - 1 ? slot(1) : slot(0)); };
-      TBPM_CK(cudaMemcpyAsync(slot(2), ctx->ws_jpsi.p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-      const bool sweep_win = sweep_window_applicable(lat, pl.precision, pl.Spad);
-      for (int64_t k = 1; k < Nn; ++k) {
-        if (k - n0 == T) {
-          TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, slot(2), T, kets, nE, m, (int64_t)nE * Nn, 1, Nn, n0));
-          TBPM_CK(cudaMemcpyAsync(slot(0), slot(T), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-          TBPM_CK(cudaMemcpyAsync(slot(1), slot(T + 1), pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-          n0 = k;
-        }
-        if (sweep_win && k >= 2 && k + 3 < Nn && k - n0 + 4 <= T) {  // terms k .. k+3 in one pass
-          void* const w[4] = {slot_of(k), slot_of(k + 1), slot_of(k + 2), slot_of(k + 3)};
-          TBPM_TRY(launch_sweep_window(ctx, lat, g.r, slot_of(k - 2), slot_of(k - 1), w));
-          k += 3;
-          continue;
-        }
-        g.r.cur = slot_of(k - 1);
-        g.r.prev_out = k >= 2 ? slot_of(k - 2) : slot_of(k - 1);  // not read by the first step
-        g.r.next = slot_of(k);
-        TBPM_TRY(launch_accum_step(ctx, g, pl.precision, k == 1 ? ACC_FIRST : ACC_REGULAR));
-      }
-      TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, slot(2), (int)(Nn - n0), kets, nE, m, (int64_t)nE * Nn, 1,
-                           Nn, n0));
-      g.r.next = nullptr;
+      char* const terms = (char*)ctx->ws_blk.p + 2 * pl.state_bytes;
+      TBPM_CK(cudaMemcpyAsync(terms, ctx->ws_jpsi.p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+      TBPM_TRY(walk_windows(ctx, lat, g.r, pl, (char*)ctx->ws_blk.p, T, Nn, [&](int64_t n0, int nt) -> int {
+        return launch_xdot(ctx, pl.precision, pl.Spad, n, terms, nt, kets, nE, m, (int64_t)nE * Nn, 1, Nn, n0);
+      }));
     } else {
     TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, ctx->ws_phi[0].p, 1, kets, nE, m, (int64_t)nE * Nn, 0, Nn, 0));
     for (int64_t k = 0; k + 1 < Nn; ++k) {
@@ -2054,43 +2159,16 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
   g.j_lo = 0;
   g.j_done = -1;
   // buffered: terms go into a window of up to 32 slots and one flush adds sum_n a_n T_n phi to
-  // the output per window (the same bookkeeping as the buffered time blocks)
-  int T = 0;
-  if (ctx->buffer_blocks) {
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pc.state_bytes) - 2;
-    T = (int)std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), fit), (int64_t)n_terms);
-  }
+  // the output per window (as the buffered time blocks)
+  const int T = ctx->buffer_blocks ? window_slots(pc, n_terms) : 0;
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pc.state_bytes * (size_t)(T + 2)));
-    char* slots = (char*)ctx->ws_blk.p;
-    auto slot = [&](int k) { return (void*)(slots + (size_t)k * pc.state_bytes); };
-    int n0 = 0;
-    auto slot_of = [&](int t) { return t >= n0 ? slot(2 + (t - n0)) : (t == n0 - 1 ? slot(1) : slot(0)); };
+    char* const terms = (char*)ctx->ws_blk.p + 2 * pc.state_bytes;
     TBPM_CK(cudaMemsetAsync(out, 0, pc.state_bytes, ctx->stream));
-    TBPM_CK(cudaMemcpyAsync(slot(2), b0, pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-    g.b = 0;
-    const bool sweep_win = sweep_window_applicable(lat, pc.precision, pc.Spad);
-    for (int n = 1; n < n_terms; ++n) {
-      if (n - n0 == T) {
-        TBPM_TRY(launch_block_flush(ctx, g.r, pc.precision, slot(2), T, out, 1, coef + 2 * (size_t)n0));
-        TBPM_CK(cudaMemcpyAsync(slot(0), slot(T), pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-        TBPM_CK(cudaMemcpyAsync(slot(1), slot(T + 1), pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-        n0 = n;
-      }
-      if (sweep_win && n >= 2 && n + 3 < n_terms && n - n0 + 4 <= T) {  // terms n .. n+3 in one pass
-        void* const w[4] = {slot_of(n), slot_of(n + 1), slot_of(n + 2), slot_of(n + 3)};
-        TBPM_TRY(launch_sweep_window(ctx, lat, g.r, slot_of(n - 2), slot_of(n - 1), w));
-        n += 3;
-        continue;
-      }
-      g.r.cur = slot_of(n - 1);
-      g.r.prev_out = n >= 2 ? slot_of(n - 2) : slot_of(n - 1);  // not read by the first step
-      g.r.next = slot_of(n);
-      TBPM_TRY(launch_accum_step(ctx, g, pc.precision, n == 1 ? ACC_FIRST : ACC_REGULAR));
-    }
-    TBPM_TRY(launch_block_flush(ctx, g.r, pc.precision, slot(2), n_terms - n0, out, 1, coef + 2 * (size_t)n0));
+    TBPM_CK(cudaMemcpyAsync(terms, b0, pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+    TBPM_TRY(walk_windows(ctx, lat, g.r, pc, (char*)ctx->ws_blk.p, T, n_terms, [&](int64_t n0, int nt) -> int {
+      return launch_block_flush(ctx, g.r, pc.precision, terms, nt, out, 1, coef + 2 * (size_t)n0);
+    }));
     release(ctx, ctx->ws_blk);  // the callers' next step sizes its blocks by the free memory
     return TBPM_OK;
   }
@@ -2148,7 +2226,7 @@ int run_response(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
     TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_psi.p, nullptr));
     if (op == 0) {
       TBPM_TRY(ensure(ctx, ctx->ws_jpsi, pl.state_bytes));
-      TBPM_TRY(launch_current(ctx, lat, pl.precision, Sh, beta, ctx->ws_psi.p, ctx->ws_jpsi.p));
+      TBPM_TRY(launch_current(ctx, lat, pl.precision, Sh, beta, ctx->ws_psi.p, ctx->ws_jpsi.p, false));
     }
     return TBPM_OK;
   };
@@ -2295,6 +2373,11 @@ int tbpm_moment_pass_kind(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_r
     const int band = (m == 8 ? 128 : m == 9 ? 192 : 256) / (pl.Spad / 2);
     *kind = (m >= 8 && m <= 10 && lat->geom.Lx >= band) ? TBPM_PASS_SWEEP
             : (m >= 3) ? TBPM_PASS_ROWS : TBPM_PASS_TILES;
+    return TBPM_OK;
+  }
+  if ((m >= 8 || m == -1) && !fused_applicable(lat, pl.precision, pl.Spad) && M / 2 - 1 >= 4 &&
+      (sweep_ok(lat, pl) || masked_sweep_ok(lat, pl))) {
+    *kind = TBPM_PASS_SWEEP;
     return TBPM_OK;
   }
   *kind = lat->path == TBPM_PATH_CSR ? TBPM_PASS_ELL : TBPM_PASS_STENCIL;
@@ -2477,6 +2560,7 @@ int tbpm_block_autotune(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
   double ta = 0, tx = 0;
+  TBPM_TRY(take_full_layout(ctx, lat, &pl));
   TBPM_TRY(choose_block(ctx, lat, req, pl, n_steps, b_opt, &ta, &tx));
   if (times_ms) {
     times_ms[0] = ta;
@@ -2499,13 +2583,27 @@ int tbpm_quasi_eigenstates(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_
   TBPM_CK(cudaSetDevice(ctx->device));
   TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE));
   TBPM_CK(cudaMemcpyAsync(ctx->ws_energies.p, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
+  TBPM_TRY(take_full_layout(ctx, lat, &pl));
   TBPM_TRY(run_qe(ctx, lat, req, pl, (const double*)ctx->ws_energies.p, (int)nE));
   const int64_t n = lat->n_sites;
-  for (int64_t k = 0; k < nE; ++k)
+  for (int64_t k = 0; k < nE; ++k) {
+    const char* block = (const char*)ctx->ws_qe.p + (size_t)k * pl.state_bytes;
+    if (pl.full) {  // back to the compact order of the active sites
+      TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
+      const int nb = grid_for(ctx, n * pl.P, kT);
+      if (pl.spt == 2)
+        k_compact_states<<<nb, kT, 0, ctx->stream>>>(n, pl.P, lat->full_of, (const float4*)block,
+                                                     (float4*)ctx->ws_phi[0].p);
+      else
+        k_compact_states<<<nb, kT, 0, ctx->stream>>>(n, pl.P, lat->full_of, (const float2*)block,
+                                                     (float2*)ctx->ws_phi[0].p);
+      TBPM_CK_LAUNCH(ctx);
+      block = (const char*)ctx->ws_phi[0].p;
+    }
     for (int s = 0; s < pl.S; ++s)
-      TBPM_CK(cudaMemcpy2DAsync((char*)out + ((size_t)k * pl.S + s) * n * pl.elem, pl.elem,
-                                (const char*)ctx->ws_qe.p + (size_t)k * pl.state_bytes + s * pl.elem,
+      TBPM_CK(cudaMemcpy2DAsync((char*)out + ((size_t)k * pl.S + s) * n * pl.elem, pl.elem, block + s * pl.elem,
                                 pl.Spad * pl.elem, pl.elem, n, cudaMemcpyDeviceToHost, ctx->stream));
+  }
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
   return TBPM_OK;
 }

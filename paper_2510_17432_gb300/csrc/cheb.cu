@@ -434,6 +434,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_accum_stencil(AccumArgs gargs) 
         if (diag) {
           const R dd = __ldg(diag + (own >> logP));
           d = (MODE == ACC_FIRST) ? dd : dd + dd;
+          if (a.masked && isnan(dd)) {  // vacant site: nothing reaches it
+            d = R(0);
+#pragma unroll
+            for (int w = 0; w < 2 * SPT; ++w) h.v[w] = R(0);
+          }
         }
         PK o;
         if constexpr (MODE == ACC_FIRST) {

@@ -40,6 +40,7 @@ struct CurArgs {
   int path;
   const int32_t* ell;
   const int64_t* full_of;
+  const float* masked;  // full layout: NaN at vacant sites, whose amplitude stays zero (else null)
   int64_t n_sites;
   int P, logP;
   double kw[2][6];  // t (r_j - r_i)_alpha per sublattice and neighbour slot
@@ -62,7 +63,8 @@ __global__ void __launch_bounds__(kThreads) k_current(CurArgs c, const void* xv,
     PK o;
 #pragma unroll
     for (int k = 0; k < 2 * SPT; ++k) o.v[k] = R(0);
-    for (int d = 0; d < c.g.z; ++d) {
+    const bool vacant = c.masked && isnan(__ldg(c.masked + i));
+    for (int d = 0; d < c.g.z && !vacant; ++d) {
       const int64_t j = csr ? (int64_t)c.ell[i * c.g.z + d] : neighbour_full(c.g, i, d);
       if (j < 0) continue;
       const R w = c.kwl ? (R)__ldg(c.kwl + sub * c.g.z + d) : (R)c.kw[sub][d];
@@ -297,13 +299,14 @@ void current_weights(int kind, int direction, double t, double kw[2][6]) {
 }
 
 int launch_current(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int S, int direction, const void* x,
-                   void* y) {
+                   void* y, bool full) {
   CurArgs c;
   c.g = lat->geom;
-  c.path = lat->path;
+  c.path = full ? TBPM_PATH_STENCIL : lat->path;
+  c.masked = full ? lat->dfull : nullptr;
   c.ell = lat->ell;
   c.full_of = lat->full_of;
-  c.n_sites = lat->n_sites;
+  c.n_sites = full ? lat->geom.n_full : lat->n_sites;
   const int spt = spt_for(precision, S);
   c.P = S / spt;
   c.logP = 0;
@@ -314,7 +317,7 @@ int launch_current(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int S,
     set_error("current operator: ELL lists missing");
     return TBPM_EINVAL;
   }
-  const int64_t n_units = lat->n_sites * c.P;
+  const int64_t n_units = c.n_sites * c.P;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n_units + kThreads - 1) / kThreads,
                                                                (int64_t)ctx->num_sms * 8));
   if (precision == TBPM_C128)

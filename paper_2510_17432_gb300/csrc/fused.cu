@@ -1008,7 +1008,7 @@ int launch_fused_pass(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceAr
     // the register sweep copies whole band rows; a lattice narrower than a band takes mode 5
     const int band = (variant == 8 ? 128 : variant == 9 ? 192 : 256) / (ra.S / 2);
     if (lat->geom.Lx >= band)
-      return launch_sweep_pass(ctx, lat, ra, prev_in, cur_in, prev_out, cur_out, step0, variant);
+      return launch_sweep_pass(ctx, lat, ra, prev_in, cur_in, prev_out, cur_out, step0, 4, variant);
     variant = 5;
   }
   if (variant == 5) return launch_rowsK<128, 4>(ctx, lat, ra, prev_in, cur_in, prev_out, cur_out, step0);

@@ -272,6 +272,8 @@ struct tbpm_lattice {
   int n_chunks[2] = {0, 0};
   int halo_x = 0, halo_y = 0;
   bool tap_exact = false;        // run pieces of every length 1..8 (else 8, 4, 2, 1)
+  // vacancy lattices on the masked stencil: D_i by full site index, NaN at vacant sites (made on first use)
+  float* dfull = nullptr;
   int64_t* compact = nullptr;  // [n_full] compact index or -1 (CSR path only)
   int64_t* full_of = nullptr;  // [n_sites] full index of each compact site (CSR path only)
 };
@@ -321,6 +323,7 @@ struct RecurrenceArgs {
   int taps_n0, taps_n1, taps_rx, taps_ry, taps_exact;
   double* tap_partials;
   const void* diag;    // per-site D_i (float* or double*), or null when the lattice is clean
+  int masked;          // diag holds NaN at vacant sites (full layout of a vacancy lattice)
   double diag_const;   // D when diag == null
   double thop;         // t / |H|
   // the same coefficients pre-rounded for the FP32 kernels: first term (x1) and regular
@@ -395,13 +398,15 @@ bool fused_applicable(const tbpm_lattice* lat, int precision, int Spad);
 // register-resident sweep (variants 8-10, csrc/sweep.cu); its bounded waits report through the
 // int status word at ctx->pinned + kSweepStatusSlot (zeroed at context creation)
 constexpr int kSweepStatusSlot = 16;
+// smallest lattices the sweep takes: cells and rows on the honeycomb, sites and rows on the square lattice
+constexpr int kSweepMinCells = 48, kSweepMinRows = 32, kSweepMinSquare = 96;
+bool sweep_shape_ok(const tbpm_lattice* lat, int precision, int Spad);
 int launch_sweep_pass(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, const void* prev_in,
-                      const void* cur_in, void* prev_out, void* cur_out, int step0, int variant);
+                      const void* cur_in, void* prev_out, void* cur_out, int step0, int nk, int variant);
 int sweep_status(tbpm_ctx* ctx);  // TBPM_ETIMEOUT (and clears the word) after an expired wait
 // window pass of the time blocks (no moments): phi_{n+1..n+4} into win[0..3]
-bool sweep_window_applicable(const tbpm_lattice* lat, int precision, int Spad);
 int launch_sweep_window(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, const void* prev_in,
-                        const void* cur_in, void* const win[4]);
+                        const void* cur_in, void* const win[4], bool first);
 int fused_steps(int variant);
 int launch_fused_pass(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, const void* prev_in,
                       const void* cur_in, void* prev_out, void* cur_out, int step0, int variant);
@@ -423,8 +428,9 @@ int launch_dos_jackson_tensor_async(tbpm_ctx* ctx, const double* mu, int S, int 
                                     int64_t nE, double H0, double half, double* D, int* h_err);
 // electronic conductivity (csrc/conduct.cu)
 void current_weights(int kind, int direction, double t, double kw[2][6]);
+// full: a vacancy lattice's blocks by full site index (vacant sites stay zero)
 int launch_current(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int S, int direction, const void* x,
-                   void* y);
+                   void* y, bool full);
 int launch_xdot(tbpm_ctx* ctx, int precision, int S, int64_t n_sites, const void* A, int nA, const void* B, int nB,
                 double* out, int64_t os, int64_t oa, int64_t ob, int64_t off);
 int launch_partial_reduce(tbpm_ctx* ctx, const double* partials, int G, int nA, int nB, int S, double* out,

@@ -38,3 +38,101 @@ def test_random_phases_are_rounded_once(capi, ctx, L, S):
     a, b = out.view(np.float32).ravel(), want.view(np.float32).ravel()
     assert np.all(np.abs(a - b) <= np.spacing(np.abs(b)))
     assert np.count_nonzero(a != b) <= a.size // 1000
+
+
+def _pair(capi, ctx, spec):
+    lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(spec["kind"], spec["L"], t=spec["t"], W=spec["W"], seed=77,
+                                                          vacancy_frac=spec.get("vac", 0.0),
+                                                          pbc=spec.get("pbc", (1, 1, 1))))
+    ol = olat.build_lattice(spec["kind"], tuple(spec["L"]) + (1,), t=spec["t"], W=spec["W"], seed=77,
+                            vacancy_frac=spec.get("vac", 0.0), pbc=spec.get("pbc", (1, 1, 1)))
+    return lat, ol
+
+
+# Shapes of the register sweep beyond honeycomb pairs: the square lattice (even and odd rows, so that
+# the last cell holds one or two sites; one band and several; open and periodic), one state per site
+# (128-cell bands), and vacancy lattices in the full layout.  M / 2 = 4 k + 1 .. 4 k + 4 steps: every
+# tail of the last pass.
+SWEEPS = [
+    ("square_one_band", dict(kind=0, L=(128, 96), t=1.0, W=0.0), 4, 42),
+    ("square_odd_W", dict(kind=0, L=(131, 97), t=1.0, W=1.0), 8, 44),
+    ("square_odd_open_x", dict(kind=0, L=(197, 99), t=-1.0, W=0.7, pbc=(0, 1, 1)), 5, 46),
+    ("square_open_y_S32", dict(kind=0, L=(96, 101), t=1.0, W=2.0, pbc=(1, 0, 1)), 32, 40),
+    ("square_open_xy_S2", dict(kind=0, L=(301, 120), t=1.0, W=0.0, pbc=(0, 0, 1)), 2, 42),
+    ("square_S1", dict(kind=0, L=(258, 98), t=1.0, W=1.0), 1, 46),
+    ("square_S1_open", dict(kind=0, L=(512, 100), t=1.0, W=0.0, pbc=(0, 0, 1)), 1, 40),
+    ("honey_S1", dict(kind=1, L=(128, 32), t=-2.7, W=0.0), 1, 44),
+    ("honey_S1_W_open", dict(kind=1, L=(253, 51), t=-2.7, W=1.0, pbc=(0, 0, 1)), 1, 42),
+    ("honey_vac_S1", dict(kind=1, L=(150, 61), t=-2.7, W=1.0, vac=0.03), 1, 46),
+    ("honey_vac_clean_S3", dict(kind=1, L=(64, 40), t=-2.7, W=0.0, vac=0.2, pbc=(1, 0, 1)), 3, 40),
+    ("honey_vac_open_x_S8", dict(kind=1, L=(70, 45), t=1.0, W=0.5, vac=0.4, pbc=(0, 1, 1)), 8, 42),
+    ("square_vac_S2", dict(kind=0, L=(257, 99), t=1.0, W=1.0, vac=0.05), 2, 44),
+    ("square_vac_S1", dict(kind=0, L=(256, 97), t=1.0, W=0.3, vac=0.1), 1, 46),
+]
+
+
+def _moments(capi, ctx, lat, S, M, mode, sites=None):
+    mu = np.zeros((S, M, 2))
+    capi.tbpm_set_fusion(ctx, mode)
+    try:
+        capi.tbpm_moments(ctx, lat, capi.request(n_states=S, n_moments=M, state_seed=3, sites=sites), mu)
+    finally:
+        capi.tbpm_set_fusion(ctx, 8)
+    return mu[..., 0] + 1j * mu[..., 1]
+
+
+@pytest.mark.parametrize("name,spec,S,M", SWEEPS, ids=[c[0] for c in SWEEPS])
+def test_sweep_shapes_match_the_one_step_pass_and_the_oracle(capi, ctx, name, spec, S, M):
+    lat, ol = _pair(capi, ctx, spec)
+    assert capi.tbpm_moment_pass_kind(ctx, lat, capi.request(n_states=S, n_moments=M)) == capi.PASS_SWEEP
+    got, one = _moments(capi, ctx, lat, S, M, 8), _moments(capi, ctx, lat, S, M, 0)
+    assert np.max(np.abs(got - one)) <= 1e-6
+    psi = oprop.random_phase_states(ol, 3, S)
+    for s in {0, S - 1}:
+        assert np.max(np.abs(got[s] - oprop.moments(ol, psi[s], psi[s], M))) <= 1e-5
+    sites = np.array([0, ol.n - 1, ol.n // 2], np.int64)  # site states: no averaging over the lattice
+    got = _moments(capi, ctx, lat, 3, M, 8, sites)
+    for k, i in enumerate(sites):
+        e = np.zeros(ol.n, np.complex128)
+        e[i] = 1.0
+        assert np.max(np.abs(got[k] - oprop.moments(ol, e, e, M))) <= 1e-5
+    capi.tbpm_lattice_destroy(lat)
+
+
+WINDOWS = [
+    ("square", dict(kind=0, L=(129, 97), t=1.0, W=1.0, pbc=(1, 0, 1)), 4),
+    ("square_S1", dict(kind=0, L=(256, 96), t=1.0, W=1.0), 1),
+    ("honey_S1", dict(kind=1, L=(130, 40), t=-2.7, W=1.0), 1),
+    ("honey_vac_S1", dict(kind=1, L=(140, 40), t=-2.7, W=1.0, vac=0.05), 1),
+    ("honey_vac_S2", dict(kind=1, L=(130, 33), t=-2.7, W=0.0, vac=0.1), 2),
+]
+
+
+@pytest.mark.parametrize("name,spec,S", WINDOWS, ids=[c[0] for c in WINDOWS])
+def test_window_passes_of_the_new_shapes(capi, ctx, name, spec, S):
+    """Correlations in every form, quasi-eigenstates and the conductivity through the window passes."""
+    from oracle import conductivity as oec, quasi as oqe
+    lat, ol = _pair(capi, ctx, spec)
+    psi = oprop.random_phase_states(ol, 8, S)
+    s = S - 1
+    Nt = 19
+    ref = oprop.correlation_sequential(ol, psi[s], Nt, np.pi)
+    for form, b in ((0, 0), (2, 5), (2, 0)):
+        C = np.zeros((S, Nt + 1), np.complex128)
+        capi.tbpm_correlation(ctx, lat, capi.request(n_states=S, form=form, n_steps=Nt, time_block=b, state_seed=8), C)
+        assert np.max(np.abs(C[s] - ref)) <= 1e-5, form
+    E = ol.H0 + np.array([-0.6, 0.05, 0.4]) * (ol.E_max - ol.E_min) / 2
+    out = np.zeros((E.size, S, ol.n), np.complex64)
+    qref = oqe.qe_concurrent_e(ol, psi[s], E, Nt)
+    for form in (3, 2):
+        capi.tbpm_quasi_eigenstates(ctx, lat, capi.request(n_states=S, form=form, n_steps=Nt, state_seed=8), E, out)
+        for k in range(E.size):
+            assert np.max(np.abs(out[k, s] - qref[k])) <= 1e-5 * np.max(np.abs(qref[k])), (form, k)
+    for form in (0, 1, 2):
+        C = np.zeros((S, E.size, Nt + 1), np.complex128)
+        sigma = np.zeros((S, E.size))
+        capi.tbpm_conductivity(ctx, lat, capi.request(n_states=S, form=form, n_steps=Nt, state_seed=8), 0, E, C, sigma)
+        Cref, _ = oec.ec_correlation_sequential(ol, psi[s], E, Nt, 0)
+        for k in range(E.size):
+            assert np.max(np.abs(C[s, k] - Cref[k])) <= 3e-5 * np.max(np.abs(Cref[k])), (form, k)
+    capi.tbpm_lattice_destroy(lat)
