@@ -1501,20 +1501,26 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
 }
 
 // Coefficient table of one time block of bb steps: coef[n][j] = exp(-i shift (j+1) tau) c_n((j+1) tau),
-// zero once n >= N((j+1) tau).  n_per[j] = N((j+1) tau).
-void block_coefficients(double tau, double shift, int bb, std::vector<double>* coef, std::vector<int>* n_per) {
+// zero once n >= N((j+1) tau).  n_per[j] = N((j+1) tau).  amp: the same as the flush takes them, real
+// amplitudes a_n((j+1) tau) [n][j] (c_n = a_n (-i)^n), then the factors exp(-i shift (j+1) tau) [j].
+void block_coefficients(double tau, double shift, int bb, std::vector<double>* coef, std::vector<int>* n_per,
+                        std::vector<double>* amp) {
   n_per->resize(bb);
   for (int j = 0; j < bb; ++j) (*n_per)[j] = (int)truncation_order_host((j + 1) * tau);
   const int nt = *std::max_element(n_per->begin(), n_per->end());
   coef->assign((size_t)nt * bb * 2, 0.0);
+  amp->assign((size_t)nt * bb + 2 * (size_t)bb, 0.0);
   std::vector<double> J(nt + 1);
   for (int j = 0; j < bb; ++j) {
     const double x = (j + 1) * tau;
     bessel_j_host(x, nt, J.data());
     double ps, pc;
     sincos(-shift * x, &ps, &pc);
+    (*amp)[(size_t)nt * bb + 2 * j] = pc;
+    (*amp)[(size_t)nt * bb + 2 * j + 1] = ps;
     for (int n = 0; n < (*n_per)[j]; ++n) {
       const double a = n == 0 ? J[0] : 2.0 * J[n];
+      (*amp)[(size_t)n * bb + j] = a;
       double cr = 0, ci = 0;
       switch (n & 3) {
         case 0: cr = a; break;
@@ -1583,12 +1589,13 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
   *t_axpy = std::max(1e-6, (double)(ms1 - ms0) / reps / k_acc);
   // buffered blocks: a step is the recurrence into a buffer slot plus its share of the flush's
   // slot reads; an accumulator update is the flush's extra cost per accumulator and term
-  const int Tm = 8;
+  const int Tm = 24;  // terms per timed flush: long enough that the accumulators' own traffic weighs little
   const bool sweep = sweep_ok(lat, pl);
   if (r == TBPM_OK && ctx->buffer_blocks && k_acc >= 2 &&
       ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)Tm) == TBPM_OK &&
-      ensure(ctx, ctx->ws_blk_coef, sizeof(double) * 2 * (size_t)Tm * k_acc) == TBPM_OK) {
-    if (cudaMemsetAsync(ctx->ws_blk_coef.p, 0, sizeof(double) * 2 * (size_t)Tm * k_acc, ctx->stream) !=
+      ensure(ctx, ctx->ws_blk_coef, sizeof(double) * (size_t)Tm * k_acc) == TBPM_OK) {
+    // tiny amplitudes, not zeros: the flush skips closed accumulators
+    if (cudaMemsetAsync(ctx->ws_blk_coef.p, 0x3c, sizeof(double) * (size_t)Tm * k_acc, ctx->stream) !=
             cudaSuccess ||
         cudaMemsetAsync(ctx->ws_blk.p, 0, pl.state_bytes * (size_t)Tm, ctx->stream) != cudaSuccess) {
       set_error("measure_pass_costs: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1613,12 +1620,12 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
       // both flushes in the 16-accumulator tile of the block sizes being chosen between, so that
       // the difference is the cost of the extra accumulators, not of another kernel
       for (int i = 0; i < reps && r == TBPM_OK; ++i)
-        r = launch_block_flush(ctx, g.r, pl.precision, ctx->ws_blk.p, Tm, ctx->ws_acc.p, 1,
-                               (const double*)ctx->ws_blk_coef.p, 16);
+        r = launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, 1,
+                         (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
       cudaEventRecord(e[2], ctx->stream);
       for (int i = 0; i < reps && r == TBPM_OK; ++i)
-        r = launch_block_flush(ctx, g.r, pl.precision, ctx->ws_blk.p, Tm, ctx->ws_acc.p, k_acc,
-                               (const double*)ctx->ws_blk_coef.p, 16);
+        r = launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, k_acc,
+                         (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
       cudaEvent_t e3;
       cudaEventCreate(&e3);
       cudaEventRecord(e3, ctx->stream);
@@ -1705,12 +1712,13 @@ int walk_windows(tbpm_ctx* ctx, tbpm_lattice* lat, const RecurrenceArgs& r, cons
   return flush(n0, (int)(n_terms - n0));
 }
 
-// Slots of a window: at most n_terms and 32, and the buffer at most half the free memory.
+// Slots of a window: at most n_terms and what a flush takes, and the buffer at most half the free memory.
 int window_slots(const Plan& pl, int64_t n_terms) {
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
   const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
-  return (int)std::min<int64_t>(std::min<int64_t>(qe_flush_max_terms(), fit), n_terms);
+  const int64_t T = std::min<int64_t>(std::min<int64_t>(flush_max_terms(), fit), n_terms);
+  return (int)(T >= 4 && T < n_terms ? T / 4 * 4 : T);  // a further window starts at a multiple of four terms
 }
 
 int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int64_t n_steps,
@@ -1746,11 +1754,11 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   if (corr) TBPM_TRY(launch_dot(ctx, g.r, pl.precision, ctx->ws_psi.p, ctx->ws_psi.p, d_C, C_len));
 
   const double shift = lat->H0 / lat->half;
-  std::vector<double> coef_full, coef_last;
+  std::vector<double> coef_full, coef_last, amp_full, amp_last;
   std::vector<int> nper_full, nper_last;
-  block_coefficients(tau, shift, (int)b, &coef_full, &nper_full);
+  block_coefficients(tau, shift, (int)b, &coef_full, &nper_full, &amp_full);
   const int64_t last_len = n_steps % b;
-  if (last_len) block_coefficients(tau, shift, (int)last_len, &coef_last, &nper_last);
+  if (last_len) block_coefficients(tau, shift, (int)last_len, &coef_last, &nper_last, &amp_last);
   const size_t tab_bytes = (coef_full.size() + coef_last.size()) * sizeof(double);
   TBPM_TRY(ensure(ctx, ctx->ws_table, tab_bytes));
   double* tab_full = (double*)ctx->ws_table.p;
@@ -1779,19 +1787,9 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
     T = window_slots(pl, *std::max_element(nper_full.begin(), nper_full.end()));
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
-    // coefficient tables with the terms past N(j tau~) set to zero, full block then last block
-    std::vector<double> cz;
-    auto zeroed = [&](const std::vector<double>& cf, const std::vector<int>& np, int bb) {
-      const int Nb = *std::max_element(np.begin(), np.end());
-      const size_t base = cz.size();
-      cz.insert(cz.end(), cf.begin(), cf.begin() + (size_t)Nb * bb * 2);
-      for (int n = 0; n < Nb; ++n)
-        for (int j = 0; j < bb; ++j)
-          if (n >= np[j]) cz[base + ((size_t)n * bb + j) * 2] = cz[base + ((size_t)n * bb + j) * 2 + 1] = 0.0;
-      return base;
-    };
-    const size_t off_full = zeroed(coef_full, nper_full, (int)b);
-    const size_t off_last = last_len ? zeroed(coef_last, nper_last, (int)last_len) : 0;
+    // amplitudes and phases, full block then last block
+    std::vector<double> cz = amp_full;
+    cz.insert(cz.end(), amp_last.begin(), amp_last.end());
     TBPM_TRY(ensure(ctx, ctx->ws_blk_coef, cz.size() * sizeof(double)));
     TBPM_CK(cudaMemcpyAsync(ctx->ws_blk_coef.p, cz.data(), cz.size() * sizeof(double), cudaMemcpyHostToDevice,
                             ctx->stream));
@@ -1802,19 +1800,21 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
     while (start < n_steps) {
       const int bb = (int)std::min<int64_t>(b, n_steps - start);
       const std::vector<int>& nper = (bb == b) ? nper_full : nper_last;
-      const double* cf = (const double*)ctx->ws_blk_coef.p + ((bb == b) ? off_full : off_last);
+      const double* amp = (const double*)ctx->ws_blk_coef.p + ((bb == b) ? 0 : amp_full.size());
       const int Nb = *std::max_element(nper.begin(), nper.end());
-      TBPM_CK(cudaMemsetAsync(ctx->ws_acc.p, 0, pl.state_bytes * (size_t)bb, ctx->stream));
-      TBPM_CK(cudaMemcpyAsync(terms, ctx->ws_phi[0].p, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+      const double* phase = shift != 0.0 ? amp + (size_t)Nb * bb : nullptr;
+      // the block starts from the last state of the one before
+      const char* first = start == 0 ? (const char*)ctx->ws_phi[0].p
+                                     : (const char*)ctx->ws_acc.p + (size_t)(b - 1) * pl.state_bytes;
+      TBPM_CK(cudaMemcpyAsync(terms, first, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
       TBPM_TRY(walk_windows(ctx, lat, g.r, pl, slots, T, Nb, [&](int64_t n0, int nt) -> int {
-        return launch_block_flush(ctx, g.r, pl.precision, terms, nt, ctx->ws_acc.p, bb, cf + (size_t)n0 * bb * 2);
+        return launch_flush(ctx, pl.precision, pl.n * pl.Spad, terms, nt, ctx->ws_acc.p, bb, amp + (size_t)n0 * bb, 1,
+                            true, n0 == 0, n0 + nt == Nb ? phase : nullptr);
       }));
       if (corr)
         TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, pl.n, ctx->ws_psi.p, 1, ctx->ws_acc.p, bb, d_C,
                              C_len, 0, 1, start + 1));
       if (hook) TBPM_TRY(hook(start, bb, ctx->ws_acc.p));
-      const char* last = (const char*)ctx->ws_acc.p + (size_t)(bb - 1) * pl.state_bytes;
-      TBPM_CK(cudaMemcpyAsync(ctx->ws_phi[0].p, last, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
       start += bb;
     }
     return TBPM_OK;
@@ -1863,7 +1863,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
 int take_full_layout(tbpm_ctx* ctx, tbpm_lattice* lat, Plan* pl) {
   if (!ctx->buffer_blocks || !masked_sweep_ok(lat, *pl)) return TBPM_OK;
   set_layout(lat, pl, true);
-  if (window_slots(*pl, qe_flush_max_terms()) < 8) set_layout(lat, pl, false);
+  if (window_slots(*pl, flush_max_terms()) < 8) set_layout(lat, pl, false);
   return pl->full ? ensure_dfull(lat) : TBPM_OK;
 }
 
@@ -1928,21 +1928,21 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     // buffered accumulation: the recurrence fills a window of T slots, and every T terms one flush
     // adds sum_t C_t(E) phi_t to all N_E accumulators
     const int T = window_slots(pl, need);
-    if (T >= 1) {
+    if (T >= 4) {
       TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes * (size_t)(T + 2)));
       char* const terms = (char*)ctx->ws_acc.p + 2 * pl.state_bytes;
       TBPM_TRY(init_states(ctx, lat, req, pl, terms, nullptr));
-      TBPM_CK(cudaMemsetAsync(ctx->ws_qe.p, 0, pl.state_bytes * (size_t)nE, ctx->stream));
       RecurrenceArgs ra;
       TBPM_TRY(base_args(ctx, lat, pl, &ra, 3));
       const int tok = phase_begin(ctx, 0);
       TBPM_TRY(walk_windows(ctx, lat, ra, pl, (char*)ctx->ws_acc.p, T, need, [&](int64_t n0, int nt) -> int {
-        return launch_qe_flush(ctx, ra, pl.precision, terms, nt, ctx->ws_qe.p, nE, coef, (int)n0);
+        return launch_flush(ctx, pl.precision, pl.n * pl.Spad, terms, nt, ctx->ws_qe.p, nE, coef + 2 * (size_t)n0 * nE, 2,
+                            false, n0 == 0, nullptr);
       }));
       phase_end(ctx, tok);
       return TBPM_OK;
     }
-    // memory for one slot only: each pass copies phi_n into it and the flush follows at once
+    // memory for a slot only: each pass copies phi_n into it and the flush follows at once
     TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
     TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
     TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
@@ -1950,7 +1950,6 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     TBPM_TRY(ensure(ctx, ctx->ws_aux, 2 * sizeof(double)));
     const double one[2] = {1.0, 0.0};
     TBPM_CK(cudaMemcpyAsync(ctx->ws_aux.p, one, sizeof(one), cudaMemcpyHostToDevice, ctx->stream));
-    TBPM_CK(cudaMemsetAsync(ctx->ws_qe.p, 0, pl.state_bytes * (size_t)nE, ctx->stream));
     AccumArgs g;
     memset(&g, 0, sizeof(g));
     TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
@@ -1967,7 +1966,8 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
       g.r.cur = ctx->ws_phi[n & 1].p;
       g.r.prev_out = ctx->ws_phi[(n + 1) & 1].p;
       TBPM_TRY(launch_accum_step(ctx, g, pl.precision, mode));
-      TBPM_TRY(launch_qe_flush(ctx, g.r, pl.precision, ctx->ws_acc.p, 1, ctx->ws_qe.p, nE, coef, (int)n));
+      TBPM_TRY(launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_acc.p, 1, ctx->ws_qe.p, nE,
+                            coef + 2 * (size_t)n * nE, 2, false, n == 0, nullptr));
     }
     phase_end(ctx, tok);
     return TBPM_OK;
@@ -2164,10 +2164,10 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pc.state_bytes * (size_t)(T + 2)));
     char* const terms = (char*)ctx->ws_blk.p + 2 * pc.state_bytes;
-    TBPM_CK(cudaMemsetAsync(out, 0, pc.state_bytes, ctx->stream));
     TBPM_CK(cudaMemcpyAsync(terms, b0, pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
     TBPM_TRY(walk_windows(ctx, lat, g.r, pc, (char*)ctx->ws_blk.p, T, n_terms, [&](int64_t n0, int nt) -> int {
-      return launch_block_flush(ctx, g.r, pc.precision, terms, nt, out, 1, coef + 2 * (size_t)n0);
+      return launch_flush(ctx, pc.precision, pc.n * pc.Spad, terms, nt, out, 1, coef + 2 * (size_t)n0, 2, false, n0 == 0,
+                          nullptr);
     }));
     release(ctx, ctx->ws_blk);  // the callers' next step sizes its blocks by the free memory
     return TBPM_OK;

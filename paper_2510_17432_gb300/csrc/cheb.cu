@@ -788,289 +788,6 @@ __global__ void __launch_bounds__(kThreads) k_qe_axpy(const void* xv, void* qev,
   }
 }
 
-// Buffered form of the energy-based quasi-eigenstate accumulation (Sec. IV, Eq. form2_concurrent):
-// the recurrence writes T Chebyshev states phi_{n0} .. phi_{n0+T-1} once into a buffer, and one
-// pass then adds sum_t C_{n0+t}(E) phi_{n0+t} to every accumulator, so each accumulator is read and
-// written once per T terms instead of once per term.  grid (energy tiles of kQeEB, unit blocks):
-// the energy tiles of one unit block run side by side and share the buffered states through L2.
-constexpr int kQeEB = 16;
-constexpr int kQeMaxT = 32;
-template <typename R, int SPT>
-__global__ void __launch_bounds__(kThreads) k_qe_flush(const void* phiv, int T, int64_t stride_packs, void* qev,
-                                                       int nE, const double* coef, int n0, int64_t n_units) {
-  using PK = Pack<R, SPT>;
-  __shared__ R cs[kQeMaxT][kQeEB];
-  const int e0 = blockIdx.x * kQeEB;
-  const int ne = min(kQeEB, nE - e0);
-  for (int i = threadIdx.x; i < T * kQeEB; i += kThreads) {
-    const int t = i / kQeEB, e = i - t * kQeEB;
-    cs[t][e] = e < ne ? (R)coef[((int64_t)(n0 + t) * nE + e0 + e) * 2] : R(0);  // C_n(E) is real
-  }
-  __syncthreads();
-  const PK* Phi = reinterpret_cast<const PK*>(phiv);
-  PK* Q = reinterpret_cast<PK*>(qev);
-  for (int64_t u = (int64_t)blockIdx.y * kThreads + threadIdx.x; u < n_units; u += (int64_t)gridDim.y * kThreads) {
-    PK acc[kQeEB];
-#pragma unroll
-    for (int e = 0; e < kQeEB; ++e) {
-      if (e < ne) acc[e] = ld(Q + (int64_t)(e0 + e) * stride_packs + u);
-      else
-#pragma unroll
-        for (int k = 0; k < 2 * SPT; ++k) acc[e].v[k] = R(0);
-    }
-    for (int t = 0; t < T; ++t) {
-      const PK x = ld(Phi + (int64_t)t * stride_packs + u);
-#pragma unroll
-      for (int e = 0; e < kQeEB; ++e) {
-        const R c = cs[t][e];
-#pragma unroll
-        for (int k = 0; k < 2 * SPT; ++k) acc[e].v[k] += c * x.v[k];
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < kQeEB; ++e)
-      if (e < ne) st(Q + (int64_t)(e0 + e) * stride_packs + u, acc[e]);
-  }
-}
-
-// Complex64 form of k_qe_flush: the real weights C_n(E) of two energies sit in one shared quad
-// (C_e, C_e, C_{e+1}, C_{e+1}), so one broadcast load feeds one packed f32x2 FMA per state and
-// energy, (q_re, q_im) += C (x_re, x_im); each thread reads TB buffered terms before their FMAs.
-template <int SPT, int TB>
-__global__ void __launch_bounds__(kThreads, 2) k_qe_flush_c64(const void* phiv, int T, int64_t stride_packs,
-                                                              void* qev, int nE, const double* coef, int n0,
-                                                              int64_t n_units) {
-  using PK = Pack<float, SPT>;
-  constexpr int EB = kQeEB;
-  __shared__ float4 cs[kQeMaxT][EB / 2];
-  const int e0 = blockIdx.x * EB;
-  const int ne = min(EB, nE - e0);
-  for (int i = threadIdx.x; i < T * (EB / 2); i += kThreads) {
-    const int t = i / (EB / 2), e = 2 * (i - t * (EB / 2));
-    const float c0 = e < ne ? (float)coef[((int64_t)(n0 + t) * nE + e0 + e) * 2] : 0.f;  // C_n(E) is real
-    const float c1 = e + 1 < ne ? (float)coef[((int64_t)(n0 + t) * nE + e0 + e + 1) * 2] : 0.f;
-    cs[t][e / 2] = make_float4(c0, c0, c1, c1);
-  }
-  __syncthreads();
-  const PK* Phi = reinterpret_cast<const PK*>(phiv);
-  PK* Q = reinterpret_cast<PK*>(qev);
-  for (int64_t u = (int64_t)blockIdx.y * kThreads + threadIdx.x; u < n_units; u += (int64_t)gridDim.y * kThreads) {
-    float2 ac[EB][SPT];
-#pragma unroll
-    for (int e = 0; e < EB; ++e) {
-      PK q;
-      if (e < ne) q = ld(Q + (int64_t)(e0 + e) * stride_packs + u);
-      else
-#pragma unroll
-        for (int c = 0; c < 2 * SPT; ++c) q.v[c] = 0.f;
-#pragma unroll
-      for (int s = 0; s < SPT; ++s) ac[e][s] = make_float2(q.v[2 * s], q.v[2 * s + 1]);
-    }
-    for (int t0 = 0; t0 < T; t0 += TB) {
-      PK x[TB];
-#pragma unroll
-      for (int j = 0; j < TB; ++j) {
-        if (t0 + j < T) x[j] = ld(Phi + (int64_t)(t0 + j) * stride_packs + u);
-        else
-#pragma unroll
-          for (int c = 0; c < 2 * SPT; ++c) x[j].v[c] = 0.f;
-      }
-#pragma unroll
-      for (int j = 0; j < TB; ++j) {
-        if (t0 + j >= T) break;  // uniform
-#pragma unroll
-        for (int e = 0; e < EB; e += 2) {
-          if (e < ne) {  // uniform
-            const float4 c = cs[t0 + j][e / 2];
-            const float2 c0 = make_float2(c.x, c.y), c1 = make_float2(c.z, c.w);
-#pragma unroll
-            for (int s = 0; s < SPT; ++s) {
-              const float2 xv = make_float2(x[j].v[2 * s], x[j].v[2 * s + 1]);
-              ac[e][s] = __ffma2_rn(c0, xv, ac[e][s]);
-              ac[e + 1][s] = __ffma2_rn(c1, xv, ac[e + 1][s]);
-            }
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < EB; ++e) {
-      if (e < ne) {
-        PK q;
-#pragma unroll
-        for (int s = 0; s < SPT; ++s) {
-          q.v[2 * s] = ac[e][s].x;
-          q.v[2 * s + 1] = ac[e][s].y;
-        }
-        st(Q + (int64_t)(e0 + e) * stride_packs + u, q);
-      }
-    }
-  }
-}
-
-// Buffered time-block accumulation: acc_j += sum_{t < T} c_t(j) phi_t for the open
-// accumulators of a time block, with T buffered Chebyshev vectors phi_t (consecutive state
-// blocks) and complex coefficients c_t(j) = coef[(t * nb + j) * 2 + {0, 1}] (zero once term t is
-// past N(j tau~)).  Each accumulator is read and written once per T terms instead of once per
-// term.  grid: (accumulator tiles of EB, unit blocks); EB = 1, 4 or 16 accumulators per tile
-// (the registers of a tile's accumulators limit how many threads, and so how many buffer loads,
-// an SM keeps in flight: a one-accumulator flush, the sequential form's, runs at full occupancy).
-// Buffer loads in flight per thread: 8 for the small tiles, 4 for 16 accumulators (whose registers
-// already bound the occupancy).
-template <int EB>
-struct FlushUnroll {
-  static constexpr int value = EB >= 16 ? 4 : 8;
-};
-
-template <typename R, int SPT, int EB>
-__global__ void __launch_bounds__(kThreads) k_block_flush(const void* phiv, int T, int64_t stride_packs, void* accv,
-                                                          int nb, const double* coef, int64_t n_units) {
-  using PK = Pack<R, SPT>;
-  __shared__ R cr[kQeMaxT][EB], ci[kQeMaxT][EB];
-  const int e0 = blockIdx.x * EB;
-  const int ne = min(EB, nb - e0);
-  for (int i = threadIdx.x; i < T * EB; i += kThreads) {
-    const int t = i / EB, e = i - t * EB;
-    const bool ok = e < ne;
-    cr[t][e] = ok ? (R)coef[((int64_t)t * nb + e0 + e) * 2] : R(0);
-    ci[t][e] = ok ? (R)coef[((int64_t)t * nb + e0 + e) * 2 + 1] : R(0);
-  }
-  __syncthreads();
-  const PK* Phi = reinterpret_cast<const PK*>(phiv);
-  PK* Q = reinterpret_cast<PK*>(accv);
-  for (int64_t u = (int64_t)blockIdx.y * kThreads + threadIdx.x; u < n_units; u += (int64_t)gridDim.y * kThreads) {
-    PK acc[EB];
-#pragma unroll
-    for (int e = 0; e < EB; ++e) {
-      if (e < ne) acc[e] = ld(Q + (int64_t)(e0 + e) * stride_packs + u);
-      else
-#pragma unroll
-        for (int k = 0; k < 2 * SPT; ++k) acc[e].v[k] = R(0);
-    }
-#pragma unroll (FlushUnroll<EB>::value)
-    for (int t = 0; t < T; ++t) {  // unrolled so that several buffer loads are in flight
-      const PK x = ld(Phi + (int64_t)t * stride_packs + u);
-#pragma unroll
-      for (int e = 0; e < EB; ++e) {
-        if (e < ne) {  // uniform: a tile of fewer accumulators does no work for the rest
-          const R a = cr[t][e], b = ci[t][e];
-#pragma unroll
-          for (int q = 0; q < SPT; ++q) {
-            const R xr = x.v[2 * q], xi = x.v[2 * q + 1];
-            acc[e].v[2 * q] += a * xr - b * xi;
-            acc[e].v[2 * q + 1] += a * xi + b * xr;
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < EB; ++e)
-      if (e < ne) st(Q + (int64_t)(e0 + e) * stride_packs + u, acc[e]);
-  }
-}
-
-// Complex64 flush of a tile of EB >= 4 accumulators with packed f32x2 FMAs.  The coefficient
-// table holds (Re c, Re c, Im c, Im c) per term and accumulator, so one broadcast shared load
-// feeds every state of the thread's U units, each with two packed FMAs:
-//   (acc_re, acc_im) += Re c (x_re, x_im) + Im c (-x_im, x_re).
-// Per term and accumulator that is 2 SPT U FMA instructions and 1 / (SPT U) shared loads per
-// state, where the scalar flush above issues 4 FMAs and 2 shared loads per state (measured on a
-// 32-term, 16-accumulator flush: 31 % fewer instructions than the same kernel with scalar FMAs).
-template <int SPT, int EB, int U, int TB>
-__global__ void __launch_bounds__(kThreads, 2) k_block_flush_c64(const void* phiv, int T, int64_t stride_packs,
-                                                              void* accv, int nb, const double* coef,
-                                                              int64_t n_units) {
-  using PK = Pack<float, SPT>;
-  __shared__ float4 cf[kQeMaxT][EB];
-  const int e0 = blockIdx.x * EB;
-  const int ne = min(EB, nb - e0);
-  for (int i = threadIdx.x; i < T * EB; i += kThreads) {
-    const int t = i / EB, e = i - t * EB;
-    const bool ok = e < ne;
-    const float cr = ok ? (float)coef[((int64_t)t * nb + e0 + e) * 2] : 0.f;
-    const float ci = ok ? (float)coef[((int64_t)t * nb + e0 + e) * 2 + 1] : 0.f;
-    cf[t][e] = make_float4(cr, cr, ci, ci);
-  }
-  __syncthreads();
-  const PK* Phi = reinterpret_cast<const PK*>(phiv);
-  PK* Q = reinterpret_cast<PK*>(accv);
-  const int64_t step = (int64_t)gridDim.y * kThreads * U;
-  for (int64_t ub = (int64_t)blockIdx.y * kThreads * U + threadIdx.x; ub < n_units; ub += step) {
-    bool valid[U];
-    float2 ac[U][EB][SPT];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      valid[k] = ub + k * kThreads < n_units;
-#pragma unroll
-      for (int e = 0; e < EB; ++e) {
-        PK q;
-        if (valid[k] && e < ne) q = ld(Q + (int64_t)(e0 + e) * stride_packs + ub + k * kThreads);
-        else
-#pragma unroll
-          for (int c = 0; c < 2 * SPT; ++c) q.v[c] = 0.f;
-#pragma unroll
-        for (int s = 0; s < SPT; ++s) ac[k][e][s] = make_float2(q.v[2 * s], q.v[2 * s + 1]);
-      }
-    }
-    // the buffered vectors are read TB terms at a time, all loads issued before the FMAs, so
-    // that TB loads per thread are in flight (the flush streams T + 2 ne state blocks)
-    for (int t0 = 0; t0 < T; t0 += TB) {
-      PK x[TB][U];
-#pragma unroll
-      for (int j = 0; j < TB; ++j)
-#pragma unroll
-        for (int k = 0; k < U; ++k) {
-          if (valid[k] && t0 + j < T) x[j][k] = ld(Phi + (int64_t)(t0 + j) * stride_packs + ub + k * kThreads);
-          else
-#pragma unroll
-            for (int c = 0; c < 2 * SPT; ++c) x[j][k].v[c] = 0.f;
-        }
-#pragma unroll
-      for (int j = 0; j < TB; ++j) {
-        if (t0 + j >= T) break;  // uniform
-        float2 xs[U][SPT], xw[U][SPT];
-#pragma unroll
-        for (int k = 0; k < U; ++k)
-#pragma unroll
-          for (int s = 0; s < SPT; ++s) {
-            xs[k][s] = make_float2(x[j][k].v[2 * s], x[j][k].v[2 * s + 1]);
-            xw[k][s] = make_float2(-x[j][k].v[2 * s + 1], x[j][k].v[2 * s]);
-          }
-#pragma unroll
-        for (int e = 0; e < EB; ++e) {
-          if (e < ne) {  // uniform: a tile of fewer accumulators does no work for the rest
-            const float4 c = cf[t0 + j][e];
-            const float2 cre = make_float2(c.x, c.y), cim = make_float2(c.z, c.w);
-#pragma unroll
-            for (int k = 0; k < U; ++k)
-#pragma unroll
-              for (int s = 0; s < SPT; ++s) {
-                ac[k][e][s] = __ffma2_rn(cre, xs[k][s], ac[k][e][s]);
-                ac[k][e][s] = __ffma2_rn(cim, xw[k][s], ac[k][e][s]);
-              }
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      if (!valid[k]) continue;
-#pragma unroll
-      for (int e = 0; e < EB; ++e) {
-        if (e < ne) {
-          PK q;
-#pragma unroll
-          for (int s = 0; s < SPT; ++s) {
-            q.v[2 * s] = ac[k][e][s].x;
-            q.v[2 * s + 1] = ac[k][e][s].y;
-          }
-          st(Q + (int64_t)(e0 + e) * stride_packs + ub + k * kThreads, q);
-        }
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------ dispatch
 template <typename R, int SPT>
 static void* moment_kernel(int kind, bool csr, bool first) {
@@ -1232,73 +949,6 @@ int launch_qe_axpy(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const 
   int64_t nu = n_units;
   void* args[] = {(void*)&x, &qe, &stride, &nu, (void*)&phase, &width, &j, &sgn, &scale, &nE};
   return launch(ctx, fn, grid, args);
-}
-
-int qe_flush_max_terms() { return kQeMaxT; }
-
-int launch_qe_flush(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* phi, int T, void* qe, int nE,
-                    const double* coef, int n0) {
-  if (T < 1 || T > kQeMaxT) {
-    set_error("quasi-eigenstate flush of %d terms", T);
-    return TBPM_EINVAL;
-  }
-  const int spt = spt_of(precision, a.S);
-  const int64_t n_units = a.n_sites * a.P;
-  const int etiles = (nE + kQeEB - 1) / kQeEB;
-  const int64_t want = std::max<int64_t>(1, (int64_t)ctx->num_sms * 8 / etiles);
-  const int ublocks = (int)std::min<int64_t>(std::min<int64_t>(want, (n_units + kThreads - 1) / kThreads), 65535);
-  void* fn;
-  if (precision == TBPM_C128) fn = (void*)k_qe_flush<double, 1>;
-  else if (spt == 2) fn = (void*)k_qe_flush_c64<2, 2>;
-  else fn = (void*)k_qe_flush_c64<1, 8>;
-  int64_t stride = n_units;
-  int64_t nu = n_units;
-  void* args[] = {(void*)&phi, &T, &stride, &qe, &nE, (void*)&coef, &n0, &nu};
-  cudaError_t e = cudaLaunchKernel(fn, dim3(etiles, ublocks), dim3(kThreads), args, 0, ctx->stream);
-  ctx->launches++;
-  if (e != cudaSuccess) {
-    set_error("kernel launch: %s", cudaGetErrorString(e));
-    return TBPM_ECUDA;
-  }
-  return TBPM_OK;
-}
-
-int launch_block_flush(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* phi, int T, void* acc,
-                       int nb, const double* coef, int tile) {
-  if (T < 1 || T > kQeMaxT || nb < 1) {
-    set_error("block flush of %d terms into %d accumulators", T, nb);
-    return TBPM_EINVAL;
-  }
-  const int spt = spt_of(precision, a.S);
-  const int64_t n_units = a.n_sites * a.P;
-  const int eb = tile > 0 ? tile : (nb == 1 ? 1 : nb <= 4 ? 4 : 16);
-  const int etiles = (nb + eb - 1) / eb;
-  const int64_t want = std::max<int64_t>(1, (int64_t)ctx->num_sms * (eb == 16 ? 8 : 16) / etiles);
-  const int ublocks = (int)std::min<int64_t>(std::min<int64_t>(want, (n_units + kThreads - 1) / kThreads), 65535);
-  void* fn;
-  auto pick = [&](auto eb_tag) -> void* {
-    constexpr int E = decltype(eb_tag)::value;
-    if (precision == TBPM_C128) return (void*)k_block_flush<double, 1, E>;
-    if constexpr (E >= 4) {  // complex64: packed FMAs
-      if (spt == 2) return (void*)k_block_flush_c64<2, E, 1, 2>;
-      return (void*)k_block_flush_c64<1, E, 1, 8>;
-    }
-    if (spt == 2) return (void*)k_block_flush<float, 2, E>;
-    return (void*)k_block_flush<float, 1, E>;
-  };
-  if (eb == 1) fn = pick(std::integral_constant<int, 1>());
-  else if (eb == 4) fn = pick(std::integral_constant<int, 4>());
-  else fn = pick(std::integral_constant<int, 16>());
-  int64_t stride = n_units;
-  int64_t nu = n_units;
-  void* args[] = {(void*)&phi, &T, &stride, &acc, &nb, (void*)&coef, &nu};
-  cudaError_t e = cudaLaunchKernel(fn, dim3(etiles, ublocks), dim3(kThreads), args, 0, ctx->stream);
-  ctx->launches++;
-  if (e != cudaSuccess) {
-    set_error("kernel launch: %s", cudaGetErrorString(e));
-    return TBPM_ECUDA;
-  }
-  return TBPM_OK;
 }
 
 int launch_dot(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* x, const void* y,

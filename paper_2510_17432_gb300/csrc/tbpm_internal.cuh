@@ -375,19 +375,19 @@ int launch_taps_moment(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);
 int launch_taps_step(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);  // recurrence only
 size_t taps_partials_bytes(const RecurrenceArgs& a);
 int launch_accum_step(tbpm_ctx* ctx, const AccumArgs& a, int precision, int mode);
-// acc_j += sum_{t<T} c_t(j) phi_t over T consecutive buffered state blocks phi and nb
-// consecutive accumulators; coef [T][nb] complex (csrc/cheb.cu)
+// acc_e (+)= sum_{t<T} a_t(e) [(-i)^t] phi_t over T consecutive buffered state blocks of n_numbers complex
+// numbers and nb consecutive accumulators (csrc/flush.cu): real amplitudes a_t(e) at
+// amp[(t * nb + e) * amp_stride]; rot: with the powers of -i (the window starts at a multiple of four terms);
+// init: the sums start here; phase: [nb] complex factors on the finished sums, or null.
 // tile: accumulators per CTA tile (1, 4 or 16); 0 = chosen from nb
-int launch_block_flush(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* phi, int T, void* acc,
-                       int nb, const double* coef, int tile = 0);
+int flush_max_terms();
+int launch_flush(tbpm_ctx* ctx, int precision, int64_t n_numbers, const void* phi, int T, void* acc, int nb,
+                 const double* amp, int amp_stride, bool rot, bool init, const double* phase, int tile = 0);
 int launch_dot(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* x, const void* y,
                double* out /* device [S][2] at stride out_stride */, int out_stride);
 int recurrence_blocks(tbpm_ctx* ctx, int precision, int S);
 int launch_qe_axpy(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* x, void* qe,
                    const double* phase, int width, int j, double sgn, double scale, int nE);
-int qe_flush_max_terms();
-int launch_qe_flush(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* phi, int T, void* qe, int nE,
-                    const double* coef, int n0);
 int launch_qe_coefficients(tbpm_ctx* ctx, const double* table, int n_steps, int n_terms, const double* energies,
                            int nE, double H0, double tphys, double* phase, double* coef);
 int launch_qe_coefficients_phase_only(tbpm_ctx* ctx, const double* energies, int nE, double tphys, int n_steps,
