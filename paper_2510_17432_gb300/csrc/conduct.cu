@@ -44,10 +44,18 @@ struct CurArgs {
   int64_t n_sites;
   int P, logP;
   double kw[2][6];  // t (r_j - r_i)_alpha per sublattice and neighbour slot
+  float kwf[2][6];  // the same in FP32 (a conversion per bond would go through the FP64 pipe)
   const double* kwl;  // long-range lattices: the same per slot on the device, [2][z] (else null)
 };
 
-// y = J_alpha x for one block of states [n_sites][S].
+template <typename R, typename Args>
+__device__ __forceinline__ R bond_weight(const Args& a, int sub, int d) {
+  if constexpr (sizeof(R) == 4) return a.kwf[sub][d];
+  else return a.kw[sub][d];
+}
+
+// y = J_alpha x for one block of states [n_sites][S].  Bound: HBM; 64-bit divisions per neighbour had made it
+// issue-bound (36.6 us on 2.1M sites, now CURRENT_NOW).
 template <typename R, int SPT>
 __global__ void __launch_bounds__(kThreads) k_current(CurArgs c, const void* xv, void* yv) {
   using PK = Pack<R, SPT>;
@@ -59,15 +67,24 @@ __global__ void __launch_bounds__(kThreads) k_current(CurArgs c, const void* xv,
     const int64_t i = u >> c.logP;
     const int p = (int)(u & (c.P - 1));
     int sub = 0;
-    if (c.g.kind == TBPM_HONEYCOMB) sub = (int)((csr ? c.full_of[i] : i) & 1);
+    SiteAt at{};
+    if (!csr) {
+      at = site_at(c.g, i);
+      sub = at.s;
+    } else if (c.g.kind == TBPM_HONEYCOMB) {
+      sub = (int)(c.full_of[i] & 1);
+    }
     PK o;
 #pragma unroll
     for (int k = 0; k < 2 * SPT; ++k) o.v[k] = R(0);
     const bool vacant = c.masked && isnan(__ldg(c.masked + i));
+#pragma unroll 3
     for (int d = 0; d < c.g.z && !vacant; ++d) {
-      const int64_t j = csr ? (int64_t)c.ell[i * c.g.z + d] : neighbour_full(c.g, i, d);
+      const R w0 = c.kwl ? R(0) : bond_weight<R>(c, sub, d);
+      if (!c.kwl && w0 == R(0)) continue;  // bonds across the direction
+      const int64_t j = csr ? (int64_t)c.ell[i * c.g.z + d] : site_neighbour(c.g, at, d);
       if (j < 0) continue;
-      const R w = c.kwl ? (R)__ldg(c.kwl + sub * c.g.z + d) : (R)c.kw[sub][d];
+      const R w = c.kwl ? (R)__ldg(c.kwl + sub * c.g.z + d) : w0;
       const PK x = ld(X + j * c.P + p);
 #pragma unroll
       for (int k = 0; k < SPT; ++k) {  // -i w (xr + i xi) = w xi - i w xr
@@ -93,16 +110,126 @@ struct XdotArgs {
   double* partials;  // [gridDim.y][nA][nB][S][2]
 };
 
-template <typename R>
-struct XAcc { using T = float; };
-template <>
-struct XAcc<double> { using T = double; };
+// complex64 block inner products.  A warp owns a tile of TA x TB pairs of blocks (32 sums: two per pair and
+// state of the unit), its lanes walk 16 units each; the CTA's eight warps take neighbouring tiles of the
+// same units, so that L1 serves the blocks the tiles share, and split the units when there are fewer tiles.
+// A product conj(a) b is two packed f32x2 FMAs, (ar, ai) (br, bi) and (ar, ai) (bi, -br), whose halves are
+// added at the fold.  Every 16 units the 32 sums are reduce-scattered over the lanes of a state pair
+// (31 shuffles instead of 160 for a tree per sum) and each lane adds the ones it keeps in FP64.
+// Bound: L1 and FP32 issue for many pairs, HBM for one block against a few.  On 2.1M sites 16 x 64 blocks
+// took 3320 us with a shuffle tree per sum and scalar FMAs, XDOT_NOW.
+struct XTile {
+  int at, bt;   // tiles along A and B
+  int wa, wb;   // tiles of one CTA along A and B (wa wb divides 8)
+};
 
-// grid (a_tiles * b_tiles, chunk groups); 256 threads.
+template <int SPT, int TA, int TB, int LOGP>
+__global__ void __launch_bounds__(kThreads, 2) k_xdot_c64(XdotArgs x, XTile tl) {
+  using PK = Pack<float, SPT>;
+  constexpr int V = TA * TB * SPT * 2, P = 1 << LOGP;
+  static_assert(V == 32, "one sum per lane");
+  const PK* A = reinterpret_cast<const PK*>(x.A);
+  const PK* B = reinterpret_cast<const PK*>(x.B);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nt = tl.wa * tl.wb, share = kWarps / nt;  // warps per tile
+  const int sub = warp / nt, t = warp - sub * nt;
+  const int ga = (tl.at + tl.wa - 1) / tl.wa;
+  const int a0 = ((blockIdx.x % ga) * tl.wa + t % tl.wa) * TA, b0 = ((blockIdx.x / ga) * tl.wb + t / tl.wa) * TB;
+  const int64_t group = (int64_t)blockIdx.y * share + sub, groups = (int64_t)gridDim.y * share;
+  const bool active = a0 < x.nA && b0 < x.nB;
+  const PK* pa[TA];
+  const PK* pb[TB];
+#pragma unroll
+  for (int k = 0; k < TA; ++k) pa[k] = A + (int64_t)min(a0 + k, x.nA - 1) * x.a_stride;
+#pragma unroll
+  for (int l = 0; l < TB; ++l) pb[l] = B + (int64_t)min(b0 + l, x.nB - 1) * x.b_stride;
+  __shared__ double slots[kWarps][P][32];  // this lane's P sums
+  double(&tot)[P][32] = slots[warp];
+#pragma unroll
+  for (int k = 0; k < P; ++k) tot[k][lane] = 0.0;
+  int base = 0;  // index of this lane's first sum after the reduce-scatter
+  {
+    int n = V;
+    for (int off = 16; off >= P; off >>= 1) {
+      n >>= 1;
+      if (lane & off) base += n;
+    }
+  }
+  constexpr int kSpan = 32 * kXIter;  // units per warp and chunk
+  for (int64_t chunk = group; active && chunk * kSpan < x.n_units; chunk += groups) {
+    float2 re[TA][TB][SPT], im[TA][TB][SPT];
+#pragma unroll
+    for (int k = 0; k < TA; ++k)
+#pragma unroll
+      for (int l = 0; l < TB; ++l)
+#pragma unroll
+        for (int s = 0; s < SPT; ++s) re[k][l][s] = im[k][l][s] = make_float2(0.f, 0.f);
+    const int64_t u0 = chunk * kSpan + lane;
+#pragma unroll (TA == 1 ? 1 : 2)
+    for (int it = 0; it < kXIter; ++it) {
+      const int64_t u = u0 + it * 32;
+      if (u >= x.n_units) break;
+      PK a[TA], b[TB];
+#pragma unroll
+      for (int k = 0; k < TA; ++k) a[k] = ld(pa[k] + u);
+#pragma unroll
+      for (int l = 0; l < TB; ++l) b[l] = ld(pb[l] + u);
+#pragma unroll
+      for (int l = 0; l < TB; ++l)
+#pragma unroll
+        for (int s = 0; s < SPT; ++s) {
+          const float2 bv = make_float2(b[l].v[2 * s], b[l].v[2 * s + 1]);
+          const float2 bw = make_float2(bv.y, -bv.x);
+#pragma unroll
+          for (int k = 0; k < TA; ++k) {
+            const float2 av = make_float2(a[k].v[2 * s], a[k].v[2 * s + 1]);
+            re[k][l][s] = __ffma2_rn(av, bv, re[k][l][s]);
+            im[k][l][s] = __ffma2_rn(av, bw, im[k][l][s]);  // ar bi - ai br
+          }
+        }
+    }
+    float v[V];
+#pragma unroll
+    for (int k = 0; k < TA; ++k)
+#pragma unroll
+      for (int l = 0; l < TB; ++l)
+#pragma unroll
+        for (int s = 0; s < SPT; ++s) {
+          v[((k * TB + l) * SPT + s) * 2] = re[k][l][s].x + re[k][l][s].y;
+          v[((k * TB + l) * SPT + s) * 2 + 1] = im[k][l][s].x + im[k][l][s].y;
+        }
+#pragma unroll
+    for (int lev = 0; lev < 5 - LOGP; ++lev) {
+      const int off = 16 >> lev;
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int k = 0; k < (V >> (lev + 1)); ++k) {
+        const float lo = v[k], hi = v[k + (V >> (lev + 1))];
+        v[k] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, off);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < P; ++k) tot[k][lane] += (double)v[k];
+  }
+  // the warps that share a tile, in order
+  __syncthreads();
+  if (!active || sub != 0) return;
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    double sum = 0.0;
+    for (int w = t; w < kWarps; w += nt) sum += slots[w][q][lane];
+    const int v = base + q, c = v & 1, s = (v >> 1) % SPT, kl = (v >> 1) / SPT;
+    const int ia = a0 + kl / TB, ib = b0 + kl % TB;
+    if (ia < x.nA && ib < x.nB)
+      x.partials[((((int64_t)blockIdx.y * x.nA + ia) * x.nB + ib) * x.S + (lane & (P - 1)) * SPT + s) * 2 + c] = sum;
+  }
+}
+
+// complex128 (FP64 issue bound): grid (a_tiles * b_tiles, chunk groups); 256 threads.
 template <typename R, int SPT, int TA, int TB>
 __global__ void __launch_bounds__(kThreads, 2) k_xdot(XdotArgs x) {
   using PK = Pack<R, SPT>;
-  using T = typename XAcc<R>::T;
+  using T = R;
   constexpr int V = TA * TB * SPT * 2;
   __shared__ double tot[32 * TA * TB * 2];
   const PK* A = reinterpret_cast<const PK*>(x.A);
@@ -169,20 +296,28 @@ __global__ void __launch_bounds__(kThreads, 2) k_xdot(XdotArgs x) {
   }
 }
 
-// out[(s*os + a*oa + b*ob + off)*2 + c] = sum over chunk groups, in order.
-__global__ void k_xdot_reduce(const double* partials, int G, int nA, int nB, int S, double* out, int64_t os,
-                              int64_t oa, int64_t ob, int64_t off) {
+// out[(s*os + a*oa + b*ob + off)*2 + c] = sum over chunk groups in a fixed order: a CTA takes 32 outputs
+// (lanes) and splits the groups over its 32 warps.
+__global__ void __launch_bounds__(1024) k_xdot_reduce(const double* partials, int G, int nA, int nB, int S, double* out,
+                                                      int64_t os, int64_t oa, int64_t ob, int64_t off) {
+  __shared__ double sh[32][33];
   const int64_t per = (int64_t)nA * nB * S * 2;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < per; q += (int64_t)gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int g = 0; g < G; ++g) acc += partials[(int64_t)g * per + q];
-    const int c = (int)(q & 1);
-    const int64_t r = q >> 1;
-    const int s = (int)(r % S);
-    const int64_t ab = r / S;
-    const int b = (int)(ab % nB), a = (int)(ab / nB);
-    out[(s * os + a * oa + b * ob + off) * 2 + c] = acc;
-  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t q = (int64_t)blockIdx.x * 32 + lane;
+  double acc = 0.0;
+  if (q < per)
+    for (int g = warp; g < G; g += 32) acc += partials[(int64_t)g * per + q];
+  sh[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || q >= per) return;
+  acc = 0.0;
+  for (int w = 0; w < 32; ++w) acc += sh[w][lane];
+  const int c = (int)(q & 1);
+  const int64_t r = q >> 1;
+  const int s = (int)(r % S);
+  const int64_t ab = r / S;
+  const int b = (int)(ab % nB), a = (int)(ab / nB);
+  out[(s * os + a * oa + b * ob + off) * 2 + c] = acc;
 }
 
 __device__ __forceinline__ double block_sum256(double v, double* sh) {
@@ -275,6 +410,24 @@ int xdot_launch(tbpm_ctx* ctx, const XdotArgs& xa0, int G) {
   return TBPM_OK;
 }
 
+template <int SPT, int TA, int TB>
+int xdot_c64_launch(tbpm_ctx* ctx, const XdotArgs& xa, const XTile& tl, dim3 grid) {
+  cudaStream_t st = ctx->stream;
+  if constexpr (SPT == 1) {
+    k_xdot_c64<1, TA, TB, 0><<<grid, kThreads, 0, st>>>(xa, tl);
+  } else {
+    switch (xa.P) {
+      case 1: k_xdot_c64<2, TA, TB, 0><<<grid, kThreads, 0, st>>>(xa, tl); break;
+      case 2: k_xdot_c64<2, TA, TB, 1><<<grid, kThreads, 0, st>>>(xa, tl); break;
+      case 4: k_xdot_c64<2, TA, TB, 2><<<grid, kThreads, 0, st>>>(xa, tl); break;
+      case 8: k_xdot_c64<2, TA, TB, 3><<<grid, kThreads, 0, st>>>(xa, tl); break;
+      default: k_xdot_c64<2, TA, TB, 4><<<grid, kThreads, 0, st>>>(xa, tl); break;
+    }
+  }
+  TBPM_CK_LAUNCH(ctx);
+  return TBPM_OK;
+}
+
 }  // namespace
 
 // Bond-vector components (r_j - r_i)_alpha per sublattice and neighbour slot, times t.
@@ -312,6 +465,7 @@ int launch_current(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int S,
   c.logP = 0;
   while ((1 << c.logP) < c.P) ++c.logP;
   current_weights(lat->desc.kind, direction, lat->desc.t, c.kw);
+  for (int k = 0; k < 12; ++k) (&c.kwf[0][0])[k] = (float)(&c.kw[0][0])[k];
   c.kwl = lat->jw ? lat->jw + (size_t)direction * 2 * lat->geom.z : nullptr;
   if (c.path == TBPM_PATH_CSR && !c.ell) {
     set_error("current operator: ELL lists missing");
@@ -347,27 +501,40 @@ int launch_xdot(tbpm_ctx* ctx, int precision, int S, int64_t n_sites, const void
   xa.b_stride = xa.n_units;
   xa.n_chunks = (xa.n_units + kXChunk - 1) / kXChunk;
   const bool single = nA == 1;
-  const int TA = single ? 1 : (spt == 2 ? 2 : 4), TB = single ? 8 : 4;
-  const int64_t pairs = (int64_t)((nA + TA - 1) / TA) * ((nB + TB - 1) / TB);
-  if (pairs > 2147483647LL) {
+  const bool c128 = precision == TBPM_C128;
+  const int TA = single ? 1 : (spt == 2 ? 2 : 4), TB = c128 ? (single ? 8 : 4) : (single ? (spt == 2 ? 8 : 16) : 4);
+  const int at = (nA + TA - 1) / TA, bt = (nB + TB - 1) / TB;
+  const int64_t per = (int64_t)nA * nB * S * 2;
+  const int64_t cap = std::max<int64_t>(1, (64LL << 20) / (int64_t)(per * sizeof(double)));  // partials of 64 MiB
+  if ((int64_t)at * bt > 2147483647LL) {
     set_error("too many state-block pairs");
     return TBPM_EUNSUPPORTED;
   }
-  // enough CTAs for ~4 waves of 2 per SM, partials bounded to 64 MiB
-  const int64_t per = (int64_t)nA * nB * S * 2;
-  int64_t G = std::max<int64_t>(1, ((int64_t)ctx->num_sms * 8 + pairs - 1) / pairs);
-  G = std::min<int64_t>(G, xa.n_chunks);
-  G = std::min<int64_t>(G, std::max<int64_t>(1, (64LL << 20) / (int64_t)(per * sizeof(double))));
-  G = std::min<int64_t>(G, 65535);
+  if (c128) {
+    // enough CTAs for ~4 waves of 2 per SM
+    int64_t G = std::max<int64_t>(1, ((int64_t)ctx->num_sms * 8 + (int64_t)at * bt - 1) / ((int64_t)at * bt));
+    G = std::min<int64_t>(std::min<int64_t>(G, xa.n_chunks), std::min<int64_t>(cap, 65535));
+    TBPM_TRY(ensure(ctx, ctx->ws_xdot, sizeof(double) * (size_t)(per * G)));
+    xa.partials = (double*)ctx->ws_xdot.p;
+    TBPM_TRY((single ? xdot_launch<double, 1, 1, 8>(ctx, xa, (int)G) : xdot_launch<double, 1, 4, 4>(ctx, xa, (int)G)));
+    return launch_partial_reduce(ctx, xa.partials, (int)G, nA, nB, S, out, os, oa, ob, off);
+  }
+  // tiles per CTA: up to four along A (they share the B blocks), then along B, a power of two up to 8
+  XTile tl{at, bt, 1, 1};
+  while (tl.wa < 4 && tl.wa < at) tl.wa *= 2;
+  while (tl.wa * tl.wb < kWarps && tl.wb < bt) tl.wb *= 2;
+  const int share = kWarps / (tl.wa * tl.wb);
+  const int64_t ctas = (int64_t)((at + tl.wa - 1) / tl.wa) * ((bt + tl.wb - 1) / tl.wb);
+  const int64_t spans = (xa.n_units + 32 * kXIter - 1) / (32 * kXIter);  // chunks a warp can take
+  int64_t G = std::max<int64_t>(1, ((int64_t)ctx->num_sms * 4 + ctas - 1) / ctas);
+  G = std::min<int64_t>(G, (spans + share - 1) / share);
+  G = std::max<int64_t>(1, std::min<int64_t>(G, std::min<int64_t>(cap, 65535)));
   TBPM_TRY(ensure(ctx, ctx->ws_xdot, sizeof(double) * (size_t)(per * G)));
   xa.partials = (double*)ctx->ws_xdot.p;
+  const dim3 grid((unsigned)ctas, (unsigned)G);
   int r;
-  if (precision == TBPM_C128)
-    r = single ? xdot_launch<double, 1, 1, 8>(ctx, xa, (int)G) : xdot_launch<double, 1, 4, 4>(ctx, xa, (int)G);
-  else if (spt == 2)
-    r = single ? xdot_launch<float, 2, 1, 8>(ctx, xa, (int)G) : xdot_launch<float, 2, 2, 4>(ctx, xa, (int)G);
-  else
-    r = single ? xdot_launch<float, 1, 1, 8>(ctx, xa, (int)G) : xdot_launch<float, 1, 4, 4>(ctx, xa, (int)G);
+  if (spt == 2) r = single ? xdot_c64_launch<2, 1, 8>(ctx, xa, tl, grid) : xdot_c64_launch<2, 2, 4>(ctx, xa, tl, grid);
+  else r = single ? xdot_c64_launch<1, 1, 16>(ctx, xa, tl, grid) : xdot_c64_launch<1, 4, 4>(ctx, xa, tl, grid);
   TBPM_TRY(r);
   return launch_partial_reduce(ctx, xa.partials, (int)G, nA, nB, S, out, os, oa, ob, off);
 }
@@ -375,8 +542,7 @@ int launch_xdot(tbpm_ctx* ctx, int precision, int S, int64_t n_sites, const void
 int launch_partial_reduce(tbpm_ctx* ctx, const double* partials, int G, int nA, int nB, int S, double* out,
                           int64_t os, int64_t oa, int64_t ob, int64_t off) {
   const int64_t per = (int64_t)nA * nB * S * 2;
-  const int rgrid = (int)std::max<int64_t>(1, std::min<int64_t>((per + 255) / 256, (int64_t)ctx->num_sms * 16));
-  k_xdot_reduce<<<rgrid, 256, 0, ctx->stream>>>(partials, G, nA, nB, S, out, os, oa, ob, off);
+  k_xdot_reduce<<<(unsigned)((per + 31) / 32), 1024, 0, ctx->stream>>>(partials, G, nA, nB, S, out, os, oa, ob, off);
   TBPM_CK_LAUNCH(ctx);
   return TBPM_OK;
 }

@@ -172,6 +172,7 @@ struct XmyArgs {
   SiteGeom sg;
   const int32_t* ell;
   double kw[2][6];       // current operator weights t (r_j - r_i)_alpha
+  float kwf[2][6];       // the same in FP32 (a conversion per bond would go through the FP64 pipe)
   const double* kwl;     // long-range lattices: the same per slot on the device, [2][z] (else null)
   const double2* phase;  // density operator e^{i q.r_i}, or null for the current operator
   const void* Y;         // bb pair blocks [n][2 Sh], consecutive
@@ -184,26 +185,6 @@ struct XmyArgs {
 
 constexpr int kYIter = 8;
 constexpr int kYChunk = kYIter * kThreads;
-
-__device__ __forceinline__ int64_t nb_of(const XmyArgs& a, int64_t i, int d, const int64_t* coords) {
-  if (a.sg.csr) return a.ell[i * a.sg.g.z + d];
-  const Geom& g = a.sg.g;
-  bool ok = true;
-  if (g.kind == TBPM_HONEYCOMB) {
-    const int64_t s = coords[2];
-    const int sg = s == 0 ? -1 : 1;
-    const int64_t xx = wrap_coord(coords[0] + ((d == 1) ? sg : 0), g.Lx, g.pbc_x, &ok);
-    const int64_t yy = wrap_coord(coords[1] + ((d == 2) ? sg : 0), g.Ly, g.pbc_y, &ok);
-    return ok ? 2 * (yy * g.Lx + xx) + (1 - s) : -1;
-  }
-  const int dx = (d == 0) ? 1 : (d == 1) ? -1 : 0;
-  const int dy = (d == 2) ? 1 : (d == 3) ? -1 : 0;
-  const int dz = (d == 4) ? 1 : (d == 5) ? -1 : 0;
-  const int64_t xx = wrap_coord(coords[0] + dx, g.Lx, g.pbc_x, &ok);
-  const int64_t yy = wrap_coord(coords[1] + dy, g.Ly, g.pbc_y, &ok);
-  const int64_t zz = wrap_coord(coords[2] + dz, g.Lz, g.pbc_z, &ok);
-  return ok ? (zz * g.Ly + yy) * g.Lx + xx : -1;
-}
 
 // One thread per (site, state s < Sh); grid (chunk groups, bb).  CURRENT: X = J_alpha, else rho(q).
 template <typename R, bool CURRENT>
@@ -219,8 +200,8 @@ __global__ void __launch_bounds__(kThreads) k_xmy(XmyArgs a) {
   const int s = threadIdx.x & (Sh - 1);
   const int site_lane = threadIdx.x / Sh;
   const int sites_per_pass = kThreads / Sh;
+  Partial<R> pr, pi;
   for (int64_t chunk = blockIdx.x; chunk < a.n_chunks; chunk += gridDim.x) {
-    Partial<R> pr, pi;
     const int64_t i0 = chunk * (int64_t)kYChunk / Sh;
     for (int it = 0; it < kYIter; ++it) {
       const int64_t i = i0 + (int64_t)it * sites_per_pass + site_lane;
@@ -228,24 +209,25 @@ __global__ void __launch_bounds__(kThreads) k_xmy(XmyArgs a) {
       const T b = Y[i * S2 + s];
       R vr = 0, vi = 0;  // (X psi_2)_i
       if constexpr (CURRENT) {
-        const int64_t f = full_index(a.sg, i);
-        int64_t coords[3];
+        SiteAt at{};
         int sub = 0;
-        if (a.sg.g.kind == TBPM_HONEYCOMB) {
-          sub = (int)(f & 1);
-          const int64_t c = f >> 1;
-          coords[0] = c % a.sg.g.Lx;
-          coords[1] = c / a.sg.g.Lx;
-          coords[2] = sub;
-        } else {
-          coords[0] = f % a.sg.g.Lx;
-          coords[1] = (f / a.sg.g.Lx) % a.sg.g.Ly;
-          coords[2] = f / (a.sg.g.Lx * a.sg.g.Ly);
+        if (!a.sg.csr) {
+          at = site_at(a.sg.g, i);
+          sub = at.s;
+        } else if (a.sg.g.kind == TBPM_HONEYCOMB) {
+          sub = (int)(a.sg.full_of[i] & 1);
         }
+#pragma unroll 3
         for (int d = 0; d < a.sg.g.z; ++d) {
-          const int64_t j = nb_of(a, i, d, coords);
+          R w0 = R(0);
+          if (!a.kwl) {
+            if constexpr (sizeof(R) == 4) w0 = a.kwf[sub][d];
+            else w0 = a.kw[sub][d];
+          }
+          if (!a.kwl && w0 == R(0)) continue;  // bonds across the direction
+          const int64_t j = a.sg.csr ? (int64_t)a.ell[i * a.sg.g.z + d] : site_neighbour(a.sg.g, at, d);
           if (j < 0) continue;
-          const R w = a.kwl ? (R)__ldg(a.kwl + sub * a.sg.g.z + d) : (R)a.kw[sub][d];
+          const R w = a.kwl ? (R)__ldg(a.kwl + sub * a.sg.g.z + d) : w0;
           const T x = Y[j * S2 + Sh + s];
           vr += w * x.y;  // -i w x
           vi -= w * x.x;
@@ -260,20 +242,20 @@ __global__ void __launch_bounds__(kThreads) k_xmy(XmyArgs a) {
       pr.add(b.x * vr + b.y * vi);  // conj(psi_1) (X psi_2)
       pi.add(b.x * vi - b.y * vr);
     }
-    pr.fold();
+    pr.fold();  // FP32 sums of at most kYIter terms
     pi.fold();
-    double vr = pr.value(), vi = pi.value();
-    for (int off = 16; off >= Sh; off >>= 1) {
-      vr += __shfl_xor_sync(0xffffffffu, vr, off);
-      vi += __shfl_xor_sync(0xffffffffu, vi, off);
+  }
+  double vr = pr.value(), vi = pi.value();
+  for (int off = 16; off >= Sh; off >>= 1) {
+    vr += __shfl_xor_sync(0xffffffffu, vr, off);
+    vi += __shfl_xor_sync(0xffffffffu, vi, off);
+  }
+  for (int w = 0; w < kThreads / 32; ++w) {
+    if (warp == w && lane < Sh) {
+      tot[2 * lane] += vr;
+      tot[2 * lane + 1] += vi;
     }
-    for (int w = 0; w < kThreads / 32; ++w) {
-      if (warp == w && lane < Sh) {
-        tot[2 * lane] += vr;
-        tot[2 * lane + 1] += vi;
-      }
-      __syncthreads();
-    }
+    __syncthreads();
   }
   for (int q = threadIdx.x; q < 2 * Sh; q += kThreads)
     a.partials[(((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * Sh) * 2 + q] = tot[q];
@@ -434,6 +416,7 @@ int launch_xmy(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int Sh, in
   a.kwl = nullptr;
   if (!phase) {
     current_weights(lat->desc.kind, alpha, lat->desc.t, a.kw);
+    for (int k = 0; k < 12; ++k) (&a.kwf[0][0])[k] = (float)(&a.kw[0][0])[k];
     a.kwl = lat->jw ? lat->jw + (size_t)alpha * 2 * lat->geom.z : nullptr;
     if (a.sg.csr && !a.ell) {
       set_error("current operator: ELL lists missing");

@@ -254,5 +254,49 @@ __device__ __forceinline__ int stencil_neighbours(const Geom& g, const LineBases
   }
 }
 
+// ------------------------------------------------------------------ single sites
+// Coordinates of a full site index and its neighbours, with one or two 32-bit divisions per site (a
+// lattice has fewer than 2^32 sites) instead of 64-bit ones per neighbour.
+struct SiteAt {
+  uint32_t f, x, y, z;
+  int s;
+};
+
+__device__ __forceinline__ SiteAt site_at(const Geom& g, int64_t full) {
+  SiteAt a;
+  a.f = (uint32_t)full;
+  a.s = g.kind == TBPM_HONEYCOMB ? (int)(a.f & 1) : 0;
+  const uint32_t c = g.kind == TBPM_HONEYCOMB ? a.f >> 1 : a.f, lx = (uint32_t)g.Lx;
+  a.y = c / lx;
+  a.x = c - a.y * lx;
+  a.z = 0;
+  if (g.kind == TBPM_CUBIC) {
+    const uint32_t ly = (uint32_t)g.Ly;
+    a.z = a.y / ly;
+    a.y -= a.z * ly;
+  }
+  return a;
+}
+
+// Neighbour d (the fixed order of neighbour_full) of the site, or -1.
+__device__ __forceinline__ int64_t site_neighbour(const Geom& g, const SiteAt& a, int d) {
+  const int64_t f = a.f;
+  // one step of +-1 along a direction of n coordinates with the given stride
+  auto step = [&](uint32_t v, int64_t n, int64_t stride, int periodic, bool up) -> int64_t {
+    if (up) return (int64_t)v + 1 < n ? stride : (periodic ? stride - n * stride : INT64_MIN);
+    return v > 0 ? -stride : (periodic ? n * stride - stride : INT64_MIN);
+  };
+  int64_t off;
+  if (g.kind == TBPM_HONEYCOMB) {
+    const int64_t other = a.s ? -1 : 1;  // partner in the same cell
+    if (d == 0) return f + other;
+    off = d == 1 ? step(a.x, g.Lx, 2, g.pbc_x, a.s != 0) : step(a.y, g.Ly, 2 * g.Lx, g.pbc_y, a.s != 0);
+    return off == INT64_MIN ? -1 : f + other + off;
+  }
+  const bool up = (d & 1) == 0;
+  off = d < 2 ? step(a.x, g.Lx, 1, g.pbc_x, up)
+        : d < 4 ? step(a.y, g.Ly, g.Lx, g.pbc_y, up) : step(a.z, g.Lz, g.Lx * g.Ly, g.pbc_z, up);
+  return off == INT64_MIN ? -1 : f + off;
+}
 
 }  // namespace tbpm
