@@ -1542,109 +1542,102 @@ int64_t block_cap(const Plan& pl, int64_t n_steps) {
   return std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(by_mem, 256), n_steps));
 }
 
+// Slots of a window: at most n_terms and what a flush takes, and the buffer at most half the free memory.
+int window_slots(const Plan& pl, int64_t n_terms) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
+  const int64_t T = std::min<int64_t>(std::min<int64_t>(flush_max_terms(), fit), n_terms);
+  return (int)(T >= 4 && T < n_terms ? T / 4 * 4 : T);  // a further window starts at a multiple of four terms
+}
+
 // Measured per-pass costs of the state-based form (Sec. II.B: "obtained via benchmarking prior
-// to the main calculation"): t_amxsy = one recurrence pass with no accumulator open,
-// t_axpy = the extra time per open accumulator.  Times in milliseconds.
+// to the main calculation"), in milliseconds.  Buffered blocks: t_amxsy = the recurrence into a buffer
+// slot plus its share of the flush's slot reads, t_axpy = the flush's extra cost per accumulator and
+// term.  Unbuffered ones: t_amxsy = one recurrence pass with no accumulator open, t_axpy = the extra time
+// per open accumulator.  Each pass runs once to warm up and once timed where a state block is large
+// enough for one launch to be timed well (16 MiB: tens of microseconds), three times otherwise; the
+// contents of the scratch blocks do not matter.  (Both sets of passes, three times each on zeroed blocks,
+// had made the choice of b 12 % of a 256-step correlation on 8.3M sites.)
 int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int k_acc,
                        double* t_amxsy, double* t_axpy) {
   TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_psi, pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes * (size_t)k_acc));
-  TBPM_TRY(ensure(ctx, ctx->ws_table, sizeof(double) * 2 * (size_t)k_acc));
-  TBPM_CK(cudaMemsetAsync(ctx->ws_table.p, 0, sizeof(double) * 2 * (size_t)k_acc, ctx->stream));
-  TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
-  TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[1].p, nullptr));
-  TBPM_CK(cudaMemsetAsync(ctx->ws_acc.p, 0, pl.state_bytes * (size_t)k_acc, ctx->stream));
   AccumArgs g;
   memset(&g, 0, sizeof(g));
   TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
   g.acc = ctx->ws_acc.p;
   g.acc_stride = pl.n * (int64_t)pl.Spad;
-  g.coef = (const double*)ctx->ws_table.p;
   g.psi = ctx->ws_psi.p;
   g.j_done = -1;
   g.r.cur = ctx->ws_phi[0].p;
   g.r.prev_out = ctx->ws_phi[1].p;
-  cudaEvent_t e[3];
-  for (auto& x : e) TBPM_CK(cudaEventCreate(&x));
-  const int reps = 3;
-  float ms0 = 0.f, ms1 = 0.f;
-  int r = TBPM_OK;
-  for (int pass = 0; pass < 2 && r == TBPM_OK; ++pass) {   // pass 0 warms up
-    g.b = 0;
-    g.j_lo = 0;
-    cudaEventRecord(e[0], ctx->stream);
-    for (int i = 0; i < reps && r == TBPM_OK; ++i) r = launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
-    cudaEventRecord(e[1], ctx->stream);
-    g.b = k_acc;
-    for (int i = 0; i < reps && r == TBPM_OK; ++i) r = launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
-    cudaEventRecord(e[2], ctx->stream);
-  }
-  if (r == TBPM_OK && cudaEventSynchronize(e[2]) == cudaSuccess) {
-    cudaEventElapsedTime(&ms0, e[0], e[1]);
-    cudaEventElapsedTime(&ms1, e[1], e[2]);
-  }
-  *t_amxsy = ms0 / reps;
-  *t_axpy = std::max(1e-6, (double)(ms1 - ms0) / reps / k_acc);
-  // buffered blocks: a step is the recurrence into a buffer slot plus its share of the flush's
-  // slot reads; an accumulator update is the flush's extra cost per accumulator and term
-  const int Tm = 24;  // terms per timed flush: long enough that the accumulators' own traffic weighs little
   const bool sweep = sweep_ok(lat, pl);
-  if (r == TBPM_OK && ctx->buffer_blocks && k_acc >= 2 &&
-      ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)Tm) == TBPM_OK &&
-      ensure(ctx, ctx->ws_blk_coef, sizeof(double) * (size_t)Tm * k_acc) == TBPM_OK) {
+  // terms per timed flush: enough that the accumulators' own traffic weighs little
+  const int Tm = ctx->buffer_blocks && k_acc >= 2 ? window_slots(pl, 24) : 0;
+  const bool buffered = Tm >= 4 && ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)Tm) == TBPM_OK &&
+                        ensure(ctx, ctx->ws_blk_coef, sizeof(double) * (size_t)Tm * k_acc) == TBPM_OK;
+  std::vector<std::function<int()>> pass;
+  if (buffered) {
     // tiny amplitudes, not zeros: the flush skips closed accumulators
-    if (cudaMemsetAsync(ctx->ws_blk_coef.p, 0x3c, sizeof(double) * (size_t)Tm * k_acc, ctx->stream) !=
-            cudaSuccess ||
-        cudaMemsetAsync(ctx->ws_blk.p, 0, pl.state_bytes * (size_t)Tm, ctx->stream) != cudaSuccess) {
-      set_error("measure_pass_costs: %s", cudaGetErrorString(cudaGetLastError()));
-      r = TBPM_ECUDA;
-    }
-    float m[3] = {0.f, 0.f, 0.f};
-    for (int pass = 0; pass < 2 && r == TBPM_OK; ++pass) {
-      g.b = 0;
-      g.j_lo = 0;
-      g.r.next = ctx->ws_blk.p;
-      cudaEventRecord(e[0], ctx->stream);
-      for (int i = 0; i < reps && r == TBPM_OK; ++i) {
-        if (sweep) {  // four terms per window pass
-          char* w0 = (char*)ctx->ws_blk.p;
-          void* const w[4] = {w0, w0 + pl.state_bytes, w0 + 2 * pl.state_bytes, w0 + 3 * pl.state_bytes};
-          r = launch_sweep_window(ctx, lat, g.r, ctx->ws_phi[1].p, ctx->ws_phi[0].p, w, false);
-        } else {
-          r = launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
-        }
-      }
-      cudaEventRecord(e[1], ctx->stream);
-      // both flushes in the 16-accumulator tile of the block sizes being chosen between, so that
-      // the difference is the cost of the extra accumulators, not of another kernel
-      for (int i = 0; i < reps && r == TBPM_OK; ++i)
-        r = launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, 1,
-                         (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
-      cudaEventRecord(e[2], ctx->stream);
-      for (int i = 0; i < reps && r == TBPM_OK; ++i)
-        r = launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, k_acc,
-                         (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
-      cudaEvent_t e3;
-      cudaEventCreate(&e3);
-      cudaEventRecord(e3, ctx->stream);
-      if (r == TBPM_OK && cudaEventSynchronize(e3) == cudaSuccess) {
-        cudaEventElapsedTime(&m[0], e[0], e[1]);
-        cudaEventElapsedTime(&m[1], e[1], e[2]);
-        cudaEventElapsedTime(&m[2], e[2], e3);
-      }
-      cudaEventDestroy(e3);
-    }
-    g.r.next = nullptr;
-    if (r == TBPM_OK) {
-      const double rec = m[0] / reps / (sweep ? 4 : 1), f1 = m[1] / reps, fk = m[2] / reps;
-      *t_amxsy = rec + f1 / Tm;
-      *t_axpy = std::max(1e-6, (fk - f1) / ((double)(k_acc - 1) * Tm));
+    TBPM_CK(cudaMemsetAsync(ctx->ws_blk_coef.p, 0x3c, sizeof(double) * (size_t)Tm * k_acc, ctx->stream));
+    char* const w0 = (char*)ctx->ws_blk.p;
+    g.r.next = w0;
+    pass.push_back([&, w0]() -> int {
+      if (!sweep) return launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
+      void* const w[4] = {w0, w0 + pl.state_bytes, w0 + 2 * pl.state_bytes, w0 + 3 * pl.state_bytes};
+      return launch_sweep_window(ctx, lat, g.r, ctx->ws_phi[1].p, ctx->ws_phi[0].p, w, false);
+    });
+    // both flushes in the 16-accumulator tile of the block sizes being chosen between, so that
+    // the difference is the cost of the extra accumulators, not of another kernel
+    for (const int k : {1, k_acc})
+      pass.push_back([&, k]() -> int {
+        return launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, k,
+                            (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
+      });
+  } else {
+    TBPM_TRY(ensure(ctx, ctx->ws_table, sizeof(double) * 2 * (size_t)k_acc));
+    TBPM_CK(cudaMemsetAsync(ctx->ws_table.p, 0, sizeof(double) * 2 * (size_t)k_acc, ctx->stream));
+    TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
+    TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[1].p, nullptr));
+    TBPM_CK(cudaMemsetAsync(ctx->ws_acc.p, 0, pl.state_bytes * (size_t)k_acc, ctx->stream));
+    g.coef = (const double*)ctx->ws_table.p;
+    for (const int k : {0, k_acc})
+      pass.push_back([&, k]() -> int {
+        g.b = k;
+        return launch_accum_step(ctx, g, pl.precision, ACC_REGULAR);
+      });
+  }
+  const int reps = pl.state_bytes >= (16u << 20) ? 1 : 3;
+  const int np = (int)pass.size();
+  cudaEvent_t e[4];
+  for (int k = 0; k <= np; ++k) TBPM_CK(cudaEventCreate(&e[k]));
+  int r = TBPM_OK;
+  for (int timed = 0; timed < 2 && r == TBPM_OK; ++timed) {
+    cudaEventRecord(e[0], ctx->stream);
+    for (int k = 0; k < np; ++k) {
+      for (int i = 0; i < reps && r == TBPM_OK; ++i) r = pass[k]();
+      cudaEventRecord(e[k + 1], ctx->stream);
     }
   }
-  for (auto& x : e) cudaEventDestroy(x);
+  double ms[3] = {0.0, 0.0, 0.0};
+  if (r == TBPM_OK && cudaEventSynchronize(e[np]) == cudaSuccess)
+    for (int k = 0; k < np; ++k) {
+      float t = 0.f;
+      cudaEventElapsedTime(&t, e[k], e[k + 1]);
+      ms[k] = (double)t / reps;
+    }
+  for (int k = 0; k <= np; ++k) cudaEventDestroy(e[k]);
   TBPM_TRY(r);
+  if (buffered) {
+    *t_amxsy = ms[0] / (sweep ? 4 : 1) + ms[1] / Tm;
+    *t_axpy = std::max(1e-6, (ms[2] - ms[1]) / ((double)(k_acc - 1) * Tm));
+  } else {
+    *t_amxsy = ms[0];
+    *t_axpy = std::max(1e-6, (ms[1] - ms[0]) / k_acc);
+  }
   return TBPM_OK;
 }
 
@@ -1710,15 +1703,6 @@ int walk_windows(tbpm_ctx* ctx, tbpm_lattice* lat, const RecurrenceArgs& r, cons
     ++n;
   }
   return flush(n0, (int)(n_terms - n0));
-}
-
-// Slots of a window: at most n_terms and what a flush takes, and the buffer at most half the free memory.
-int window_slots(const Plan& pl, int64_t n_terms) {
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
-  const int64_t T = std::min<int64_t>(std::min<int64_t>(flush_max_terms(), fit), n_terms);
-  return (int)(T >= 4 && T < n_terms ? T / 4 * 4 : T);  // a further window starts at a multiple of four terms
 }
 
 int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int64_t n_steps,
@@ -2146,6 +2130,15 @@ int fermi_series(tbpm_ctx* ctx, const tbpm_lattice* lat, double mu, double kT, i
   return TBPM_OK;
 }
 
+// Workspaces of the response drivers are given back between their phases only where memory is short
+// (a block above an eighth of the free memory): freeing and allocating them again on every call cost
+// 7 of 85 ms of the optical conductivity of 2.1M sites.
+void release_if_tight(tbpm_ctx* ctx, DevBuf& b) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  if (b.cap > free_b / 8) release(ctx, b);
+}
+
 // out = sum_{n < n_terms} coef_n T_n(H~) X for one state block of plan pc.  The recurrence runs
 // in b0 (which holds X on entry and is overwritten) and b1; out is distinct from both.
 int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0, void* b1, void* out,
@@ -2169,7 +2162,7 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
       return launch_flush(ctx, pc.precision, pc.n * pc.Spad, terms, nt, out, 1, coef + 2 * (size_t)n0, 2, false, n0 == 0,
                           nullptr);
     }));
-    release(ctx, ctx->ws_blk);  // the callers' next step sizes its blocks by the free memory
+    release_if_tight(ctx, ctx->ws_blk);  // the callers' next step sizes its blocks by the free memory
     return TBPM_OK;
   }
   void* buf[2] = {b0, b1};
@@ -2234,19 +2227,19 @@ int run_response(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
   TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pc.state_bytes));
   TBPM_TRY(launch_pair_init(ctx, pl.precision, n, Sh, ctx->ws_psi.p, op == 0 ? ctx->ws_jpsi.p : nullptr, phase,
                             ctx->ws_phi[0].p));
-  release(ctx, ctx->ws_psi);
-  release(ctx, ctx->ws_jpsi);
+  release_if_tight(ctx, ctx->ws_psi);
+  release_if_tight(ctx, ctx->ws_jpsi);
   TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pc.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_phi2[1], pc.state_bytes));
   // F = f(H) X, consuming X in ws_phi[0]
   TBPM_TRY(apply_series_bufs(ctx, lat, pc, ctx->ws_phi[0].p, ctx->ws_phi[1].p, ctx->ws_phi2[1].p, coef, nf));
-  release(ctx, ctx->ws_phi[0]);
+  release_if_tight(ctx, ctx->ws_phi[0]);
   TBPM_TRY(make_states());
   TBPM_TRY(launch_pair_split(ctx, pl.precision, n, Sh, ctx->ws_psi.p, op == 0 ? ctx->ws_jpsi.p : nullptr, phase,
                              ctx->ws_phi2[1].p));
-  release(ctx, ctx->ws_psi);
-  release(ctx, ctx->ws_jpsi);
-  release(ctx, ctx->ws_phi2[0]);
+  release_if_tight(ctx, ctx->ws_psi);
+  release_if_tight(ctx, ctx->ws_jpsi);
+  release_if_tight(ctx, ctx->ws_phi2[0]);
   std::swap(ctx->ws_phi[0], ctx->ws_phi2[1]);  // Y(0) = [f psi | (1 - f) O psi] starts the propagation
   const int64_t W = n_steps + 1;
   TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * 2 * (size_t)W * Sh));
@@ -2259,8 +2252,8 @@ int run_response(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
     std::swap(ctx->ws_phi[0], ctx->ws_phi2[0]);
     const int r = choose_block(ctx, lat, &rc, pc, n_steps, &b, nullptr, nullptr);
     std::swap(ctx->ws_phi[0], ctx->ws_phi2[0]);
-    release(ctx, ctx->ws_phi2[0]);
-    release(ctx, ctx->ws_psi);
+    release_if_tight(ctx, ctx->ws_phi2[0]);
+    release_if_tight(ctx, ctx->ws_psi);
     TBPM_TRY(r);
   }
   BlockHook hook = [&](int64_t start, int bb, const void* first) -> int {
@@ -2818,7 +2811,7 @@ int tbpm_charge_density(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
     // phi = f^{1/2}(H) psi into ws_phi2[0], consuming psi in ws_phi[0]
     TBPM_TRY(apply_series_bufs(ctx, lat, pl, ctx->ws_phi[0].p, ctx->ws_phi[1].p, ctx->ws_phi2[0].p, coef, nf));
     std::swap(ctx->ws_phi[0], ctx->ws_phi2[0]);
-    release(ctx, ctx->ws_phi2[0]);
+    release_if_tight(ctx, ctx->ws_phi2[0]);
     const int64_t elems = n * pl.Spad;
     TBPM_TRY(ensure(ctx, ctx->ws_ec, sizeof(double) * (size_t)elems));
     double* z = (double*)ctx->ws_ec.p;
@@ -2831,8 +2824,8 @@ int tbpm_charge_density(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
         std::swap(ctx->ws_phi[0], ctx->ws_phi2[0]);
         const int r = choose_block(ctx, lat, rq, pc, rq->n_steps, &b, nullptr, nullptr);
         std::swap(ctx->ws_phi[0], ctx->ws_phi2[0]);
-        release(ctx, ctx->ws_phi2[0]);
-        release(ctx, ctx->ws_psi);
+        release_if_tight(ctx, ctx->ws_phi2[0]);
+        release_if_tight(ctx, ctx->ws_psi);
         TBPM_TRY(r);
       }
       BlockHook hook = [&](int64_t, int bb, const void* first) -> int {

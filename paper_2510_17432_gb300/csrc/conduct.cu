@@ -55,7 +55,7 @@ __device__ __forceinline__ R bond_weight(const Args& a, int sub, int d) {
 }
 
 // y = J_alpha x for one block of states [n_sites][S].  Bound: HBM; 64-bit divisions per neighbour had made it
-// issue-bound (36.6 us on 2.1M sites, now CURRENT_NOW).
+// issue-bound (36.6 us on 2.1M sites of the full layout, now 26.9 us).
 template <typename R, int SPT>
 __global__ void __launch_bounds__(kThreads) k_current(CurArgs c, const void* xv, void* yv) {
   using PK = Pack<R, SPT>;
@@ -117,7 +117,7 @@ struct XdotArgs {
 // added at the fold.  Every 16 units the 32 sums are reduce-scattered over the lanes of a state pair
 // (31 shuffles instead of 160 for a tree per sum) and each lane adds the ones it keeps in FP64.
 // Bound: L1 and FP32 issue for many pairs, HBM for one block against a few.  On 2.1M sites 16 x 64 blocks
-// took 3320 us with a shuffle tree per sum and scalar FMAs, XDOT_NOW.
+// took 3320 us with a shuffle tree per sum and scalar FMAs, now 1206 us.
 struct XTile {
   int at, bt;   // tiles along A and B
   int wa, wb;   // tiles of one CTA along A and B (wa wb divides 8)
