@@ -517,7 +517,7 @@ int tbpm_destroy(tbpm_ctx* ctx) {
                     &ctx->ws_counter, &ctx->ws_mu, &ctx->ws_table, &ctx->ws_aux, &ctx->ws_out,
                     &ctx->ws_energies, &ctx->ws_recon, &ctx->ws_phi2[0], &ctx->ws_phi2[1],
                     &ctx->ws_fused_partials, &ctx->ws_qe, &ctx->ws_qe_coef, &ctx->ws_xdot, &ctx->ws_blk, &ctx->ws_blk_coef,
-                    &ctx->ws_jpsi, &ctx->ws_ec, &ctx->ws_fermi};
+                    &ctx->ws_jpsi, &ctx->ws_ec, &ctx->ws_fermi, &ctx->ws_packets};
   for (DevBuf* b : bufs) release(ctx, *b);
   cudaStreamSynchronize(ctx->stream);
   for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
@@ -560,6 +560,7 @@ int tbpm_set_fusion(tbpm_ctx* ctx, int enable) {
     return TBPM_EINVAL;
   }
   ctx->fusion = enable;
+  ctx->fusion_set = true;
   return TBPM_OK;
 }
 
@@ -1349,6 +1350,21 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
   ctx->queue_live[k] = true;
 }
 
+// Whether the resident kernel runs this moment request: a small lattice, unless a chosen fusion mode names
+// another pass that takes it (mode 0: one step per launch).  Where the register sweep takes the lattice as
+// well, the resident kernel is the faster one up to its own limit for four and more states (us per step,
+// resident against sweep: 8 states on 300 x 300 honeycomb cells 8.8 / 13.4, 4 states on 256 x 256 4.6 / 7.1),
+// but not for large blocks of one or two states, whose 8-byte and single-pair units leave its shared-memory
+// reads half empty (two states: 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state: 262k 4.5 / 4.3,
+// 33k 2.1 / 2.9, 1.6M 16.2 / 6.4).
+bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
+  if (ctx->fusion_set && (ctx->fusion == 0 || fused_applicable(lat, pl.precision, pl.Spad) ||
+                          (ctx->fusion >= 8 && sweep_ok(lat, pl))))
+    return false;
+  if (pl.Spad <= 2 && pl.n * pl.Spad > (pl.Spad == 1 ? 200000 : 1000000) && sweep_ok(lat, pl)) return false;
+  return resident_applicable(ctx, lat, pl.precision, pl.Spad, steps);
+}
+
 // Moments of all Spad states into d_mu [Spad][M][2].
 int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl_in, int64_t M,
                 double* d_mu) {
@@ -1357,6 +1373,18 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     return TBPM_EINVAL;
   }
   Plan pl = pl_in;
+  if (use_resident(ctx, lat, pl, M / 2)) {
+    TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
+    TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
+    RecurrenceArgs a;
+    TBPM_TRY(base_args(ctx, lat, pl, &a, 3));
+    a.mu = d_mu;
+    a.M = (int)M;
+    const int tok = phase_begin(ctx, 0);
+    TBPM_TRY(launch_resident(ctx, lat, a, pl.precision, ctx->ws_phi[0].p, M / 2));
+    phase_end(ctx, tok);
+    return TBPM_OK;
+  }
   int fmode = 0;
   TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));
   const int64_t steps = M / 2;
@@ -2362,6 +2390,10 @@ int tbpm_moment_pass_kind(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_r
   }
   const int m = ctx->fusion;  // -1: autotuned on first use, reported as the mode it would time first
   const int64_t M = req->n_moments > 0 ? req->n_moments : truncation_order_host(req->n_steps * pl.tau);
+  if (use_resident(ctx, lat, pl, M / 2)) {
+    *kind = TBPM_PASS_STENCIL;
+    return TBPM_OK;
+  }
   if (m > 0 && fused_applicable(lat, pl.precision, pl.Spad) && M / 2 - 1 >= fused_steps(m)) {
     const int band = (m == 8 ? 128 : m == 9 ? 192 : 256) / (pl.Spad / 2);
     *kind = (m >= 8 && m <= 10 && lat->geom.Lx >= band) ? TBPM_PASS_SWEEP

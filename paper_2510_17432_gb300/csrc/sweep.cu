@@ -926,7 +926,7 @@ int sweep_status(tbpm_ctx* ctx) {
   const int v = *st;
   if (v != 0) {
     *st = 0;
-    set_error("fused sweep: a bounded wait for a row copy expired (code %d)", v);
+    set_error("moment recurrence: a bounded wait expired (code %d: 1, 2 a row copy of the sweep, 3 a neighbour's step)", v);
     return TBPM_ETIMEOUT;
   }
   return TBPM_OK;

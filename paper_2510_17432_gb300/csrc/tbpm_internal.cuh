@@ -199,6 +199,7 @@ struct tbpm_ctx {
   // time blocks buffer up to 32 Chebyshev vectors and flush them into the accumulators at once
   bool buffer_blocks = true;
   int fusion = 8;  // temporal-fusion mode of the moment pass (8 = four-step register sweep; -1 = autotuned)
+  bool fusion_set = false;  // chosen by tbpm_set_fusion: a lattice a mode's fused pass takes then runs that pass
   // autotuned fusion modes: key (kind, Lx, Ly, Lz, pbc bits, path, Spad, precision, disorder) -> mode
   std::vector<std::pair<std::vector<int64_t>, int>> fusion_choice;
   std::vector<std::pair<int, double>> fusion_timings;  // last autotune: (mode, ms per step)
@@ -212,6 +213,10 @@ struct tbpm_ctx {
   bool use_graphs = true;
   std::vector<Graph> graphs;
   std::vector<std::vector<uint64_t>> graph_seen;
+  // packets of the resident recurrence and the last tag they carry
+  tbpm::DevBuf ws_packets;
+  size_t packet_cap = 0;
+  int64_t packet_tag = 0;
   int max_pass_states = 0;  // cap on states per pass of the OC, DP and CD drivers (0 = by memory)
   double* pinned = nullptr;
   size_t pinned_cap = 0;
@@ -410,6 +415,11 @@ int launch_sweep_window(tbpm_ctx* ctx, const tbpm_lattice* lat, const Recurrence
 int fused_steps(int variant);
 int launch_fused_pass(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, const void* prev_in,
                       const void* cur_in, void* prev_out, void* cur_out, int step0, int variant);
+
+// every step of a small lattice's moment recurrence in one launch (csrc/resident.cu)
+bool resident_applicable(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, int Spad, int64_t steps);
+int launch_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, int precision, const void* x0,
+                    int64_t steps);
 
 enum { ACC_FIRST = 0, ACC_REGULAR = 1, ACC_NOSPMV = 2 };
 

@@ -44,7 +44,7 @@ def _pair(capi, ctx, spec):
     lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(spec["kind"], spec["L"], t=spec["t"], W=spec["W"], seed=77,
                                                           vacancy_frac=spec.get("vac", 0.0),
                                                           pbc=spec.get("pbc", (1, 1, 1))))
-    ol = olat.build_lattice(spec["kind"], tuple(spec["L"]) + (1,), t=spec["t"], W=spec["W"], seed=77,
+    ol = olat.build_lattice(spec["kind"], (tuple(spec["L"]) + (1,))[:3], t=spec["t"], W=spec["W"], seed=77,
                             vacancy_frac=spec.get("vac", 0.0), pbc=spec.get("pbc", (1, 1, 1)))
     return lat, ol
 
@@ -84,6 +84,7 @@ def _moments(capi, ctx, lat, S, M, mode, sites=None):
 @pytest.mark.parametrize("name,spec,S,M", SWEEPS, ids=[c[0] for c in SWEEPS])
 def test_sweep_shapes_match_the_one_step_pass_and_the_oracle(capi, ctx, name, spec, S, M):
     lat, ol = _pair(capi, ctx, spec)
+    capi.tbpm_set_fusion(ctx, 8)
     assert capi.tbpm_moment_pass_kind(ctx, lat, capi.request(n_states=S, n_moments=M)) == capi.PASS_SWEEP
     got, one = _moments(capi, ctx, lat, S, M, 8), _moments(capi, ctx, lat, S, M, 0)
     assert np.max(np.abs(got - one)) <= 1e-6
@@ -136,3 +137,47 @@ def test_window_passes_of_the_new_shapes(capi, ctx, name, spec, S):
         for k in range(E.size):
             assert np.max(np.abs(C[s, k] - Cref[k])) <= 3e-5 * np.max(np.abs(Cref[k])), (form, k)
     capi.tbpm_lattice_destroy(lat)
+
+
+# Small lattices whose whole recurrence runs in one launch: one line per CTA and several, fewer lines than
+# CTAs, a ragged last CTA, a lattice near the shared-memory limit, every kind and boundary, widths of one
+# and two cells, both precisions, and M / 2 around the batches of eight steps whose sums are stored together.
+RESIDENT = [
+    ("square64_c128", dict(kind=0, L=(64, 64), t=1.0, W=1.0), 1, 1, 96),
+    ("square_thin_c128", dict(kind=0, L=(2, 300), t=1.0, W=0.5), 3, 1, 34),
+    ("square_one_row", dict(kind=0, L=(50, 1), t=1.0, W=1.0), 2, 0, 32),
+    ("honey_ribbon", dict(kind=1, L=(45, 47), t=1.0, W=1.0, pbc=(1, 0, 1)), 4, 0, 48),
+    ("honey_two_cells_open", dict(kind=1, L=(2, 155), t=-2.7, W=0.0, pbc=(0, 1, 1)), 1, 0, 50),
+    ("honey_c128_S5", dict(kind=1, L=(31, 160), t=-2.7, W=1.0), 5, 1, 30),
+    ("cubic_S32", dict(kind=2, L=(7, 9, 11), t=1.0, W=1.5, pbc=(1, 1, 0)), 32, 0, 20),
+    ("cubic_c128", dict(kind=2, L=(12, 5, 8), t=1.0, W=0.3, pbc=(0, 1, 1)), 2, 1, 18),
+    ("cubic_lines_over_ctas", dict(kind=2, L=(10, 31, 13), t=1.0, W=2.0), 8, 0, 16),
+    ("square_large_S2", dict(kind=0, L=(95, 2900), t=1.0, W=0.0), 2, 0, 12),
+    ("square_large_S1", dict(kind=0, L=(61, 9000), t=1.0, W=1.0, pbc=(1, 0, 1)), 1, 0, 36),
+]
+
+
+@pytest.mark.parametrize("name,spec,S,prec,M", RESIDENT, ids=[c[0] for c in RESIDENT])
+def test_resident_recurrence_matches_the_oracle(capi, name, spec, S, prec, M):
+    ctx = capi.tbpm_create(0)  # the resident kernel is the default; a chosen mode may name another pass
+    try:
+        lat, ol = _pair(capi, ctx, spec)
+        req = capi.request(n_states=S, precision=prec, n_moments=M, state_seed=3)
+        mu = np.zeros((S, M, 2))
+        capi.tbpm_moments(ctx, lat, req, mu)
+        again = np.zeros_like(mu)
+        launches = capi.tbpm_launch_count(ctx)
+        capi.tbpm_moments(ctx, lat, req, again)
+        assert capi.tbpm_launch_count(ctx) - launches == 3  # states, recurrence, sums
+        assert np.array_equal(mu, again)
+        capi.tbpm_set_fusion(ctx, 0)
+        one = np.zeros_like(mu)
+        capi.tbpm_moments(ctx, lat, req, one)
+        assert np.max(np.abs(mu - one)) <= (1e-12 if prec else 1e-6)
+        psi = oprop.random_phase_states(ol, 3, S)
+        for s in {0, S - 1}:
+            ref = oprop.moments(ol, psi[s], psi[s], M)
+            assert np.max(np.abs(mu[s, :, 0] + 1j * mu[s, :, 1] - ref)) <= (1e-11 if prec else 1e-5)
+        capi.tbpm_lattice_destroy(lat)
+    finally:
+        capi.tbpm_destroy(ctx)
