@@ -905,6 +905,10 @@ int launch_moment_step(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, bo
   const int spt = spt_of(precision, a.S);
   if (a.taps && precision == TBPM_C64 && spt == 2) return launch_taps_moment(ctx, a, first);
   if (ell_batched(a)) return launch_ell<true>(ctx, a, precision, first);
+  if (!csr && a.geom.kind == TBPM_CUBIC) {
+    const int r = launch_cubic_march(ctx, a, precision, first, true);
+    if (r != TBPM_EUNSUPPORTED) return r;
+  }
   void* fn;
   if (precision == TBPM_C128) fn = moment_kernel<double, 1>(a.geom.kind, csr, first);
   else if (spt == 2) fn = moment_kernel<float, 2>(a.geom.kind, csr, first);
@@ -926,6 +930,10 @@ int launch_accum_step(tbpm_ctx* ctx, const AccumArgs& g, int precision, int mode
   }
   if (mode != ACC_NOSPMV && g.j_lo >= g.b && g.j_done < 0 && ell_batched(g.r))
     return launch_ell<false>(ctx, g.r, precision, mode == ACC_FIRST);  // a plain step, loads batched
+  if (mode != ACC_NOSPMV && g.j_lo >= g.b && g.j_done < 0 && !csr && g.r.geom.kind == TBPM_CUBIC) {
+    const int r = launch_cubic_march(ctx, g.r, precision, mode == ACC_FIRST, false);
+    if (r != TBPM_EUNSUPPORTED) return r;
+  }
   void* fn;
   if (precision == TBPM_C128) fn = accum_kernel<double, 1>(g.r.geom.kind, csr, mode);
   else if (spt == 2) fn = accum_kernel<float, 2>(g.r.geom.kind, csr, mode);

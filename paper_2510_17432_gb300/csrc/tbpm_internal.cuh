@@ -380,6 +380,8 @@ int launch_taps_moment(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);
 int launch_taps_step(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);  // recurrence only
 size_t taps_partials_bytes(const RecurrenceArgs& a);
 int launch_accum_step(tbpm_ctx* ctx, const AccumArgs& a, int precision, int mode);
+// one step on the cubic stencil (csrc/march.cu); TBPM_EUNSUPPORTED: too many columns for it
+int launch_cubic_march(tbpm_ctx* ctx, const RecurrenceArgs& ra, int precision, bool first, bool moments);
 // acc_e (+)= sum_{t<T} a_t(e) [(-i)^t] phi_t over T consecutive buffered state blocks of n_numbers complex
 // numbers and nb consecutive accumulators (csrc/flush.cu): real amplitudes a_t(e) at
 // amp[(t * nb + e) * amp_stride]; rot: with the powers of -i (the window starts at a multiple of four terms);

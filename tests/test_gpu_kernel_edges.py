@@ -181,3 +181,39 @@ def test_resident_recurrence_matches_the_oracle(capi, name, spec, S, prec, M):
         capi.tbpm_lattice_destroy(lat)
     finally:
         capi.tbpm_destroy(ctx)
+
+
+# The cubic march: tiles cut at every edge, lattices of one tile and less, one and two planes, every number of
+# state pairs per CTA, segments of planes, open boundaries, both precisions.
+MARCH = [
+    ("tile_and_one_S8", (9, 9, 5), dict(), 8, 0),
+    ("one_plane_S1", (33, 7, 1), dict(), 1, 0),
+    ("two_planes_open_z", (5, 4, 2), dict(pbc=(1, 1, 0)), 2, 0),
+    ("thin_x_S32", (1, 17, 6), dict(), 32, 0),
+    ("open_all_S16", (13, 21, 9), dict(pbc=(0, 0, 0)), 16, 0),
+    ("many_segments_S4", (8, 8, 200), dict(), 4, 0),
+    ("c128_S3", (10, 11, 12), dict(pbc=(0, 1, 1)), 3, 1),
+    ("c128_S1_wide", (70, 3, 4), dict(pbc=(1, 0, 1)), 1, 1),
+]
+
+
+@pytest.mark.parametrize("name,L,kw,S,prec", MARCH, ids=[c[0] for c in MARCH])
+def test_cubic_march_matches_the_oracle(capi, ctx, name, L, kw, S, prec):
+    spec = dict(kind=2, L=L, t=1.0, W=1.0, **kw)
+    lat, ol = _pair(capi, ctx, spec)
+    psi = oprop.random_phase_states(ol, 3, S)
+    M, Nt = 18, 7
+    mu = np.zeros((S, M, 2))
+    capi.tbpm_set_fusion(ctx, 0)  # one step per launch
+    try:
+        capi.tbpm_moments(ctx, lat, capi.request(n_states=S, precision=prec, n_moments=M, state_seed=3), mu)
+    finally:
+        capi.tbpm_set_fusion(ctx, 8)
+    C = np.zeros((S, Nt + 1), np.complex128)
+    capi.tbpm_correlation(ctx, lat, capi.request(n_states=S, precision=prec, form=2, n_steps=Nt, time_block=4,
+                                                 state_seed=3), C)
+    tol = 1e-11 if prec else 1e-5
+    for s in {0, S - 1}:
+        assert np.max(np.abs(mu[s, :, 0] + 1j * mu[s, :, 1] - oprop.moments(ol, psi[s], psi[s], M))) <= tol
+        assert np.max(np.abs(C[s] - oprop.correlation_sequential(ol, psi[s], Nt, np.pi))) <= tol
+    capi.tbpm_lattice_destroy(lat)
