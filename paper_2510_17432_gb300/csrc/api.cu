@@ -166,16 +166,19 @@ __global__ void k_bounds_final(const Bounds3* part, int n, double* out) {
   }
   sh[threadIdx.x] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Bounds3 r = sh[0];
-    for (int w = 1; w < kT; ++w) {
-      r.emax = fmax(r.emax, sh[w].emax);
-      r.emin = fmin(r.emin, sh[w].emin);
-      r.deg += sh[w].deg;
+  for (int w = kT / 2; w >= 1; w >>= 1) {  // maxima, minima and a sum of integers: any order gives the same
+    if (threadIdx.x < w) {
+      Bounds3 &r = sh[threadIdx.x], o = sh[threadIdx.x + w];
+      r.emax = fmax(r.emax, o.emax);
+      r.emin = fmin(r.emin, o.emin);
+      r.deg += o.deg;
     }
-    out[0] = r.emax;
-    out[1] = r.emin;
-    out[2] = r.deg;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    out[0] = sh[0].emax;
+    out[1] = sh[0].emin;
+    out[2] = sh[0].deg;
   }
 }
 

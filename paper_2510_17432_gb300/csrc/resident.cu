@@ -104,24 +104,6 @@ __device__ __forceinline__ bool receive(const ulonglong2* p, unsigned tag, Pack<
   return true;
 }
 
-// Sums that travel through the shuffles: FP32 as value + error, FP64 plain.
-struct Pair32 {
-  float h, l;
-};
-__device__ __forceinline__ Pair32 sum_of(float v) { return {v, 0.f}; }
-__device__ __forceinline__ double sum_of(double v) { return v; }
-__device__ __forceinline__ Pair32 add(Pair32 a, Pair32 b) {
-  const float s = a.h + b.h, t = s - a.h;
-  return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
-}
-__device__ __forceinline__ double add(double a, double b) { return a + b; }
-__device__ __forceinline__ Pair32 xor_lane(Pair32 v, int off) {
-  return {__shfl_xor_sync(0xffffffffu, v.h, off), __shfl_xor_sync(0xffffffffu, v.l, off)};
-}
-__device__ __forceinline__ double xor_lane(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-__device__ __forceinline__ double value_of(Pair32 v) { return (double)v.h + (double)v.l; }
-__device__ __forceinline__ double value_of(double v) { return v; }
-
 // Neighbour lines of a line, in the neighbour order of the stencil: y + 1, y - 1, z + 1, z - 1 (-1: none).
 template <int KIND>
 __device__ __forceinline__ void line_neighbours(const Geom& g, int64_t row, int64_t (&nb)[4]) {
@@ -283,8 +265,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
       if (tid == 0) atomicExch(a.status, 3);
       return;
     }
-    // warp sums of this step: the lanes of a state pair first halve the NV values they share (as long as
-    // there are lanes to share them), then add up the rest
+    // warp sums of this step
     {
       using SumT = decltype(sum_of(R(0)));
       SumT v[NV];
@@ -298,35 +279,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
           }
         }
       }
-      int m = NV, base = 0;  // values this lane still holds, and the first one's index
-#pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) {
-        if (off < P) break;
-        const bool up = (lane & off) != 0;
-        if (m > 1) {
-          m >>= 1;
-          if (up) base += m;
-#pragma unroll
-          for (int k = 0; k < NV / 2; ++k) {
-            if (k < m) {
-              const SumT keep = up ? v[k + m] : v[k], send = up ? v[k] : v[k + m];
-              v[k] = add(keep, xor_lane(send, off));
-            }
-          }
-        } else {
-          v[0] = add(v[0], xor_lane(v[0], off));
-        }
-      }
-      // one lane per (pair, group of values) writes: lanes that differ only in the plain levels agree
-      const int levels = 5 - logP;                    // halvings plus plain levels
-      const int halvings = levels < (NV == 4 ? 2 : 1) ? levels : (NV == 4 ? 2 : 1);
-      const int plain_mask = (32 >> halvings) - P;    // lane bits summed plainly
       double* slot = red + ((size_t)(n & (kResBatch - 1)) * warps + warp) * P * NV + (lane & (P - 1)) * NV;
-      if ((lane & plain_mask) == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-          if (k < m) slot[base + k] = value_of(v[k]);
-      }
+      reduce_lanes<NV>(v, P, logP, lane, [&](int k, double t) { slot[k] = t; });
     }
     if ((n & (kResBatch - 1)) == kResBatch - 1 || n == a.steps - 1) {
       const int n0 = n & ~(kResBatch - 1), have = n - n0 + 1;

@@ -5,9 +5,12 @@
 // the cost halving of Eq. cheby_prod) per launch of k_serve_step.  Requests of different
 // lattice kinds, sizes, state counts and moment counts share that launch: the grid walks a
 // global list of tiles, each tile belongs to one request and is processed with that request's
-// stencil or ELL neighbour rule.  Every tile writes its own FP64 partial sums and the last tile
-// of a request sums them in tile order, so a request's moments do not depend on what else is in
-// the batch: results are bit-identical alone and in any mix.  A request that has produced its
+// stencil or ELL neighbour rule.  Every tile writes its own FP64 partial sums; the next launch holds one
+// more tile per request that adds them in a fixed order and writes the step's two moments (the last
+// step's are added before the reconstruction), so a request's moments do not depend on what else is in
+// the batch: results are bit-identical alone and in any mix.  (The last tile of a step to finish used to
+// add them at the end of the same launch: up to 96 sums over a hundred tiles by one CTA while the others
+// were idle, about 45 of the 107 us of a step of sixteen mixed requests of 11M site-states; now 67 us beside a lane.)  A request that has produced its
 // M moments leaves the batch, its DOS is reconstructed (Jackson kernel) and copied to pinned
 // host memory, and its memory is released for the next admission.
 //
@@ -35,15 +38,16 @@
 
 namespace tbpm {
 
-constexpr int kServeTU = 32 * kThreads;  // largest tile (32 units per thread, FP32 partial sums)
+constexpr int kServeTU = 16 * kThreads;  // largest tile (16 units per thread, FP32 partial sums)
+constexpr int kItemCache = 128;
 constexpr int64_t kLaneSiteStates = 1 << 21;  // full sites x padded states of a direct-lane request
 
-// Units per tile of a request with `units` thread units: 32 per thread (the per-tile reduction
-// and bookkeeping amortised) unless the request would get fewer than 64 tiles, then fewer.
+// Units per tile of a request with `units` thread units: 16 per thread (the per-tile reduction
+// and bookkeeping amortised; 32 left the last of two waves of tiles nearly empty) unless the request would get fewer than 64 tiles, then fewer.
 // Depends only on the request, so its partial sums (and results) are the same alone and in any mix.
 __host__ __device__ inline int serve_tile_units(int64_t units) {
   int upt = 1;
-  while (upt < 32 && (int64_t)upt * kThreads * 64 < units) upt <<= 1;
+  while (upt < 16 && (int64_t)upt * kThreads * 64 < units) upt <<= 1;
   return upt * kThreads;
 }
 
@@ -64,18 +68,17 @@ struct ServeItem {
   uint32_t line_magic;  // ceil(2^32 / upr), for u / upr with u < tu <= kServeTU
   int tu;               // units per tile (a multiple of kThreads, <= kServeTU)
   int64_t n_tiles, tile_begin;
-  double* tile_partials;  // [n_tiles][S][3]
-  unsigned* counter;
+  double* tile_partials;  // [step & 1][n_tiles][S][2]
   double* mu;
   int M;
-  int step;
+  int step;  // of the first launch after the item was uploaded
 };
 
 // One unit: neighbour sum, output, and the unit's terms of A, B.
 template <int KIND, bool CSR, typename R, int SPT>
 __device__ __forceinline__ void serve_unit(const ServeItem& it, const Pack<R, SPT>* __restrict__ cur,
                                            Pack<R, SPT>* __restrict__ po, const LineBases& b, int64_t site_unit,
-                                           int u, int p, bool first, R th, R dc, R (&acc)[3 * SPT]) {
+                                           int u, int p, bool first, R th, R dc, R (&acc)[2 * SPT]) {
   using PK = Pack<R, SPT>;
   constexpr int Z = CSR ? 6 : (KIND == TBPM_HONEYCOMB ? 3 : (KIND == TBPM_SQUARE ? 4 : 6));
   const int64_t own = site_unit;
@@ -123,20 +126,16 @@ __device__ __forceinline__ void serve_unit(const ServeItem& it, const Pack<R, SP
 #pragma unroll
   for (int q = 0; q < SPT; ++q) {
     const R pr = ph.v[2 * q], pi = ph.v[2 * q + 1], orr = o.v[2 * q], oi = o.v[2 * q + 1];
-    acc[3 * q] += pr * pr + pi * pi;
-    acc[3 * q + 1] += orr * pr + oi * pi;
-    acc[3 * q + 2] += orr * pi - oi * pr;
+    acc[2 * q] += pr * pr + pi * pi;
+    acc[2 * q + 1] += orr * pr + oi * pi;  // the imaginary part vanishes for a Hermitian H~
   }
 }
 
-// One tile of one request; the last tile of the request finishes its step.
-// `it` is the block's shared-memory copy; `git` the item in global memory, whose step field the
-// last tile advances for the next launch.
+// One tile of one request at the given step; `it` is the block's shared-memory copy of the item.
 template <int KIND, bool CSR, typename R, int SPT>
-__device__ void serve_tile(const ServeItem* itp, ServeItem* git, int64_t lt, double (*red)[32][6], unsigned& ticket) {
+__device__ void serve_tile(const ServeItem* itp, int64_t lt, int step, double (*red)[32][4]) {
   using PK = Pack<R, SPT>;
   const ServeItem& it = *itp;
-  const int step = it.step;
   const bool first = step == 0;
   const PK* cur = reinterpret_cast<const PK*>((step & 1) ? it.buf1 : it.buf0);
   PK* po = reinterpret_cast<PK*>((step & 1) ? it.buf0 : it.buf1);
@@ -149,9 +148,9 @@ __device__ void serve_tile(const ServeItem* itp, ServeItem* git, int64_t lt, dou
     th = first ? it.thop : 2.0 * it.thop;
     dc = first ? it.diag_const : 2.0 * it.diag_const;
   }
-  R acc[3 * SPT];
+  R acc[2 * SPT];
 #pragma unroll
-  for (int k = 0; k < 3 * SPT; ++k) acc[k] = R(0);
+  for (int k = 0; k < 2 * SPT; ++k) acc[k] = R(0);
 
   if constexpr (CSR) {
     const int64_t n_units = it.n_sites * P;
@@ -186,80 +185,77 @@ __device__ void serve_tile(const ServeItem* itp, ServeItem* git, int64_t lt, dou
     }
   }
 
-  // tile partial sums: FP32 (at most 32 units per thread) -> FP64 warp and block trees
-  double v[3 * SPT];
-#pragma unroll
-  for (int k = 0; k < 3 * SPT; ++k) v[k] = (double)acc[k];
+  // tile partial sums: FP32 (at most 32 units per thread), compensated over the lanes, FP64 over the warps
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  decltype(sum_of(R(0))) v[2 * SPT];
 #pragma unroll
-  for (int k = 0; k < 3 * SPT; ++k)
-    for (int off = 16; off >= P; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-  if (lane < P) {
-#pragma unroll
-    for (int k = 0; k < 3 * SPT; ++k) red[warp][lane][k] = v[k];
-  }
+  for (int k = 0; k < 2 * SPT; ++k) v[k] = sum_of(acc[k]);
+  reduce_lanes<2 * SPT>(v, P, it.logP, lane, [&](int k, double t) { red[warp][lane & (P - 1)][k] = t; });
   __syncthreads();
-  const int SC = it.S * 3;
+  const int SC = it.S * 2;
   if (threadIdx.x < SC) {
-    const int q = threadIdx.x, s = q / 3, c = q - 3 * s;
-    const int pp = s / SPT, k = (s - pp * SPT) * 3 + c;
+    const int q = threadIdx.x, s = q >> 1, c = q & 1;
+    const int pp = s / SPT, k = (s - pp * SPT) * 2 + c;
     double a = 0.0;
     for (int w = 0; w < kWarps; ++w) a += red[w][pp][k];
-    it.tile_partials[(size_t)lt * SC + q] = a;
-    __threadfence();
+    it.tile_partials[((size_t)(step & 1) * it.n_tiles + lt) * SC + q] = a;
   }
   __syncthreads();
-  if (threadIdx.x == 0) ticket = atomicAdd(it.counter, 1u);
-  __syncthreads();
-  if (ticket == (unsigned)(it.n_tiles - 1)) {
-    __threadfence();
-    for (int q = warp; q < SC; q += kWarps) {
-      double a = 0.0;
-      for (int64_t t = lane; t < it.n_tiles; t += 32) a += __ldcg(it.tile_partials + (size_t)t * SC + q);
-      for (int off = 16; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-      if (lane == 0) {
-        const int s = q / 3, c = q - 3 * s;
-        double* ms = it.mu + (size_t)s * it.M * 2;
-        if (first) {
-          if (c == 0) { ms[0] = a; ms[1] = 0.0; }
-          else if (c == 1) ms[2] = a;
-          else ms[3] = a;
-        } else {
-          if (c == 0) { ms[4 * step] = 2.0 * a - ms[0]; ms[4 * step + 1] = -ms[1]; }
-          else if (c == 1) ms[4 * step + 2] = 2.0 * a - ms[2];
-          else ms[4 * step + 3] = 2.0 * a - ms[3];
-        }
-      }
+}
+
+// The moments of one finished step from its tiles' sums: lanes take the 2 S values, warps the tiles.
+__device__ void serve_moments(const ServeItem& it, int step, double (*red)[32][4]) {
+  const int SC = it.S * 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double* p = it.tile_partials + (size_t)(step & 1) * it.n_tiles * SC;
+  double* sh = &red[0][0][0];  // [warps][32]
+  for (int q0 = 0; q0 < SC; q0 += 32) {
+    const int q = q0 + lane;
+    double a = 0.0;
+    if (q < SC) {
+#pragma unroll 16
+      for (int t = warp; t < (int)it.n_tiles; t += kWarps) a += __ldcg(p + (size_t)t * SC + q);
+    }
+    sh[warp * 32 + lane] = a;
+    __syncthreads();
+    if (warp == 0 && q < SC) {
+      a = 0.0;
+      for (int w = 0; w < kWarps; ++w) a += sh[w * 32 + lane];
+      double* ms = it.mu + (size_t)(q >> 1) * it.M * 2 + 2 * (q & 1);
+      ms[4 * (size_t)step] = step == 0 ? a : 2.0 * a - ms[0];
+      ms[4 * (size_t)step + 1] = 0.0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      *it.counter = 0u;
-      git->step = step + 1;
-    }
   }
-  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kThreads) k_serve_last(ServeItem it, int step) {
+  __shared__ double red[kWarps][32][4];
+  serve_moments(it, step, red);
 }
 
 template <int KIND, bool CSR>
-__device__ __forceinline__ void serve_dispatch_prec(const ServeItem* it, ServeItem* git, int64_t lt,
-                                                    double (*red)[32][6], unsigned& ticket) {
-  if (it->precision == TBPM_C128) serve_tile<KIND, CSR, double, 1>(it, git, lt, red, ticket);
-  else if (it->spt == 2) serve_tile<KIND, CSR, float, 2>(it, git, lt, red, ticket);
-  else serve_tile<KIND, CSR, float, 1>(it, git, lt, red, ticket);
+__device__ __forceinline__ void serve_dispatch_prec(const ServeItem* it, int64_t lt, int step, double (*red)[32][4]) {
+  if (it->precision == TBPM_C128) serve_tile<KIND, CSR, double, 1>(it, lt, step, red);
+  else if (it->spt == 2) serve_tile<KIND, CSR, float, 2>(it, lt, step, red);
+  else serve_tile<KIND, CSR, float, 1>(it, lt, step, red);
 }
 
-__global__ void __launch_bounds__(kThreads, 4) k_serve_step(ServeItem* items, int n_items, int64_t total_tiles) {
-  __shared__ double red[kWarps][32][6];
-  __shared__ unsigned ticket;
+// tick: launches since the items were uploaded.  A request has n_tiles tiles and one that adds the sums of its
+// previous step.
+__global__ void __launch_bounds__(kThreads, 4) k_serve_step(const ServeItem* items, int n_items, int64_t total_tiles,
+                                                            int tick) {
+  __shared__ double red[kWarps][32][4];
   __shared__ ServeItem sit;  // the tile's work item, staged once per tile
   __shared__ int sit_index;
+  __shared__ int begins[kItemCache];  // the items' first tiles: the search below in shared memory
+  for (int i = threadIdx.x; i < min(n_items, kItemCache); i += kThreads) begins[i] = (int)items[i].tile_begin;
   if (threadIdx.x == 0) sit_index = -1;
   __syncthreads();
   for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
     int lo = 0, hi = n_items - 1;
     while (lo < hi) {  // last item with tile_begin <= t
       const int mid = (lo + hi + 1) >> 1;
-      if (items[mid].tile_begin <= t) lo = mid;
+      if ((mid < kItemCache ? (int64_t)begins[mid] : items[mid].tile_begin) <= t) lo = mid;
       else hi = mid - 1;
     }
     if (lo != sit_index) {
@@ -272,10 +268,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_serve_step(ServeItem* items, in
       __syncthreads();
     }
     const int64_t lt = t - sit.tile_begin;
-    if (sit.path == TBPM_PATH_CSR) serve_dispatch_prec<0, true>(&sit, items + lo, lt, red, ticket);
-    else if (sit.geom.kind == TBPM_HONEYCOMB) serve_dispatch_prec<TBPM_HONEYCOMB, false>(&sit, items + lo, lt, red, ticket);
-    else if (sit.geom.kind == TBPM_SQUARE) serve_dispatch_prec<TBPM_SQUARE, false>(&sit, items + lo, lt, red, ticket);
-    else serve_dispatch_prec<TBPM_CUBIC, false>(&sit, items + lo, lt, red, ticket);
+    const int step = sit.step + tick;
+    if (lt == sit.n_tiles) {
+      if (step > 0) serve_moments(sit, step - 1, red);
+    } else if (sit.path == TBPM_PATH_CSR) serve_dispatch_prec<0, true>(&sit, lt, step, red);
+    else if (sit.geom.kind == TBPM_HONEYCOMB) serve_dispatch_prec<TBPM_HONEYCOMB, false>(&sit, lt, step, red);
+    else if (sit.geom.kind == TBPM_SQUARE) serve_dispatch_prec<TBPM_SQUARE, false>(&sit, lt, step, red);
+    else serve_dispatch_prec<TBPM_CUBIC, false>(&sit, lt, step, red);
   }
 }
 
@@ -300,7 +299,6 @@ struct ServeJob {
   void* buf[2] = {nullptr, nullptr};
   double* mu = nullptr;
   double* tile_partials = nullptr;
-  unsigned* counter = nullptr;
   double* dE = nullptr;
   double* dD = nullptr;
   double* hD = nullptr;
@@ -347,6 +345,7 @@ struct tbpm_server {
   ServeItem* h_items[2] = {nullptr, nullptr};
   cudaEvent_t items_ev[2] = {nullptr, nullptr};
   int items_cap = 0, items_slot = 0;
+  int tick = 0;                              // launches since the items were uploaded
   std::vector<cudaEvent_t> inflight;      // end of each in-flight launch (timed)
   std::vector<cudaEvent_t> inflight_beg;  // start of each in-flight launch
   std::vector<char> inflight_live;
@@ -360,7 +359,7 @@ static size_t job_footprint(const ServeJob* j, int64_t n_sites, int64_t n_full, 
   // a direct lane holds up to four state blocks (the fused passes write a second pair) and the
   // partial sums of its passes
   const size_t states = j->lane ? 4 * j->state_bytes + (16u << 20) : 2 * j->state_bytes;
-  return lat + states + (size_t)j->n_tiles * j->Spad * 3 * 8 + (size_t)j->Spad * j->req.n_moments * 16 +
+  return lat + states + (size_t)j->n_tiles * j->Spad * 4 * 8 + (size_t)j->Spad * j->req.n_moments * 16 +
          j->energies.size() * 8 * (1 + j->S) + 4096;
 }
 
@@ -404,12 +403,11 @@ static void fail_job(tbpm_server* srv, ServeJob* j, int code) {
 
 static void release_job(tbpm_server* srv, ServeJob* j) {
   cudaStream_t st = j->lane_ctx ? j->lane_ctx->stream : srv->ctx->stream;
-  void* ps[] = {j->buf[0], j->buf[1], j->mu, j->tile_partials, j->counter, j->dE, j->dD};
+  void* ps[] = {j->buf[0], j->buf[1], j->mu, j->tile_partials, j->dE, j->dD};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, st);
   j->buf[0] = j->buf[1] = nullptr;
   j->mu = j->tile_partials = j->dE = j->dD = nullptr;
-  j->counter = nullptr;
   if (j->lat) {
     tbpm_lattice_destroy(j->lat);
     j->lat = nullptr;
@@ -486,11 +484,9 @@ static int setup_job(tbpm_server* srv, ServeJob* j) {
   TBPM_TRY(alloc(&j->buf[0], j->state_bytes));
   TBPM_TRY(alloc(&j->buf[1], j->state_bytes));
   TBPM_TRY(alloc((void**)&j->mu, sizeof(double) * 2 * (size_t)M * j->Spad));
-  TBPM_TRY(alloc((void**)&j->tile_partials, sizeof(double) * 3 * (size_t)j->Spad * j->n_tiles));
-  TBPM_TRY(alloc((void**)&j->counter, 256));
+  TBPM_TRY(alloc((void**)&j->tile_partials, sizeof(double) * 4 * (size_t)j->Spad * j->n_tiles));
   TBPM_TRY(alloc((void**)&j->dE, sizeof(double) * j->energies.size()));
   TBPM_TRY(alloc((void**)&j->dD, sizeof(double) * j->energies.size() * j->S));
-  TBPM_CK(cudaMemsetAsync(j->counter, 0, 256, st));
   TBPM_CK(cudaMemcpyAsync(j->dE, j->energies.data(), sizeof(double) * j->energies.size(), cudaMemcpyHostToDevice, st));
   TBPM_CK(cudaEventCreateWithFlags(&j->done_ev, cudaEventDisableTiming));
   tbpm_request rq = j->req;
@@ -518,7 +514,6 @@ static int setup_job(tbpm_server* srv, ServeJob* j) {
   it.n_sites = lat->n_sites;
   it.n_tiles = j->n_tiles;
   it.tile_partials = j->tile_partials;
-  it.counter = j->counter;
   it.mu = j->mu;
   it.M = (int)M;
   it.step = 0;
@@ -549,8 +544,9 @@ static int upload_items(tbpm_server* srv) {
     j->item.tile_begin = begin;
     j->item.step = (int)j->steps_done;
     srv->h_items[slot][k] = j->item;
-    begin += j->n_tiles;
+    begin += j->n_tiles + 1;
   }
+  srv->tick = 0;
   TBPM_CK(cudaMemcpyAsync(srv->d_items, srv->h_items[slot], sizeof(ServeItem) * n, cudaMemcpyHostToDevice,
                           srv->ctx->stream));
   TBPM_CK(cudaEventRecord(srv->items_ev[slot], srv->ctx->stream));
@@ -561,6 +557,8 @@ static int finish_job(tbpm_server* srv, ServeJob* j) {
   tbpm_ctx* ctx = srv->ctx;
   const int64_t nE = (int64_t)j->energies.size();
   const int M = (int)j->req.n_moments;
+  k_serve_last<<<1, kThreads, 0, ctx->stream>>>(j->item, (int)j->steps_done - 1);  // the last step's sums
+  TBPM_CK_LAUNCH(ctx);
   int r;
   if (srv->cfg.recon == TBPM_RECON_TENSOR)
     r = launch_dos_jackson_tensor_async(ctx, j->mu, j->S, M, j->dE, nE, j->lat->H0, j->lat->half, j->dD, j->h_err);
@@ -642,7 +640,7 @@ static void scheduler(tbpm_server* srv) {
         dirty = false;
       }
       int64_t total = 0;
-      for (ServeJob* j : srv->active) total += j->n_tiles;
+      for (ServeJob* j : srv->active) total += j->n_tiles + 1;
       // bound the queue depth so completion times and admission follow the device
       const size_t h = srv->inflight_head;
       if (srv->inflight.size() < depth) {
@@ -660,7 +658,7 @@ static void scheduler(tbpm_server* srv) {
       }
       const int grid = (int)std::min<int64_t>(total, (int64_t)srv->ctx->num_sms * 4);
       cudaEventRecord(srv->inflight_beg[h], srv->ctx->stream);
-      k_serve_step<<<grid, kThreads, 0, srv->ctx->stream>>>(srv->d_items, (int)srv->active.size(), total);
+      k_serve_step<<<grid, kThreads, 0, srv->ctx->stream>>>(srv->d_items, (int)srv->active.size(), total, srv->tick++);
       cudaEventRecord(srv->inflight[h], srv->ctx->stream);
       srv->inflight_live[h] = 1;
       srv->ctx->launches++;

@@ -148,6 +148,58 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NV], int P, int S, doubl
 }
 
 
+// Sums that travel through the shuffles: FP32 as value + error, FP64 plain.
+struct Pair32 {
+  float h, l;
+};
+__device__ __forceinline__ Pair32 sum_of(float v) { return {v, 0.f}; }
+__device__ __forceinline__ double sum_of(double v) { return v; }
+__device__ __forceinline__ Pair32 add(Pair32 a, Pair32 b) {
+  const float s = a.h + b.h, t = s - a.h;
+  return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
+}
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ Pair32 xor_lane(Pair32 v, int off) {
+  return {__shfl_xor_sync(0xffffffffu, v.h, off), __shfl_xor_sync(0xffffffffu, v.l, off)};
+}
+__device__ __forceinline__ double xor_lane(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ __forceinline__ double value_of(Pair32 v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double value_of(double v) { return v; }
+
+// Adds NV values over the lanes with the same lane % P (P a power of two): these lanes first halve the values
+// they share, as long as there are lanes and values to halve, then add up the rest; one lane per value calls
+// put(value index, sum).  A tree per value would take NV (5 - log P) shuffles; this takes NV - 1 + the rest.
+template <int NV, typename SumT, typename Put>
+__device__ __forceinline__ void reduce_lanes(SumT (&v)[NV], int P, int logP, int lane, Put put) {
+  static_assert(NV == 2 || NV == 4, "two or four values");
+  int m = NV, base = 0;  // values this lane still holds, and the first one's index
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    if (off < P) break;
+    const bool up = (lane & off) != 0;
+    if (m > 1) {
+      m >>= 1;
+      if (up) base += m;
+#pragma unroll
+      for (int k = 0; k < NV / 2; ++k) {
+        if (k < m) {
+          const SumT keep = up ? v[k + m] : v[k], send = up ? v[k] : v[k + m];
+          v[k] = add(keep, xor_lane(send, off));
+        }
+      }
+    } else {
+      v[0] = add(v[0], xor_lane(v[0], off));
+    }
+  }
+  const int levels = 5 - logP;  // halvings, then plain levels, whose lanes agree
+  const int most = NV == 4 ? 2 : 1, halvings = levels < most ? levels : most;
+  if ((lane & ((32 >> halvings) - P)) == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (k < m) put(base + k, value_of(v[k]));
+  }
+}
+
 // Recurrence coefficients t/|H| and D (clean lattices) for the first (x1) or a regular (x2)
 // term, in the kernel's precision.
 template <typename R>
