@@ -829,7 +829,7 @@ static int build_lattice(tbpm_ctx* ctx, tbpm_lattice* lat) {
       TBPM_CK_LAUNCH(ctx);
     }
   }
-  if (lr && d.path == TBPM_PATH_AUTO) TBPM_TRY(build_tap_chunks(ctx, lat));
+  if (lr && d.path == TBPM_PATH_AUTO) TBPM_TRY(build_tap_table(lat));
   double* res = (double*)((char*)ctx->ws_aux.p + sizeof(Bounds3) * (size_t)ctx->num_sms * 16);
   k_bounds_final<<<1, kT, 0, ctx->stream>>>(part, nb, res);
   TBPM_CK_LAUNCH(ctx);
@@ -913,7 +913,7 @@ static int ensure_dfull(tbpm_lattice* lat) {
 static void free_lattice_mem(tbpm_lattice* lat) {
   tbpm_ctx* ctx = lat->ctx;
   void* ps[] = {lat->d32, lat->d64, lat->v64, lat->ell, lat->compact, lat->full_of, lat->wrel32, lat->wrel64,
-                lat->chunks, lat->jw, lat->dfull};
+                lat->jw, lat->dfull};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, ctx->stream);
 }
@@ -1220,13 +1220,8 @@ int base_args(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pl, RecurrenceArgs* 
   a->geom = lat->geom;
   a->path = pl.full ? TBPM_PATH_STENCIL : lat->path;
   a->wrel = lat->wrel64 ? (pl.precision == TBPM_C128 ? (const void*)lat->wrel64 : (const void*)lat->wrel32) : nullptr;
-  if (lat->chunks && pl.precision == TBPM_C64 && pl.Spad >= 2) {
-    a->taps = lat->chunks;
-    a->taps_n0 = lat->n_chunks[0];
-    a->taps_n1 = lat->n_chunks[1];
-    a->taps_rx = lat->halo_x;
-    a->taps_ry = lat->halo_y;
-    a->taps_exact = lat->tap_exact ? 1 : 0;
+  if (lat->taps && pl.precision == TBPM_C64 && pl.Spad >= 2) {
+    a->taps = lat->taps.get();
   }
   if (!a->taps) TBPM_TRY(ensure_ell(ctx, lat));
   a->ell = lat->ell;
@@ -1473,7 +1468,8 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     const Geom& g = lat->geom;
     // every device pointer the captured passes read must be part of the key: a graph replays
     // only where those same addresses are allocated again (a lattice created anew at the same
-    // addresses holds the same data there); a missing one would replay freed memory
+    // addresses holds the same data there); a missing one would replay freed memory.  The tap table
+    // is copied into the captured launches: cutoff and decay fix it
     const std::vector<uint64_t> key = {
         (uint64_t)ctx->ws_phi[0].p, (uint64_t)ctx->ws_phi[1].p, (uint64_t)ctx->ws_phi2[0].p,
         (uint64_t)ctx->ws_phi2[1].p, (uint64_t)d_mu, (uint64_t)lat, (uint64_t)lat->d32, (uint64_t)lat->d64,
@@ -1481,8 +1477,7 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
         (uint64_t)M, (uint64_t)fmode, (uint64_t)pl.precision, (uint64_t)pl.Spad, bits(a.thop), bits(a.diag_const),
         (uint64_t)g.Lx, (uint64_t)g.Ly, (uint64_t)g.Lz, (uint64_t)g.kind,
         (uint64_t)(g.pbc_x | (g.pbc_y << 1) | (g.pbc_z << 2)), (uint64_t)lat->path, (uint64_t)pl.n,
-        (uint64_t)lat->chunks, (uint64_t)a.taps_rx, (uint64_t)a.taps_ry, (uint64_t)a.taps_n0, (uint64_t)a.taps_n1,
-        (uint64_t)a.taps_exact,
+        (uint64_t)(a.taps != nullptr), bits(lat->desc.cutoff), bits(lat->desc.decay),
         (uint64_t)lat->wrel32, (uint64_t)lat->wrel64};
     tbpm_ctx::Graph* hit = nullptr;
     for (auto& e : ctx->graphs)
@@ -2387,7 +2382,7 @@ int tbpm_moment_pass_kind(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_r
   tbpm_lattice* lat = const_cast<tbpm_lattice*>(lat_c);
   Plan pl;
   TBPM_TRY(make_plan(lat, req, &pl));
-  if (lat->chunks && pl.precision == TBPM_C64 && pl.Spad >= 2) {
+  if (lat->taps && pl.precision == TBPM_C64 && pl.Spad >= 2) {
     *kind = TBPM_PASS_TAPS;
     return TBPM_OK;
   }

@@ -14,6 +14,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -241,12 +242,16 @@ struct tbpm_ctx {
   std::vector<nvtxRangeId_t> nvtx_open;
 };
 
-// One piece of a column run of long-range taps for the matrix-free tap kernel: the taps
-// (dx, dy0 + k, ds), k < n (1 <= n <= 8), of one destination sublattice, with weights t_k/t
-// (0 where the run has a hole or the piece is padded).
-struct TapChunk {
-  int dx, dy0, ds, n;
-  float w[8];
+// Taps of a cell of two sites for the matrix-free tap kernel, a kernel argument: its uniform reads
+// come from the constant bank and cost the kernel no shared-memory cycles and no registers per lane.
+// Columns: (pack offset of the first row in the tile, steps, first weight); a step's weights are
+// (w0, w0, w1, w1), each twice as the packed FMA takes it.  The longest hopping, 12, has 466 steps
+// on the square lattice and 34 columns on the honeycomb.
+constexpr int kTapMaxSteps = 480, kTapMaxCols = 40;
+struct TapTable {
+  float4 w[kTapMaxSteps];
+  int4 col[kTapMaxCols];
+  int n_cols, rx, ry, unused;
 };
 
 struct tbpm_lattice {
@@ -271,12 +276,8 @@ struct tbpm_lattice {
   std::vector<int> tap_off;      // [z][4] (dx, dy, dz, ds) of each slot (long-range only)
   std::vector<double> tap_t;     // [z] t(r) of each slot (long-range only)
   double* jw = nullptr;          // [3 directions][2 sublattices][z] t_k (r_j - r_i)_a of each slot
-  // matrix-free tap kernel (clean long-range square / honeycomb lattices): column-run pieces
-  // of destination sublattice 0 then 1 on the device, their counts and the tile halo
-  TapChunk* chunks = nullptr;
-  int n_chunks[2] = {0, 0};
-  int halo_x = 0, halo_y = 0;
-  bool tap_exact = false;        // run pieces of every length 1..8 (else 8, 4, 2, 1)
+  // matrix-free tap kernel (clean long-range square / honeycomb lattices), host memory
+  std::unique_ptr<TapTable> taps;
   // vacancy lattices on the masked stencil: D_i by full site index, NaN at vacant sites (made on first use)
   float* dfull = nullptr;
   int64_t* compact = nullptr;  // [n_full] compact index or -1 (CSR path only)
@@ -323,9 +324,8 @@ struct RecurrenceArgs {
   int path;
   const int32_t* ell;  // CSR/ELL neighbour lists
   const void* wrel;    // per-slot weights t_k/t (float* or double*), or null (every bond t)
-  // matrix-free tap kernel (complex64, >= 2 states): chunk table, counts, halo, partial sums
-  const TapChunk* taps;
-  int taps_n0, taps_n1, taps_rx, taps_ry, taps_exact;
+  // matrix-free tap kernel (complex64, >= 2 states): tap table (host memory), partial sums
+  const TapTable* taps;
   double* tap_partials;
   const void* diag;    // per-site D_i (float* or double*), or null when the lattice is clean
   int masked;          // diag holds NaN at vacant sites (full layout of a vacancy lattice)
@@ -374,7 +374,7 @@ inline void set_float_coefficients(RecurrenceArgs* a) {
 int launch_moment_step(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, bool first);
 // matrix-free tap kernel (csrc/taps.cu): chunk table of a clean long-range lattice, the moment
 // pass over it, and the size of its per-CTA partial sums
-int build_tap_chunks(tbpm_ctx* ctx, tbpm_lattice* lat);
+int build_tap_table(tbpm_lattice* lat);
 int ensure_ell(tbpm_ctx* ctx, tbpm_lattice* lat);  // ELL lists of a long-range lattice, on first need
 int launch_taps_moment(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);
 int launch_taps_step(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first);  // recurrence only

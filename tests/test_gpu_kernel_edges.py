@@ -217,3 +217,32 @@ def test_cubic_march_matches_the_oracle(capi, ctx, name, L, kw, S, prec):
         assert np.max(np.abs(mu[s, :, 0] + 1j * mu[s, :, 1] - oprop.moments(ol, psi[s], psi[s], M))) <= tol
         assert np.max(np.abs(C[s] - oprop.correlation_sequential(ol, psi[s], Nt, np.pi))) <= tol
     capi.tbpm_lattice_destroy(lat)
+
+
+# The tap kernel: rows of an odd number of sites (cells of two), tiles cut by one and short by one, open and
+# wrapped halos, a lattice smaller than the halo, and the longest hopping there is.
+TAPS = [
+    ("odd_periodic", (129, 33), dict(kind=0, cutoff=3.3), 2),
+    ("odd_open_x", (127, 31), dict(kind=0, cutoff=2.1, pbc=(0, 1, 1)), 3),
+    ("one_column", (1, 40), dict(kind=0, cutoff=2.1), 2),
+    ("nearest_only_open", (5, 7), dict(kind=0, cutoff=1.0, pbc=(0, 0, 1)), 4),
+    ("honeycomb_cells", (65, 33), dict(kind=1, cutoff=5.1, pbc=(1, 0, 1)), 2),
+    ("honeycomb_images", (3, 2), dict(kind=1, cutoff=5.1), 2),
+    ("longest_square", (131, 37), dict(kind=0, cutoff=12.0), 2),
+    ("longest_honeycomb", (67, 30), dict(kind=1, cutoff=12.0), 3),
+]
+
+
+@pytest.mark.parametrize("name,L,kw,S", TAPS, ids=[c[0] for c in TAPS])
+def test_tap_kernel_matches_the_oracle(capi, ctx, name, L, kw, S):
+    kind, pbc, cutoff = kw["kind"], kw.get("pbc", (1, 1, 1)), kw["cutoff"]
+    lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(kind, L, t=1.0, W=0.5, seed=7, pbc=pbc, cutoff=cutoff,
+                                                          decay=0.6))
+    ol = olat.build_lattice(kind, L + (1,), t=1.0, W=0.5, seed=7, pbc=pbc, cutoff=cutoff, decay=0.6)
+    M = 18
+    mu = np.zeros((S, M, 2))
+    capi.tbpm_moments(ctx, lat, capi.request(n_states=S, n_moments=M, state_seed=3), mu)
+    psi = oprop.random_phase_states(ol, 3, S)
+    for s in {0, S - 1}:
+        assert np.max(np.abs(mu[s, :, 0] + 1j * mu[s, :, 1] - oprop.moments(ol, psi[s], psi[s], M))) <= 1e-5
+    capi.tbpm_lattice_destroy(lat)
