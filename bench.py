@@ -726,12 +726,12 @@ def state_based_bytes(passes, blocks, n_sites, S, elem, z, diag_bytes, n_steps, 
 
 
 def state_based_bytes_buffered(n_steps: int, b: int, tau: float, trunc, n_sites, S, elem, z, diag_bytes,
-                               T: int = 32, corr=True) -> float:
-    """Bytes moved by the buffered time blocks (b >= 2): per block the accumulators are cleared,
-    phi_0 copied into the buffer; every recurrence step reads phi_n, phi_{n-1} (not the first),
-    the ELL lists and D_i and writes phi_{n+1} into a slot; every window of <= T terms is read
-    once per 16 accumulators and each accumulator read and written once; two slots are carried
-    to the next window; <psi|acc_j> reads psi and the accumulators; the last state is copied."""
+                               T: int = 96, corr=True) -> float:
+    """Bytes moved by the buffered time blocks (b >= 2): every recurrence step reads phi_n, phi_{n-1}
+    (not the first), the ELL lists and D_i and writes phi_{n+1} into a slot; every window of <= T
+    terms is read once per 16 accumulators and each accumulator written once and, from the second
+    window on, read; two slots are carried to the next window; <psi|acc_j> reads psi and the
+    accumulators; the last state is copied."""
     st = float(n_sites) * S * elem
     total = 0.0
     start = 0
@@ -739,11 +739,10 @@ def state_based_bytes_buffered(n_steps: int, b: int, tau: float, trunc, n_sites,
         bb = min(b, n_steps - start)
         Nb = max(trunc((j + 1) * tau) for j in range(bb))
         tiles = (bb + 15) // 16
-        total += bb * st + 2 * st
         for n in range(1, Nb):
             total += (2 if n == 1 else 3) * st + 4.0 * z * n_sites + diag_bytes * n_sites
         windows = (Nb + T - 1) // T
-        total += Nb * st * tiles + windows * 2 * bb * st + (windows - 1) * 4 * st
+        total += Nb * st * tiles + (2 * windows - 1) * bb * st + (windows - 1) * 4 * st
         if corr:
             total += st * tiles + bb * st
         total += 2 * st
@@ -889,11 +888,12 @@ def run_state_based(args, work):
     value = whole_job_rate(c64["concurrent_s"]["site_updates_per_s"], world, 1.0)
     roofline = {"bound": "hbm", "achieved": c64["concurrent_s"]["algorithmic_gbs"], "peak": peak, "unit": "GB/s",
                 "frac": c64["concurrent_s"]["frac_of_hbm"], "traffic": None, "peak_source": peak_kind,
-                "kernel": ("k_ell_step (ELL recurrence into buffer slots) + k_block_flush_c64 (packed flush), complex64"
+                "kernel": ("k_ell_step (ELL recurrence into buffer slots) + k_flush, complex64"
                            if c64["concurrent_s"]["b"] >= 2 else "k_accum_step (ELL, complex64, time-block accumulation)"),
                 "bytes_model": ("buffered blocks: per step phi_n, phi_{n-1}, phi_{n+1}, 4z B ELL + D_i per site; per "
-                                "window of <= 32 terms each slot read once per 16 accumulators and each accumulator "
-                                "read and written once; per block clear, copies and one block inner product"
+                                "window of <= 96 terms each slot read once per 16 accumulators and each accumulator "
+                                "written once (read from the second window on); per block one copy and one block "
+                                "inner product"
                                 if c64["concurrent_s"]["b"] >= 2 else
                                 "per pass: phi_n, phi_{n-1}, phi_{n+1}, 4z B ELL + D_i per site, 8 or 16 B per "
                                 "open accumulator, psi once per time step, one copy per block")}

@@ -199,11 +199,11 @@ int tbpm_fusion_report(tbpm_ctx* ctx, double ms_per_step[16]);
  * (tbpm_profile) runs the passes without graphs.  enable = 0 drops the cached graphs. */
 int tbpm_set_graphs(tbpm_ctx* ctx, int enable);
 /* Buffered time blocks (default on): the state-based and sequential forms (Sec. II.B, Eq. TE)
- * keep the Chebyshev vectors phi_n of up to 32 consecutive terms in buffer slots and add
+ * keep the Chebyshev vectors phi_n of up to 96 consecutive terms in buffer slots and add
  * sum_n c_n(j tau~) phi_n to every open accumulator of the block in one pass, instead of one
  * accumulator update per term; C(t_j) = <psi|psi(t_j)> of the block then comes from one block
  * inner product.  The arithmetic is the same sum in another order (results agree to rounding).
- * The buffer takes up to 34 state blocks and shrinks with free memory; with fewer than 4 slots,
+ * The buffer takes up to 98 state blocks and shrinks with free memory; with fewer than 4 slots,
  * the sequential form (b = 1), or enable = 0, every term updates the accumulators in the
  * recurrence pass itself. */
 int tbpm_set_block_buffering(tbpm_ctx* ctx, int enable);
