@@ -2018,6 +2018,44 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
   return TBPM_OK;
 }
 
+// The overlaps O(E) = <psi|Psi(E)> that the conductivity divides by, in 64 bits where FP32 does not do.  Psi(E) in
+// complex64 gives O with an absolute error that does not shrink with O: the rounding of H~ and of C_n(E), 1e-8 to
+// 1e-7 of O's mean 1 / (2 |H|) over the window, and the recurrence's own, about 8e-9 of it on 1e5 sites and falling
+// as 1 / sqrt(N).  Next to the Dirac point of a sample with few vacancies O passes through zero between energies: at
+// |O| = 2e-4 of the mean (380 x 200 cells, W = 1.7, 127 steps) C(t, E) was 1.3e-4 off, now 6e-7.  The line lies
+// where the recurrence's share passes 1e-7 of O: a tenth of the mean at 2e5 sites, falling with 1 / sqrt(N) to 0.03
+// (the first two shares stay) and 0.5 for small samples and site states.  Below it, all overlaps of the request are
+// formed again from the complex128 moments of the same states, need / 2 steps in FP64: on 2.1M sites and 128 time
+// steps 26 ms beside the 16 ms of 9 energies.  Long-range lattices keep the complex64 overlaps (an FP64 step of 235
+// neighbours costs more than the request).
+int refine_overlaps(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, const double* d_E,
+                    int nE, double* nrm) {
+  if (pl.precision != TBPM_C64 || !lat->tap_t.empty()) return TBPM_OK;
+  std::vector<double> h(2 * (size_t)pl.S * nE);
+  TBPM_CK(cudaMemcpyAsync(h.data(), nrm, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, ctx->stream));
+  TBPM_CK(cudaStreamSynchronize(ctx->stream));
+  double least = INFINITY;
+  for (size_t k = 0; k < h.size(); k += 2) least = std::min(least, hypot(h[k], h[k + 1]));
+  const double n_eff = req->states == TBPM_STATES_SITES ? 1.0 : (double)lat->n_sites;
+  const double line = std::min(0.5, std::max(0.03, 0.1 * sqrt(2e5 / n_eff)));
+  if (!(least < line / (2.0 * lat->half))) return TBPM_OK;
+  tbpm_request r128 = *req;
+  r128.precision = TBPM_C128;
+  r128.form = TBPM_CONCURRENT_M;
+  r128.n_moments = 0;
+  Plan p128;
+  TBPM_TRY(make_plan(lat, &r128, &p128));
+  int r = ensure(ctx, ctx->ws_out, sizeof(double) * 2 * (size_t)p128.Spad * (req->n_steps + 1));
+  if (r == TBPM_OK) r = run_correlation(ctx, lat, &r128, p128, (double*)ctx->ws_out.p);
+  if (r == TBPM_ENOMEM) {  // no room for two complex128 blocks: the complex64 overlaps stay
+    clear_error();
+    return TBPM_OK;
+  }
+  TBPM_TRY(r);
+  return launch_ec_overlap(ctx, (const double*)ctx->ws_out.p, d_E, nE, pl.Spad * nE, (int)req->n_steps,
+                           pl.tau / lat->half, nrm);
+}
+
 // Electronic conductivity (Sec. V) along `direction` for all Spad states and nE energies.
 // Leaves C(t_j, E_k) in ws_out as [Spad][nE][n_steps+1][2] and sigma in ws_ec (after the
 // 2*Spad*nE norms) as [Spad][nE].  Returns the sigma pointer through *d_sigma.
@@ -2051,12 +2089,13 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
   double* sigma = nrm + 2 * (size_t)rows;
   TBPM_TRY(ensure(ctx, ctx->ws_psi, pl.state_bytes));
   TBPM_TRY(ensure(ctx, ctx->ws_jpsi, pl.state_bytes));
-  TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
-  TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
   TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_psi.p, nullptr));
   const int64_t n = pl.n;
   // <psi|Psi(E)> before the kets are overwritten
   TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, ctx->ws_psi.p, 1, ctx->ws_qe.p, nE, nrm, nE, 0, 1, 0));
+  TBPM_TRY(refine_overlaps(ctx, lat, req, pl, d_E, nE, nrm));
+  TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
+  TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
   // |psi_2(E)> = J |Psi(E)> in place (through one scratch block), |psi_1> = J |psi>
   for (int k = 0; k < nE; ++k) {
     char* qk = (char*)ctx->ws_qe.p + (size_t)k * pl.state_bytes;

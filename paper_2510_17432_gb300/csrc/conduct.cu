@@ -399,6 +399,26 @@ __global__ void __launch_bounds__(256) k_ec_finish(double* C, const double* nrm,
   if (threadIdx.x == 0) sigma[row] = mag > 0.0 ? nr / area * tphys * tot : 0.0;
 }
 
+// <psi|Psi(E_k)> = tau / 2 pi sum_{|j| <= n_steps} e^{i E_k t_j} C(t_j) with C(-t) = C(t)^*: one block per row s*nE + k.
+__global__ void __launch_bounds__(256) k_ec_overlap(const double* corr, const double* energies, int nE, int n_steps,
+                                                    double tphys, double* nrm) {
+  __shared__ double sh[8];
+  const int row = blockIdx.x, k = row % nE;
+  const double* c = corr + (int64_t)(row / nE) * (n_steps + 1) * 2;
+  const double E = energies[k];
+  double acc = 0.0;
+  for (int j = threadIdx.x; j <= n_steps; j += blockDim.x) {
+    double sn, cs;
+    sincos(E * (double)j * tphys, &sn, &cs);
+    acc += (j == 0 ? 1.0 : 2.0) * (cs * c[2 * j] - sn * c[2 * j + 1]);
+  }
+  const double tot = block_sum256(acc, sh);
+  if (threadIdx.x == 0) {
+    nrm[2 * row] = tphys / (2.0 * M_PI) * tot;
+    nrm[2 * row + 1] = 0.0;
+  }
+}
+
 int spt_for(int precision, int S) { return (precision == TBPM_C64 && S >= 2) ? 2 : 1; }
 
 template <typename R, int SPT, int TA, int TB>
@@ -551,6 +571,13 @@ int launch_ec_corr_from_moments(tbpm_ctx* ctx, const double* table, const int* n
                                 const double* m, int rows, int Nn, double shift, double tau, double* C) {
   k_ec_corr_m<<<dim3(n_steps + 1, (rows + kEcRows - 1) / kEcRows), 256, 0, ctx->stream>>>(
       table, n_per_step, n_steps, m, rows, Nn, shift, tau, C);
+  TBPM_CK_LAUNCH(ctx);
+  return TBPM_OK;
+}
+
+int launch_ec_overlap(tbpm_ctx* ctx, const double* corr, const double* energies, int nE, int rows, int n_steps,
+                      double tphys, double* nrm) {
+  k_ec_overlap<<<rows, 256, 0, ctx->stream>>>(corr, energies, nE, n_steps, tphys, nrm);
   TBPM_CK_LAUNCH(ctx);
   return TBPM_OK;
 }

@@ -449,6 +449,9 @@ int launch_partial_reduce(tbpm_ctx* ctx, const double* partials, int G, int nA, 
                           int64_t os, int64_t oa, int64_t ob, int64_t off);
 int launch_ec_corr_from_moments(tbpm_ctx* ctx, const double* table, const int* n_per_step, int n_steps,
                                 const double* m, int rows, int Nn, double shift, double tau, double* C);
+// <psi|Psi(E)> [rows = Spad * nE][2] from C(t_j) = <psi|psi(t_j)> [Spad][n_steps+1][2]
+int launch_ec_overlap(tbpm_ctx* ctx, const double* corr, const double* energies, int nE, int rows, int n_steps,
+                      double tphys, double* nrm);
 int launch_ec_finish(tbpm_ctx* ctx, double* C, const double* nrm, const double* energies, int nE, int rows,
                      int n_steps, double tphys, double area, double* sigma);
 // Fermi-Dirac filtered responses (csrc/response.cu)

@@ -126,3 +126,30 @@ def test_conductivity_rejects_bad_direction_and_form(capi, ctx):
     with pytest.raises(capi.TbpmError):
         capi.tbpm_conductivity(ctx, lat, capi.request(n_states=1, n_steps=4, form=3), 0, E, C, sigma)
     capi.tbpm_lattice_destroy(lat)
+
+
+@pytest.mark.parametrize("form", [2, 1, 0])
+@pytest.mark.parametrize("nE,S", [(9, 1), (1, 2)])
+def test_correlation_where_the_overlap_passes_near_zero(capi, ctx, nE, S, form):
+    """Weak disorder, no vacancies, an energy at H0: <psi|Psi(E)> there is a thousandth of its largest value and
+    below, and C is divided by it.  FP32 rounds H~ by at most 2 x 2^-25 of |H|, a phase of pi N_t 2^-24 = 2.4e-5
+    over the propagation, which bounds C's numerator; the overlap must add nothing to it."""
+    spec = dict(kind=1, L=(190, 100), t=-2.7, W=0.428, seed=1003)
+    lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(**spec))
+    ol = _oracle_lattice(spec)
+    w = 0.8 * ol.half_width
+    E = ol.H0 - w + 2 * w * (np.arange(nE) + 0.5) / nE
+    Nt = 127
+    C = np.zeros((S, nE, Nt + 1), np.complex128)
+    sigma = np.zeros((S, nE))
+    overlap = np.zeros((S, nE), np.complex128)
+    req = capi.request(n_states=S, form=form, n_steps=Nt, state_seed=1004)
+    capi.tbpm_conductivity_overlap(ctx, lat, req, 0, E, C, sigma, overlap)
+    psi = oprop.random_phase_states(ol, 1004, S)
+    for s in range(S):
+        Cref, qe = oec.ec_correlation_sequential(ol, psi[s], E, Nt, 0)
+        O = (qe @ psi[s].conj()).real
+        assert np.max(np.abs(overlap[s] - O) / np.abs(O)) <= 1e-9
+        for k in range(nE):
+            assert np.max(np.abs(C[s, k] - Cref[k])) <= 2.4e-5 * np.max(np.abs(Cref[k])), (s, k)
+    capi.tbpm_lattice_destroy(lat)
