@@ -1526,36 +1526,24 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
   return TBPM_OK;
 }
 
-// Coefficient table of one time block of bb steps: coef[n][j] = exp(-i shift (j+1) tau) c_n((j+1) tau),
-// zero once n >= N((j+1) tau).  n_per[j] = N((j+1) tau).  amp: the same as the flush takes them, real
-// amplitudes a_n((j+1) tau) [n][j] (c_n = a_n (-i)^n), then the factors exp(-i shift (j+1) tau) [j].
-void block_coefficients(double tau, double shift, int bb, std::vector<double>* coef, std::vector<int>* n_per,
+// Coefficient table of one time block of bb steps: coef[n][j] = c_n((j+1) tau), zero once n >= N((j+1) tau);
+// n_per[j] = N((j+1) tau).  amp: the real amplitudes a_n as the flush takes them, c_n = a_n (-i)^n.  The
+// factor exp(-i H0 t) of the whole propagation is left out of the states -- it multiplies what is formed from
+// them, in FP64 (k_turn_rows): rounded to FP32 in every block, its error was the same each time and added up.
+void block_coefficients(double tau, int bb, std::vector<double>* coef, std::vector<int>* n_per,
                         std::vector<double>* amp) {
   n_per->resize(bb);
   for (int j = 0; j < bb; ++j) (*n_per)[j] = (int)truncation_order_host((j + 1) * tau);
   const int nt = *std::max_element(n_per->begin(), n_per->end());
   coef->assign((size_t)nt * bb * 2, 0.0);
-  amp->assign((size_t)nt * bb + 2 * (size_t)bb, 0.0);
+  amp->assign((size_t)nt * bb, 0.0);
   std::vector<double> J(nt + 1);
   for (int j = 0; j < bb; ++j) {
-    const double x = (j + 1) * tau;
-    bessel_j_host(x, nt, J.data());
-    double ps, pc;
-    sincos(-shift * x, &ps, &pc);
-    (*amp)[(size_t)nt * bb + 2 * j] = pc;
-    (*amp)[(size_t)nt * bb + 2 * j + 1] = ps;
+    bessel_j_host((j + 1) * tau, nt, J.data());
     for (int n = 0; n < (*n_per)[j]; ++n) {
       const double a = n == 0 ? J[0] : 2.0 * J[n];
       (*amp)[(size_t)n * bb + j] = a;
-      double cr = 0, ci = 0;
-      switch (n & 3) {
-        case 0: cr = a; break;
-        case 1: ci = -a; break;
-        case 2: cr = -a; break;
-        default: ci = a; break;
-      }
-      (*coef)[((size_t)n * bb + j) * 2] = pc * cr - ps * ci;
-      (*coef)[((size_t)n * bb + j) * 2 + 1] = pc * ci + ps * cr;
+      (*coef)[((size_t)n * bb + j) * 2 + (n & 1)] = (n & 3) == 1 || (n & 3) == 2 ? -a : a;  // (-i)^n a
     }
   }
 }
@@ -1621,7 +1609,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
     for (const int k : {1, k_acc})
       pass.push_back([&, k]() -> int {
         return launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_blk.p, Tm, ctx->ws_acc.p, k,
-                            (const double*)ctx->ws_blk_coef.p, 1, true, true, nullptr, 16);
+                            (const double*)ctx->ws_blk_coef.p, 1, true, true, 16);
       });
   } else {
     TBPM_TRY(ensure(ctx, ctx->ws_table, sizeof(double) * 2 * (size_t)k_acc));
@@ -1683,8 +1671,8 @@ int choose_block(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
 }
 
 // State-based propagation in blocks of b steps; b = 1 is the sequential form.
-// d_C [Spad][n_steps+1][2].  The hook sees each finished time block: psi(t_{start+1}) ..
-// psi(t_{start+bb}) as bb consecutive state blocks.  init (device, optional) replaces the
+// d_C [Spad][n_steps+1][2].  The hook sees each finished time block: psi~(t_{start+1}) ..
+// psi~(t_{start+bb}) as bb consecutive state blocks, without the common factor: psi(t) = e^{-i H0 t} psi~(t).  init (device, optional) replaces the
 // request's initial states.
 using BlockHook = std::function<int(int64_t /*start*/, int /*bb*/, const void* /*first state block*/)>;
 
@@ -1760,15 +1748,17 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   memset(&g, 0, sizeof(g));
   TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
   const int C_len = (int)(n_steps + 1);
+  auto turn = [&]() -> int {  // C(t_j) = e^{-i H0 t_j} <psi|psi~(t_j)>
+    return corr ? launch_turn_rows(ctx, d_C, pl.Spad, C_len, -lat->H0 / lat->half * tau) : TBPM_OK;
+  };
   // C(0) = <psi|psi>
   if (corr) TBPM_TRY(launch_dot(ctx, g.r, pl.precision, ctx->ws_psi.p, ctx->ws_psi.p, d_C, C_len));
 
-  const double shift = lat->H0 / lat->half;
   std::vector<double> coef_full, coef_last, amp_full, amp_last;
   std::vector<int> nper_full, nper_last;
-  block_coefficients(tau, shift, (int)b, &coef_full, &nper_full, &amp_full);
+  block_coefficients(tau, (int)b, &coef_full, &nper_full, &amp_full);
   const int64_t last_len = n_steps % b;
-  if (last_len) block_coefficients(tau, shift, (int)last_len, &coef_last, &nper_last, &amp_last);
+  if (last_len) block_coefficients(tau, (int)last_len, &coef_last, &nper_last, &amp_last);
   const size_t tab_bytes = (coef_full.size() + coef_last.size()) * sizeof(double);
   TBPM_TRY(ensure(ctx, ctx->ws_table, tab_bytes));
   double* tab_full = (double*)ctx->ws_table.p;
@@ -1797,7 +1787,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
     T = window_slots(pl, *std::max_element(nper_full.begin(), nper_full.end()));
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
-    // amplitudes and phases, full block then last block
+    // amplitudes, full block then last block
     std::vector<double> cz = amp_full;
     cz.insert(cz.end(), amp_last.begin(), amp_last.end());
     TBPM_TRY(ensure(ctx, ctx->ws_blk_coef, cz.size() * sizeof(double)));
@@ -1812,14 +1802,13 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
       const std::vector<int>& nper = (bb == b) ? nper_full : nper_last;
       const double* amp = (const double*)ctx->ws_blk_coef.p + ((bb == b) ? 0 : amp_full.size());
       const int Nb = *std::max_element(nper.begin(), nper.end());
-      const double* phase = shift != 0.0 ? amp + (size_t)Nb * bb : nullptr;
       // the block starts from the last state of the one before
       const char* first = start == 0 ? (const char*)ctx->ws_phi[0].p
                                      : (const char*)ctx->ws_acc.p + (size_t)(b - 1) * pl.state_bytes;
       TBPM_CK(cudaMemcpyAsync(terms, first, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
       TBPM_TRY(walk_windows(ctx, lat, g.r, pl, slots, T, Nb, [&](int64_t n0, int nt) -> int {
         return launch_flush(ctx, pl.precision, pl.n * pl.Spad, terms, nt, ctx->ws_acc.p, bb, amp + (size_t)n0 * bb, 1,
-                            true, n0 == 0, n0 + nt == Nb ? phase : nullptr);
+                            true, n0 == 0);
       }));
       if (corr)
         TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, pl.n, ctx->ws_psi.p, 1, ctx->ws_acc.p, bb, d_C,
@@ -1827,7 +1816,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
       if (hook) TBPM_TRY(hook(start, bb, ctx->ws_acc.p));
       start += bb;
     }
-    return TBPM_OK;
+    return turn();
   }
 
   int64_t start = 0;
@@ -1865,7 +1854,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
     TBPM_CK(cudaMemcpyAsync(ctx->ws_phi[0].p, last, pl.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
     start += bb;
   }
-  return TBPM_OK;
+  return turn();
 }
 
 // Time blocks, quasi-eigenstates and the conductivity of a vacancy lattice take the full layout where
@@ -1947,7 +1936,7 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
       const int tok = phase_begin(ctx, 0);
       TBPM_TRY(walk_windows(ctx, lat, ra, pl, (char*)ctx->ws_acc.p, T, need, [&](int64_t n0, int nt) -> int {
         return launch_flush(ctx, pl.precision, pl.n * pl.Spad, terms, nt, ctx->ws_qe.p, nE, coef + 2 * (size_t)n0 * nE, 2,
-                            false, n0 == 0, nullptr);
+                            false, n0 == 0);
       }));
       phase_end(ctx, tok);
       return TBPM_OK;
@@ -1977,7 +1966,7 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
       g.r.prev_out = ctx->ws_phi[(n + 1) & 1].p;
       TBPM_TRY(launch_accum_step(ctx, g, pl.precision, mode));
       TBPM_TRY(launch_flush(ctx, pl.precision, pl.n * pl.Spad, ctx->ws_acc.p, 1, ctx->ws_qe.p, nE,
-                            coef + 2 * (size_t)n * nE, 2, false, n == 0, nullptr));
+                            coef + 2 * (size_t)n * nE, 2, false, n == 0));
     }
     phase_end(ctx, tok);
     return TBPM_OK;
@@ -1986,13 +1975,13 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     set_error("quasi-eigenstates: form must be SEQUENTIAL, CONCURRENT_S or CONCURRENT_E");
     return TBPM_EINVAL;
   }
-  // explicit states psi(+-t_j), each folded into the N_E accumulators with (tau/2pi) e^{+-i E t_j}
+  // explicit states psi~(+-t_j), each folded into the N_E accumulators with (tau/2pi) e^{+-i (E - H0) t_j}
   TBPM_TRY(ensure(ctx, ctx->ws_qe_coef, phase_bytes));
   double* phase = (double*)ctx->ws_qe_coef.p;
   {
     const int64_t tot = (int64_t)nE * (n_steps + 1);
     (void)tot;
-    TBPM_TRY(launch_qe_coefficients_phase_only(ctx, d_E, nE, tphys, (int)n_steps, phase));
+    TBPM_TRY(launch_qe_phases(ctx, d_E, nE, lat->H0, tphys, (int)n_steps, phase));
   }
   TBPM_CK(cudaMemsetAsync(ctx->ws_qe.p, 0, pl.state_bytes * (size_t)nE, ctx->stream));
   RecurrenceArgs ra;
@@ -2156,6 +2145,7 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     };
     TBPM_TRY(run_blocks(ctx, lat, req, pl, n_steps, b, nullptr, 0.0, hook, ctx->ws_jpsi.p, false));
     TBPM_TRY(launch_xdot(ctx, pl.precision, pl.Spad, n, ctx->ws_jpsi.p, 1, kets, nE, C, (int64_t)nE * W, 0, W, 0));
+    TBPM_TRY(launch_turn_rows(ctx, C, rows, W, lat->H0 / lat->half * pl.tau));
     phase_end(ctx, tok);
   }
   const double area = lat->desc.kind == TBPM_HONEYCOMB ? 3.0 * sqrt(3.0) / 4.0 : 1.0;
@@ -2224,8 +2214,7 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
     char* const terms = (char*)ctx->ws_blk.p + 2 * pc.state_bytes;
     TBPM_CK(cudaMemcpyAsync(terms, b0, pc.state_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
     TBPM_TRY(walk_windows(ctx, lat, g.r, pc, (char*)ctx->ws_blk.p, T, n_terms, [&](int64_t n0, int nt) -> int {
-      return launch_flush(ctx, pc.precision, pc.n * pc.Spad, terms, nt, out, 1, coef + 2 * (size_t)n0, 2, false, n0 == 0,
-                          nullptr);
+      return launch_flush(ctx, pc.precision, pc.n * pc.Spad, terms, nt, out, 1, coef + 2 * (size_t)n0, 2, false, n0 == 0);
     }));
     release_if_tight(ctx, ctx->ws_blk);  // the callers' next step sizes its blocks by the free memory
     return TBPM_OK;

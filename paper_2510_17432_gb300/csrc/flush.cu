@@ -1,11 +1,10 @@
 // Buffered accumulation (Sec. II.B time blocks, Sec. IV quasi-eigenstates, the Fermi-Dirac series):
 //     acc_e += sum_{t < T} a_t(e) r_t phi_t        (e < n_acc)
 // over T buffered Chebyshev vectors phi_t (consecutive state blocks) with real amplitudes a_t(e).
-// Every coefficient family of the method is real up to a power of -i common to all accumulators and a
-// phase per accumulator: c_n(j tau~) = e^{-i H0 t_j} a_n (-i)^n with a_n = (2 - delta_n0) J_n, so the
-// vector is turned by (-i)^n once per term (r_t: a swap and a sign of the amplitude), one real
-// multiply-add per component does the rest, and the phase is applied when the last window is written.
-// The coefficients C_n(E) of the quasi-eigenstates and a_n of the Fermi-Dirac series are real as they are.
+// Every coefficient family of the method is real up to a power of -i common to all accumulators:
+// c_n(j tau~) = a_n (-i)^n with a_n = (2 - delta_n0) J_n (the factor e^{-i H0 t_j} stays out of the states),
+// so the vector is turned by (-i)^n once per term (r_t: a swap and a sign of the amplitude) and one real
+// multiply-add per component does the rest.  The coefficients C_n(E) of the quasi-eigenstates and a_n of the Fermi-Dirac series are real as they are.
 //
 // All states take the same coefficients, so a state block is a flat array of complex numbers here.  A
 // thread holds the accumulators of one 16-byte unit (two complex64 or one complex128 number) in
@@ -42,7 +41,6 @@ struct FlushArgs {
   const double* amp;   // amplitude of term t and accumulator e at amp[(t * nb + e) * as]
   int as;
   int init;            // 1: the window starts the sums (nothing is read from acc)
-  const double* phase; // [nb] complex factors applied to the finished sums, or null
   int64_t n_units;
 };
 
@@ -139,15 +137,6 @@ __global__ void __launch_bounds__(kThreads, EB >= 16 ? 2 : 3) k_flush(FlushArgs 
 #pragma unroll
     for (int e = 0; e < EB; ++e) {
       if (e < ne) {
-        if (f.phase) {
-          const R pr = (R)__ldg(f.phase + 2 * (e0 + e)), pi = (R)__ldg(f.phase + 2 * (e0 + e) + 1);
-#pragma unroll
-          for (int k = 0; k < C; ++k) {
-            const V2 s = ac[e][k];
-            ac[e][k].x = pr * s.x - pi * s.y;
-            ac[e][k].y = pr * s.y + pi * s.x;
-          }
-        }
         __stcs(Q + (int64_t)(e0 + e) * f.stride + u, join(ac[e]));
       }
     }
@@ -165,7 +154,7 @@ void launch_flush(const FlushArgs& f, bool rot, dim3 grid, cudaStream_t st) {
 int flush_max_terms() { return kFlushT; }
 
 int launch_flush(tbpm_ctx* ctx, int precision, int64_t n_numbers, const void* phi, int T, void* acc, int nb,
-                 const double* amp, int amp_stride, bool rot, bool init, const double* phase, int tile) {
+                 const double* amp, int amp_stride, bool rot, bool init, int tile) {
   if (T < 1 || T > kFlushT || nb < 1) {
     set_error("flush of %d terms into %d accumulators", T, nb);
     return TBPM_EINVAL;
@@ -178,7 +167,6 @@ int launch_flush(tbpm_ctx* ctx, int precision, int64_t n_numbers, const void* ph
   f.amp = amp;
   f.as = amp_stride;
   f.init = init ? 1 : 0;
-  f.phase = phase;
   // two complex64 numbers per unit where every block holds an even number of them (blocks are then
   // 16-byte aligned); an odd number only comes from one state on an odd number of sites
   const bool wide = precision == TBPM_C64 && n_numbers % 2 == 0;

@@ -299,6 +299,25 @@ __global__ void k_qe_phase(const double* energies, int nE, double H0, double tph
   }
 }
 
+// c[row][j] *= exp(i angle j): the common phase of a propagation, on what was formed from its states.
+__global__ void k_turn_rows(double* c, int64_t total, int64_t width, double angle) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    double sn, cs;
+    sincos(angle * (double)(e % width), &sn, &cs);
+    const double re = c[2 * e], im = c[2 * e + 1];
+    c[2 * e] = cs * re - sn * im;
+    c[2 * e + 1] = cs * im + sn * re;
+  }
+}
+
+int launch_turn_rows(tbpm_ctx* ctx, double* c, int64_t rows, int64_t width, double angle) {
+  if (angle == 0.0) return TBPM_OK;
+  k_turn_rows<<<(int)std::min<int64_t>((rows * width + 255) / 256, 4096), 256, 0, ctx->stream>>>(c, rows * width, width,
+                                                                                                 angle);
+  TBPM_CK_LAUNCH(ctx);
+  return TBPM_OK;
+}
+
 // One block per (n, group of 8 energies); threads over j.  coef[(n*nE + k)*2] = C_n(E_k), imag 0.
 __global__ void __launch_bounds__(256) k_qe_coeffs(const double* table, int n_steps, const double* phase, int nE,
                                                    double scale, double* coef) {
@@ -335,11 +354,11 @@ __global__ void __launch_bounds__(256) k_qe_coeffs(const double* table, int n_st
   }
 }
 
-// (cos, sin)(E_k t_j) without the H0 shift: the phases of explicitly propagated states.
-int launch_qe_coefficients_phase_only(tbpm_ctx* ctx, const double* energies, int nE, double tphys, int n_steps,
-                                      double* phase) {
+// (cos, sin)((E_k - H0) t_j): the phases of explicitly propagated states.
+int launch_qe_phases(tbpm_ctx* ctx, const double* energies, int nE, double H0, double tphys, int n_steps,
+                     double* phase) {
   const int64_t tot = (int64_t)nE * (n_steps + 1);
-  k_qe_phase<<<(int)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, ctx->stream>>>(energies, nE, 0.0, tphys,
+  k_qe_phase<<<(int)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, ctx->stream>>>(energies, nE, H0, tphys,
                                                                                       n_steps, phase);
   TBPM_CK_LAUNCH(ctx);
   return TBPM_OK;
@@ -347,10 +366,7 @@ int launch_qe_coefficients_phase_only(tbpm_ctx* ctx, const double* energies, int
 
 int launch_qe_coefficients(tbpm_ctx* ctx, const double* table, int n_steps, int n_terms, const double* energies,
                            int nE, double H0, double tphys, double* phase, double* coef) {
-  const int64_t tot = (int64_t)nE * (n_steps + 1);
-  k_qe_phase<<<(int)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, ctx->stream>>>(energies, nE, H0, tphys,
-                                                                                      n_steps, phase);
-  TBPM_CK_LAUNCH(ctx);
+  TBPM_TRY(launch_qe_phases(ctx, energies, nE, H0, tphys, n_steps, phase));
   k_qe_coeffs<<<dim3(n_terms, (nE + 7) / 8), 256, 0, ctx->stream>>>(table, n_steps, phase, nE,
                                                                      tphys / (2.0 * M_PI), coef);
   TBPM_CK_LAUNCH(ctx);

@@ -385,11 +385,11 @@ int launch_cubic_march(tbpm_ctx* ctx, const RecurrenceArgs& ra, int precision, b
 // acc_e (+)= sum_{t<T} a_t(e) [(-i)^t] phi_t over T consecutive buffered state blocks of n_numbers complex
 // numbers and nb consecutive accumulators (csrc/flush.cu): real amplitudes a_t(e) at
 // amp[(t * nb + e) * amp_stride]; rot: with the powers of -i (the window starts at a multiple of four terms);
-// init: the sums start here; phase: [nb] complex factors on the finished sums, or null.
+// init: the sums start here.
 // tile: accumulators per CTA tile (1, 4 or 16); 0 = chosen from nb
 int flush_max_terms();
 int launch_flush(tbpm_ctx* ctx, int precision, int64_t n_numbers, const void* phi, int T, void* acc, int nb,
-                 const double* amp, int amp_stride, bool rot, bool init, const double* phase, int tile = 0);
+                 const double* amp, int amp_stride, bool rot, bool init, int tile = 0);
 int launch_dot(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const void* x, const void* y,
                double* out /* device [S][2] at stride out_stride */, int out_stride);
 int recurrence_blocks(tbpm_ctx* ctx, int precision, int S);
@@ -397,8 +397,9 @@ int launch_qe_axpy(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, const 
                    const double* phase, int width, int j, double sgn, double scale, int nE);
 int launch_qe_coefficients(tbpm_ctx* ctx, const double* table, int n_steps, int n_terms, const double* energies,
                            int nE, double H0, double tphys, double* phase, double* coef);
-int launch_qe_coefficients_phase_only(tbpm_ctx* ctx, const double* energies, int nE, double tphys, int n_steps,
-                                      double* phase);
+int launch_qe_phases(tbpm_ctx* ctx, const double* energies, int nE, double H0, double tphys, int n_steps,
+                     double* phase);
+int launch_turn_rows(tbpm_ctx* ctx, double* c, int64_t rows, int64_t width, double angle);
 
 // temporal fusion (csrc/fused.cu)
 bool fused_applicable(const tbpm_lattice* lat, int precision, int Spad);

@@ -132,3 +132,21 @@ def test_fermi_operator_through_window_passes(capi, ctx, sqrt_f):
         ref = R.fermi_operator_exact(ol, psi[s], mu, kT, power=0.5 if sqrt_f else 1.0)
         assert np.max(np.abs(out[s] - ref)) / np.max(np.abs(ref)) <= 3e-5, s
     capi.tbpm_lattice_destroy(lat)
+
+
+def test_phase_of_a_block_is_not_rounded_into_the_next(capi, ctx):
+    """Nearly isolated sites (t = 0.002 W), whose C(t) keeps |C| = 1, over 400 blocks of one step.  exp(-i H0 tau) of
+    this lattice and time step is 2.8e-8 from its FP32 value, the amplitudes at these two sites 6e-10: with the
+    phase in the states the error grew to 400 x 2.8e-8 = 1.1e-5; the bound is half an ulp of 1 a step and lane."""
+    ol = olat.build_lattice(1, (64, 40, 1), t=0.002, W=1.0, seed=5)
+    lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(1, (64, 40), t=0.002, W=1.0, seed=5))
+    sites = np.array([2353, 1371, 0, 1], np.int64)
+    Nt, tau = 400, 3.69
+    C = np.zeros((4, Nt + 1), np.complex128)
+    capi.tbpm_correlation(ctx, lat, capi.request(n_states=4, sites=sites, form=0, n_steps=Nt, tau=tau), C)
+    for s in (0, 1):
+        e = np.zeros(ol.n, np.complex128)
+        e[sites[s]] = 1.0
+        ref = oprop.correlation_sequential(ol, e, Nt, tau)
+        assert np.max(np.abs(C[s] - ref)) <= 400 * 2.0**-26, s
+    capi.tbpm_lattice_destroy(lat)
