@@ -1392,7 +1392,8 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     TBPM_TRY(ensure_dfull(lat));
   }
   const int band = (fmode == 9 ? 192 : fmode == 10 ? 256 : 128) / std::max(1, pl.Spad / 2);
-  const bool wide_ok = fmode == 8 || lat->geom.kind != TBPM_HONEYCOMB || pl.Spad < 2 || lat->geom.Lx >= band;
+  // the masked, square and one-state sweeps have 128 threads in every mode
+  const bool wide_ok = pl.full || fmode == 8 || lat->geom.kind != TBPM_HONEYCOMB || pl.Spad < 2 || lat->geom.Lx >= band;
   const bool sweep = fmode >= 8 && steps - 1 >= K && wide_ok && sweep_ok(lat, pl);
   const bool fuse = !sweep && fmode > 0 && fused_applicable(lat, pl.precision, pl.Spad) && steps - 1 >= K;
   TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));

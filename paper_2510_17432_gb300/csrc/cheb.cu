@@ -903,6 +903,10 @@ static int launch_ell(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, boo
 int launch_moment_step(tbpm_ctx* ctx, const RecurrenceArgs& a, int precision, bool first) {
   const bool csr = a.path == TBPM_PATH_CSR;
   const int spt = spt_of(precision, a.S);
+  if (a.masked) {  // only the sweep's moment pass and the accumulation pass mask vacant sites
+    set_error("one-step moment pass on a masked state block");
+    return TBPM_EUNSUPPORTED;
+  }
   if (a.taps && precision == TBPM_C64 && spt == 2) return launch_taps_moment(ctx, a, first);
   if (ell_batched(a)) return launch_ell<true>(ctx, a, precision, first);
   if (!csr && a.geom.kind == TBPM_CUBIC) {

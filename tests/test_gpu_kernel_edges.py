@@ -100,6 +100,28 @@ def test_sweep_shapes_match_the_one_step_pass_and_the_oracle(capi, ctx, name, sp
     capi.tbpm_lattice_destroy(lat)
 
 
+# Vacancy honeycombs narrower than the bands of modes 9 and 10 (192 / P and 256 / P cells) and not than the
+# masked sweep's own (128 / P): the masked sweep has 128 threads in every mode.
+NARROW = [
+    ("S2_below_192", dict(kind=1, L=(190, 33), t=-2.7, W=1.0, vac=0.01), 2),
+    ("S2_below_256", dict(kind=1, L=(200, 40), t=-2.7, W=0.0, vac=0.05), 2),
+    ("S4_one_band", dict(kind=1, L=(64, 37), t=-2.7, W=0.5, vac=0.1, pbc=(1, 0, 1)), 4),
+    ("S8_between", dict(kind=1, L=(50, 32), t=1.0, W=0.0, vac=0.02, pbc=(0, 1, 1)), 8),
+]
+
+
+@pytest.mark.parametrize("mode", [8, 9, 10])
+@pytest.mark.parametrize("name,spec,S", NARROW, ids=[c[0] for c in NARROW])
+def test_wide_modes_on_narrow_vacancy_lattices(capi, ctx, name, spec, S, mode):
+    lat, ol = _pair(capi, ctx, spec)
+    M = 42
+    got = _moments(capi, ctx, lat, S, M, mode)
+    psi = oprop.random_phase_states(ol, 3, S)
+    for s in {0, S - 1}:
+        assert np.max(np.abs(got[s] - oprop.moments(ol, psi[s], psi[s], M))) <= 1e-5
+    capi.tbpm_lattice_destroy(lat)
+
+
 WINDOWS = [
     ("square", dict(kind=0, L=(129, 97), t=1.0, W=1.0, pbc=(1, 0, 1)), 4),
     ("square_S1", dict(kind=0, L=(256, 96), t=1.0, W=1.0), 1),
