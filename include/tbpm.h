@@ -158,8 +158,8 @@ const char* tbpm_last_error(void);
 /* The context's cudaStream_t, returned as void*, for event timing by the caller. */
 void* tbpm_stream(tbpm_ctx* ctx);
 /* Block until all work enqueued on the context's stream has finished.  Returns TBPM_ETIMEOUT
- * (once) when a bounded device wait of a fused moment pass expired since the last check; the
- * synchronous tbpm_moments and tbpm_dos report it the same way. */
+ * (once) when a bounded device wait of a sweep or resident pass expired since the last check; every
+ * synchronous compute call reports it the same way, and its results are then void. */
 int tbpm_sync(tbpm_ctx* ctx);
 /* Number of kernels the library has launched on this context since creation. */
 int64_t tbpm_launch_count(const tbpm_ctx* ctx);

@@ -2511,7 +2511,7 @@ int tbpm_correlation(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_reques
   TBPM_TRY(run_correlation(ctx, lat, req, pl, (double*)ctx->ws_out.p));
   TBPM_TRY(copy_rows(ctx, C, (double*)ctx->ws_out.p, pl.S, row, cudaMemcpyDeviceToHost));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
-  return TBPM_OK;
+  return sweep_status(ctx);
 }
 
 int tbpm_dos_device(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, const double* d_E,
@@ -2618,7 +2618,7 @@ int tbpm_block_autotune(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
     times_ms[0] = ta;
     times_ms[1] = tx;
   }
-  return TBPM_OK;
+  return sweep_status(ctx);  // the timed passes have ended
 }
 
 int tbpm_quasi_eigenstates(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, const double* energies,
@@ -2657,7 +2657,7 @@ int tbpm_quasi_eigenstates(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_
                                 pl.Spad * pl.elem, pl.elem, n, cudaMemcpyDeviceToHost, ctx->stream));
   }
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
-  return TBPM_OK;
+  return sweep_status(ctx);
 }
 
 int tbpm_conductivity(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, int direction,
@@ -2692,7 +2692,7 @@ int tbpm_conductivity_overlap(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tb
   if (overlap)
     TBPM_CK(cudaMemcpyAsync(overlap, ctx->ws_ec.p, sizeof(double) * 2 * rows, cudaMemcpyDeviceToHost, ctx->stream));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
-  return TBPM_OK;
+  return sweep_status(ctx);
 }
 
 int tbpm_fermi_apply(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, double mu, double kT,
@@ -2721,7 +2721,7 @@ int tbpm_fermi_apply(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_reques
                               (const char*)ctx->ws_phi2[0].p + s * pl.elem, pl.Spad * pl.elem, pl.elem, n,
                               cudaMemcpyDeviceToHost, ctx->stream));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
-  return TBPM_OK;
+  return sweep_status(ctx);
 }
 
 namespace {
@@ -2799,7 +2799,7 @@ int tbpm_optical_conductivity(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tb
     TBPM_CK(cudaMemcpyAsync(sigma + 2 * (size_t)pk.s0 * n_omega, d_sig, sizeof(double) * 2 * (size_t)pk.S * n_omega,
                             cudaMemcpyDeviceToHost, ctx->stream));
     TBPM_CK(cudaStreamSynchronize(ctx->stream));
-    return TBPM_OK;
+    return sweep_status(ctx);
   });
 }
 
@@ -2832,7 +2832,7 @@ int tbpm_polarization(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_reque
     TBPM_CK(cudaMemcpyAsync(Pi + 2 * (size_t)pk.s0 * n_omega, d_pi, sizeof(double) * 2 * (size_t)pk.S * n_omega,
                             cudaMemcpyDeviceToHost, ctx->stream));
     TBPM_CK(cudaStreamSynchronize(ctx->stream));
-    return TBPM_OK;
+    return sweep_status(ctx);
   });
 }
 
@@ -2899,7 +2899,7 @@ int tbpm_charge_density(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
     TBPM_CK(cudaMemcpyAsync(rho + (size_t)pl.s0 * n, ctx->ws_out.p, sizeof(double) * (size_t)n * pl.S,
                             cudaMemcpyDeviceToHost, ctx->stream));
     TBPM_CK(cudaStreamSynchronize(ctx->stream));
-    return TBPM_OK;
+    return sweep_status(ctx);
   });
 }
 

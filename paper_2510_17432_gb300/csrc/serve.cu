@@ -707,6 +707,10 @@ static void scheduler(tbpm_server* srv) {
             j->result = TBPM_ETIMEOUT;
             j->message = "tensor-core reconstruction: bounded wait expired";
           }
+          if (sweep_status(j->lane_ctx) != TBPM_OK) {  // the lane's moment passes
+            j->result = TBPM_ETIMEOUT;
+            j->message = tbpm_last_error();
+          }
           j->status = JOB_DONE;
           srv->completed++;
         }
