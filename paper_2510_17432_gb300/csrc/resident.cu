@@ -11,15 +11,16 @@
 // after them took 2.7 us per step on 64 x 64 complex128 sites, packets take 2.0).  A buffer is safe to reuse: the thread that
 // overwrites its packet of phi_n with phi_{n+2} has read the phi_{n+1} of every thread that reads the packet
 // (neighbours are mutual), and those were formed from phi_n.  Tags are never used twice (a counter in the
-// context).  All CTAs are resident (cooperative launch), so every wait ends; each is bounded all the same,
-// and one that expires is reported through the status word.
+// context).  All CTAs are resident (cooperative launch), so every wait ends; each is bounded all the same.  A
+// thread whose wait expired waits no more, its CTA ends with the step, the CTAs that wait for it follow within
+// their own two seconds, and the status word reports it.
 //
 // Moments: <phi_n|phi_n> and Re <phi_{n+1}|phi_n> (real for a Hermitian H~), summed per thread (at most 32
-// units in FP32 at a time), reduce-scattered over the lanes of a state pair -- FP32 values as compensated
+// units), reduce-scattered over the lanes of a state pair -- FP32 values as compensated
 // pairs, so no precision is lost in the tree -- and added in FP64 over the warps in a fixed order; the
 // per-CTA sums of every step are added in CTA order by a second kernel.  Deterministic.
 //
-// Bound: the exchange latency per step (flag, fence, L2 round trip) for small lattices; shared-memory
+// Bound: the exchange latency per step (a packet's way through L2 to the polling thread) for small lattices; shared-memory
 // bandwidth (complex64) or FP64 issue (complex128) when the blocks are large.  Measured, us per step, one
 // launch per step -> resident: 64 x 64 square, complex128, one state 6.6 -> 2.1; 45 x 47 honeycomb, 4 states
 // 8.1 -> 2.0; 40^3 cubic, 8 states 23.8 -> 7.5; 300 x 300 honeycomb, 8 states 25.8 -> 8.8.
@@ -38,6 +39,8 @@ namespace {
 constexpr int kResThreads = 512;     // at most; fewer where a CTA owns fewer units
 constexpr int kResBatch = 8;         // steps whose warp sums are added and stored together
 constexpr int kResMaxCtas = 256;
+constexpr int kResMaxUnits = 32;     // units of a thread, summed in FP32
+constexpr uint64_t kResWaitNs = 2000000000ull;  // 2 s per packet
 
 struct ResArgs {
   Geom g;
@@ -78,9 +81,9 @@ __device__ __forceinline__ void publish(ulonglong2* p, const Pack<R, SPT>& v, un
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p + k), "l"(t | w[2 * k]), "l"(t | w[2 * k + 1])
                  : "memory");
 }
-// The unit once it carries the tag; false when two seconds pass without it.
+// The unit once it carries the tag; false when budget_ns pass without it.
 template <typename R, int SPT>
-__device__ __forceinline__ bool receive(const ulonglong2* p, unsigned tag, Pack<R, SPT>& v) {
+__device__ __forceinline__ bool receive(const ulonglong2* p, unsigned tag, uint64_t budget_ns, Pack<R, SPT>& v) {
   constexpr int N = Packets<R, SPT>::N;
   uint64_t q[2 * N], t0 = 0;
   for (int spin = 0;; ++spin) {
@@ -94,7 +97,7 @@ __device__ __forceinline__ bool receive(const ulonglong2* p, unsigned tag, Pack<
     if ((spin & 255) == 255) {
       const uint64_t t = now_ns();
       if (t0 == 0) t0 = t;
-      else if (t - t0 > 2000000000ull) return false;
+      else if (t - t0 > budget_ns) return false;
     }
   }
   unsigned w[2 * N];
@@ -102,6 +105,15 @@ __device__ __forceinline__ bool receive(const ulonglong2* p, unsigned tag, Pack<
   for (int k = 0; k < 2 * N; ++k) w[k] = (unsigned)q[k];
   memcpy(&v, w, sizeof(v));
   return true;
+}
+
+// The same for a thread that has many to wait for: zero once one of its waits has expired (failed).
+template <typename R, int SPT>
+__device__ __forceinline__ Pack<R, SPT> receive_or_zero(const ulonglong2* p, unsigned tag, uint64_t budget_ns,
+                                                        bool& failed) {
+  Pack<R, SPT> v{};
+  if (!failed) failed = !receive<R, SPT>(p, tag, budget_ns, v);
+  return v;
 }
 
 // Neighbour lines of a line, in the neighbour order of the stencil: y + 1, y - 1, z + 1, z - 1 (-1: none).
@@ -177,13 +189,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
     ulonglong2* pr_out = a.packets + (((n + 1) & 1) * a.n_units + l0 * upr) * NP;
     const unsigned tag = a.tag + (unsigned)n;
     R s[NV];
-    double sd[NV];  // complex64: sums of 32 units folded in FP64
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      s[k] = R(0);
-      sd[k] = 0.0;
-    }
-    int cnt = 0;
+    for (int k = 0; k < NV; ++k) s[k] = R(0);
 #pragma unroll 2
     for (int u = tid; u < nu; u += NT) {
       const int li = (int)(((uint64_t)(uint32_t)u * a.magic) >> 32);
@@ -201,10 +208,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
         if (t >= 0) take(cur[(int)t + off]);
         else if (t != -1) {
           const int64_t r = -(t + 2) + off;
-          PK v;
-          if (first) v = reinterpret_cast<const PK*>(a.x0)[r];
-          else failed |= !receive<R, SPT>(pr_in + r * NP, tag, v);
-          take(v);
+          if (first) take(reinterpret_cast<const PK*>(a.x0)[r]);
+          else take(receive_or_zero<R, SPT>(pr_in + r * NP, tag, kResWaitNs, failed));
         }
       };
 #pragma unroll
@@ -252,14 +257,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
         s[2 * k] = fma(pr, pr, fma(pi, pi, s[2 * k]));
         s[2 * k + 1] = fma(o.v[2 * k], pr, fma(o.v[2 * k + 1], pi, s[2 * k + 1]));
       }
-      if (sizeof(R) == 4 && ++cnt == 32) {
-        cnt = 0;
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          sd[k] += (double)s[k];
-          s[k] = R(0);
-        }
-      }
     }
     if (__syncthreads_or(failed ? 1 : 0)) {
       if (tid == 0) atomicExch(a.status, 3);
@@ -270,15 +267,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
       using SumT = decltype(sum_of(R(0)));
       SumT v[NV];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        v[k] = sum_of(s[k]);
-        if constexpr (sizeof(R) == 4) {
-          if (nu > 32 * NT) {
-            const float hi = (float)sd[k];
-            v[k] = add(v[k], Pair32{hi, (float)(sd[k] - (double)hi)});
-          }
-        }
-      }
+      for (int k = 0; k < NV; ++k) v[k] = sum_of(s[k]);
       double* slot = red + ((size_t)(n & (kResBatch - 1)) * warps + warp) * P * NV + (lane & (P - 1)) * NV;
       reduce_lanes<NV>(v, P, logP, lane, [&](int k, double t) { slot[k] = t; });
     }
@@ -338,8 +327,9 @@ bool plan_resident(tbpm_ctx* ctx, const Geom& g, int precision, int Spad, bool d
   const size_t unit = precision == TBPM_C64 ? 8 * (size_t)spt : 16, real = precision == TBPM_C64 ? 4 : 8;
   const int64_t upr = g.row_sites * P, most = std::min(ctx->num_sms, kResMaxCtas);
   const int64_t lines = (g.n_rows + most - 1) / most;
-  // beyond what fits in any case (and the range of the division by multiplication)
-  if (lines * upr > 32768 || upr < 2) return false;
+  // a thread's share of FP32 sums (220 KB hold at most 28 units a thread), within the range of the division
+  // by multiplication
+  if (lines * upr > kResMaxUnits * kResThreads || upr < 2) return false;
   const size_t cap = (size_t)(lines * upr);
   r->lines = (int)lines;
   r->ctas = (int)((g.n_rows + lines - 1) / lines);

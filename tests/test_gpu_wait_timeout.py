@@ -63,3 +63,27 @@ def test_expired_wait_is_reported_and_the_context_stays_usable(capi):
         capi.tbpm_lattice_destroy(lat)
     finally:
         capi.tbpm_destroy(ctx)
+
+
+@pytest.mark.gpu
+def test_a_thread_with_many_remote_units_waits_once(capi, tmp_path):
+    """The resident recurrence's packet wait in a one-warp kernel on a zeroed buffer: 40 units that nobody publishes
+    cost each thread one budget of 0.1 s, not 40."""
+    import os
+    import shutil
+    import subprocess
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    pkg = os.path.join(root, "paper_2510_17432_gb300")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    out = str(tmp_path / "libpacket_wait.so")
+    subprocess.run([nvcc, "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-I", os.path.join(root, "include"), "-I", os.path.join(pkg, "csrc"), "-o", out,
+                    os.path.join(root, "tests", "packet_wait.cu"), "-L", pkg, "-ltbpm", "-Xlinker", "-rpath," + pkg],
+                   check=True, capture_output=True)
+    lib = C.CDLL(out)
+    lib.packet_wait.argtypes = [C.c_int, C.c_double]
+    assert lib.packet_wait(1, 0.001) == 32  # module loaded, context up
+    t0 = time.perf_counter()
+    assert lib.packet_wait(40, 0.1) == 32
+    dt = time.perf_counter() - t0
+    assert 0.08 <= dt < 1.0, dt
