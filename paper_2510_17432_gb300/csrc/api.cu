@@ -1379,9 +1379,10 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     a.mu = d_mu;
     a.M = (int)M;
     const int tok = phase_begin(ctx, 0);
-    TBPM_TRY(launch_resident(ctx, lat, a, pl.precision, ctx->ws_phi[0].p, M / 2));
+    const int r = launch_resident(ctx, lat, a, pl.precision, ctx->ws_phi[0].p, M / 2);
     phase_end(ctx, tok);
-    return TBPM_OK;
+    if (r != TBPM_EUNSUPPORTED) return r;
+    clear_error();
   }
   int fmode = 0;
   TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));

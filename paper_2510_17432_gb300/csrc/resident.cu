@@ -351,7 +351,8 @@ bool resident_applicable(tbpm_ctx* ctx, const tbpm_lattice* lat, int precision, 
   return (size_t)steps * 2 * Spad * r.ctas * sizeof(double) <= (512u << 20);  // per-CTA sums of every step
 }
 
-// All `steps` steps from phi_0 in x0.
+// All `steps` steps from phi_0 in x0.  TBPM_EUNSUPPORTED where the grid cannot be resident as a whole (fewer SMs
+// for this process than the device has, no cooperative launches): the caller takes another pass.
 int launch_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs& ra, int precision, const void* x0,
                     int64_t steps) {
   ResPlan r;
@@ -397,7 +398,13 @@ int launch_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs
   a.partials = (double*)ctx->ws_fused_partials.p;
   a.status = reinterpret_cast<int*>(ctx->pinned + kSweepStatusSlot);
   void* args[] = {&a};
-  TBPM_CK(cudaLaunchCooperativeKernel(fn, dim3(r.ctas), dim3(r.threads), args, r.smem, ctx->stream));
+  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(r.ctas), dim3(r.threads), args, r.smem, ctx->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    set_error("resident recurrence: %s", cudaGetErrorString(e));
+    return TBPM_EUNSUPPORTED;
+  }
+  TBPM_CK(e);
   ctx->launches++;
   k_resident_moments<<<(unsigned)steps, 256, 0, ctx->stream>>>(a.partials, r.ctas, ra.S, ra.mu, ra.M);
   TBPM_CK_LAUNCH(ctx);

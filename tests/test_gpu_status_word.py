@@ -3,7 +3,7 @@
 The register sweep, its window passes and the resident recurrence record an expired wait in the
 context's status word and return; results formed after that are void.  Here the word is written
 from the host (no wait expires on the device): each call must return TBPM_ETIMEOUT once, and the
-same call made again must succeed."""
+same call made again must succeed.  A cooperative launch that the driver refuses is no failure either."""
 import ctypes as C
 import os
 import shutil
@@ -33,7 +33,8 @@ def poke(tmp_path_factory):
                     "-o", out, os.path.join(ROOT, "tests", "status_word.cu")], check=True, capture_output=True)
     lib = C.CDLL(out)
     lib.set_status_word.argtypes = [C.c_void_p, C.c_int]
-    return lib.set_status_word
+    lib.set_num_sms.argtypes = [C.c_void_p, C.c_int]
+    return lib
 
 
 S, NT, NE = 2, 4, 3
@@ -70,11 +71,11 @@ def test_synchronous_calls_report_an_expired_wait_once(capi, poke):
         missed = []
         for name, call in _calls(capi, ctx, lat, capi.tbpm_lattice_info(lat).n_sites).items():
             call()
-            poke(ctx, 1)
+            poke.set_status_word(ctx, 1)
             try:
                 call()
                 missed.append(name)
-                poke(ctx, 0)
+                poke.set_status_word(ctx, 0)
             except capi.TbpmError as e:
                 assert e.status == -4, (name, str(e))
             call()
@@ -82,3 +83,21 @@ def test_synchronous_calls_report_an_expired_wait_once(capi, poke):
         capi.tbpm_lattice_destroy(lat)
     finally:
         capi.tbpm_destroy(ctx)
+
+
+def test_a_cooperative_grid_that_does_not_fit_takes_another_pass(capi, poke):
+    """A context that believes in more SMs than there are plans 256 CTAs of 205 KB, one to an SM; the launch is
+    refused on the host and the request runs in the register sweep."""
+    mu = []
+    for sms in (0, 300):
+        ctx = capi.tbpm_create(0)
+        try:
+            lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(0, (360, 1024), t=1.0, W=1.0, seed=3))
+            if sms:
+                poke.set_num_sms(ctx, sms)
+            mu.append(np.zeros((8, 32, 2)))
+            capi.tbpm_moments(ctx, lat, capi.request(n_states=8, n_moments=32, state_seed=3), mu[-1])
+            capi.tbpm_lattice_destroy(lat)
+        finally:
+            capi.tbpm_destroy(ctx)
+    assert np.max(np.abs(mu[0] - mu[1])) <= 1e-6
