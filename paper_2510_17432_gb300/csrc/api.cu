@@ -1350,15 +1350,23 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
 
 // Whether the resident kernel runs this moment request: a small lattice, unless a chosen fusion mode names
 // another pass that takes it (mode 0: one step per launch).  Where the register sweep takes the lattice as
-// well, the resident kernel is the faster one up to its own limit for four and more states (us per step,
-// resident against sweep: 8 states on 300 x 300 honeycomb cells 8.8 / 13.4, 4 states on 256 x 256 4.6 / 7.1),
-// but not for large blocks of one or two states, whose 8-byte and single-pair units leave its shared-memory
-// reads half empty (two states: 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state: 262k 4.5 / 4.3,
-// 33k 2.1 / 2.9, 1.6M 16.2 / 6.4).
+// well, the resident kernel is faster alone, but its grid must be resident as a whole: requests of several
+// contexts overlap only as far as several grids fit, while sweeps and one-step passes fill each other's gaps.
+// Requests of 512 moments a second from one and from eight contexts, one-step or sweep before -> resident:
+// honeycomb pairs 64 x 64 x 8 states 506 / 3591 -> 1292 / 3962, 100 x 100 x 4 693 / 4737 -> 1379 / 3225,
+// 250 x 250 x 8 247 / 849 -> 493 / 503 (sweep now 302 / 998).  So honeycomb pairs, which had the sweep, go
+// resident up to 70,000 site-states, where no number of contexts is slower; other kinds gained at both
+// ends (300 x 300 square, 8 states 156 / 361 -> 566 / 812) but for complex128 honeycombs, whose FP64 time does not
+// overlap: 160 x 160 x 4 states 160 / 340 -> 216 / 260, so four states and more stop at 90,000 (below it, two
+// states on 110 x 110 cells 438 / 1294 -> 951 / 1043; four contexts 960 -> 1036).  Blocks of one or two states leave the shared-memory
+// reads half empty and stop where the sweep is as fast alone (us per step, resident / sweep: two states
+// 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1 / 2.9).
 bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
   if (ctx->fusion_set && (ctx->fusion == 0 || fused_applicable(lat, pl.precision, pl.Spad) ||
                           (ctx->fusion >= 8 && sweep_ok(lat, pl))))
     return false;
+  if (fused_applicable(lat, pl.precision, pl.Spad) && pl.n * pl.Spad > 70000) return false;
+  if (pl.precision == TBPM_C128 && lat->geom.kind == TBPM_HONEYCOMB && pl.Spad >= 4 && pl.n * pl.Spad > 90000) return false;
   if (pl.Spad <= 2 && pl.n * pl.Spad > (pl.Spad == 1 ? 200000 : 1000000) && sweep_ok(lat, pl)) return false;
   return resident_applicable(ctx, lat, pl.precision, pl.Spad, steps);
 }

@@ -126,8 +126,12 @@ __device__ __forceinline__ void line_neighbours(const Geom& g, int64_t row, int6
   nb[3] = b.zdn;
 }
 
-template <int KIND, typename R, int SPT>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs a) {
+// MAXT: threads at most.  512 threads with the registers they would like (78 to 84) fill an SM's register file, and
+// requests of two contexts took turns: with two CTAs to an SM (48 registers, no spills) 100 x 100 honeycomb cells
+// with 8 states from eight contexts went from 1086 to 2355 requests a second and one context's from 1026 to 970.
+// Smaller CTAs leave room as they are.
+template <int KIND, typename R, int SPT, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == kResThreads ? 2 : 1) k_resident(ResArgs a) {
   using PK = Pack<R, SPT>;
   constexpr int NL = KIND == TBPM_CUBIC ? 4 : 2;  // neighbour lines
   constexpr int NV = 2 * SPT;                     // sums per thread: A and B of each state of the unit
@@ -308,13 +312,16 @@ __global__ void __launch_bounds__(256) k_resident_moments(const double* partials
   }
 }
 
-template <int KIND, typename R, int SPT>
-void* resident_fn() { return (void*)k_resident<KIND, R, SPT>; }
+template <typename R, int SPT, int MAXT>
+void* resident_kind(int kind) {
+  return kind == TBPM_SQUARE      ? (void*)k_resident<TBPM_SQUARE, R, SPT, MAXT>
+         : kind == TBPM_HONEYCOMB ? (void*)k_resident<TBPM_HONEYCOMB, R, SPT, MAXT>
+                                  : (void*)k_resident<TBPM_CUBIC, R, SPT, MAXT>;
+}
 
 template <typename R, int SPT>
-void* resident_kind(int kind) {
-  return kind == TBPM_SQUARE ? resident_fn<TBPM_SQUARE, R, SPT>()
-         : kind == TBPM_HONEYCOMB ? resident_fn<TBPM_HONEYCOMB, R, SPT>() : resident_fn<TBPM_CUBIC, R, SPT>();
+void* resident_fn(int kind, int threads) {
+  return threads <= kResThreads / 2 ? resident_kind<R, SPT, kResThreads / 2>(kind) : resident_kind<R, SPT, kResThreads>(kind);
 }
 
 // Lines per CTA and shared memory of a request; false when it does not fit.
@@ -361,8 +368,9 @@ int launch_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs
     return TBPM_EUNSUPPORTED;
   }
   const int spt = precision == TBPM_C64 && ra.S >= 2 ? 2 : 1;
-  void* fn = precision == TBPM_C128 ? resident_kind<double, 1>(lat->geom.kind)
-             : spt == 2 ? resident_kind<float, 2>(lat->geom.kind) : resident_kind<float, 1>(lat->geom.kind);
+  const int kind = lat->geom.kind;
+  void* fn = precision == TBPM_C128 ? resident_fn<double, 1>(kind, r.threads)
+             : spt == 2 ? resident_fn<float, 2>(kind, r.threads) : resident_fn<float, 1>(kind, r.threads);
   TBPM_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   TBPM_TRY(ensure(ctx, ctx->ws_fused_partials, sizeof(double) * (size_t)steps * 2 * ra.S * r.ctas));
   // packets: their tags must never meet an earlier launch's, so the buffer starts at zero and the tags count on
