@@ -86,6 +86,65 @@ static void release(tbpm_ctx* ctx, DevBuf& b) {
   b.cap = 0;
 }
 
+static std::vector<DevBuf*> workspaces(tbpm_ctx* ctx) {
+  return {&ctx->ws_phi[0], &ctx->ws_phi[1], &ctx->ws_psi, &ctx->ws_acc, &ctx->ws_partials,
+          &ctx->ws_counter, &ctx->ws_mu, &ctx->ws_table, &ctx->ws_aux, &ctx->ws_out,
+          &ctx->ws_energies, &ctx->ws_recon, &ctx->ws_phi2[0], &ctx->ws_phi2[1],
+          &ctx->ws_fused_partials, &ctx->ws_qe, &ctx->ws_qe_coef, &ctx->ws_xdot, &ctx->ws_blk, &ctx->ws_blk_coef,
+          &ctx->ws_jpsi, &ctx->ws_ec, &ctx->ws_fermi, &ctx->ws_packets};
+}
+
+// Bytes that further allocations can have: free on the device, and idle in the pool that keeps freed memory.
+static size_t memory_left(tbpm_ctx* ctx) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  cudaMemPool_t pool;
+  uint64_t reserved = 0, used = 0;
+  if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    cudaGetLastError();
+    return free_b;
+  }
+  return free_b + (size_t)(reserved > used ? reserved - used : 0);
+}
+
+static size_t kept_bytes(tbpm_ctx* ctx) {
+  size_t sum = 0;
+  for (DevBuf* b : workspaces(ctx)) sum += b->cap;
+  return sum;
+}
+
+static int release_workspaces(tbpm_ctx* ctx) {
+  for (DevBuf* b : workspaces(ctx)) release(ctx, *b);
+  ctx->packet_cap = 0;  // the packet buffer's tags start anew with the next one
+  TBPM_CK(cudaStreamSynchronize(ctx->stream));
+  return TBPM_OK;
+}
+
+// Before a request that sizes its blocks by the memory there is: workspaces kept from earlier requests go where
+// they are more than half of what is left, so that the request sees the device that a context's first one sees.
+// (With less than that kept, a window that the first call could have in full fits again: at most a third of the
+// memory is kept, and a window takes up to half of what is left.)
+static int fresh_workspaces(tbpm_ctx* ctx) {
+  return 2 * kept_bytes(ctx) > memory_left(ctx) ? release_workspaces(ctx) : TBPM_OK;
+}
+
+// Runs a request; where memory does not suffice, again without what earlier requests kept, and then in the form
+// with the fewest state blocks (index lists instead of the full layout, one step per pass).
+template <typename F>
+static int with_memory(tbpm_ctx* ctx, F body) {
+  int r = body();
+  for (int lean = 0; lean < 2 && r == TBPM_ENOMEM; ++lean) {
+    clear_error();
+    TBPM_TRY(release_workspaces(ctx));
+    ctx->lean = lean != 0;
+    r = body();
+  }
+  ctx->lean = false;
+  return r;
+}
+
 template <typename T>
 static int dev_alloc(tbpm_ctx* ctx, T** p, size_t count) {
   cudaError_t e = cudaMallocAsync((void**)p, std::max<size_t>(1, count) * sizeof(T), ctx->stream);
@@ -516,12 +575,7 @@ int tbpm_destroy(tbpm_ctx* ctx) {
   clear_error();
   if (!ctx) return TBPM_OK;
   cudaSetDevice(ctx->device);
-  DevBuf* bufs[] = {&ctx->ws_phi[0], &ctx->ws_phi[1], &ctx->ws_psi, &ctx->ws_acc, &ctx->ws_partials,
-                    &ctx->ws_counter, &ctx->ws_mu, &ctx->ws_table, &ctx->ws_aux, &ctx->ws_out,
-                    &ctx->ws_energies, &ctx->ws_recon, &ctx->ws_phi2[0], &ctx->ws_phi2[1],
-                    &ctx->ws_fused_partials, &ctx->ws_qe, &ctx->ws_qe_coef, &ctx->ws_xdot, &ctx->ws_blk, &ctx->ws_blk_coef,
-                    &ctx->ws_jpsi, &ctx->ws_ec, &ctx->ws_fermi, &ctx->ws_packets};
-  for (DevBuf* b : bufs) release(ctx, *b);
+  for (DevBuf* b : workspaces(ctx)) release(ctx, *b);
   cudaStreamSynchronize(ctx->stream);
   for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
   ctx->graphs.clear();
@@ -1362,6 +1416,7 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
 // reads half empty and stop where the sweep is as fast alone (us per step, resident / sweep: two states
 // 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1 / 2.9).
 bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
+  if (ctx->lean) return false;
   if (ctx->fusion_set && (ctx->fusion == 0 || fused_applicable(lat, pl.precision, pl.Spad) ||
                           (ctx->fusion >= 8 && sweep_ok(lat, pl))))
     return false;
@@ -1393,7 +1448,7 @@ int run_moments(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const
     clear_error();
   }
   int fmode = 0;
-  TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));
+  if (!ctx->lean) TBPM_TRY(choose_fusion(ctx, lat, req, pl, M, &fmode));
   const int64_t steps = M / 2;
   const int K = fused_steps(fmode);
   if (fmode >= 8 && steps - 1 >= K && masked_sweep_ok(lat, pl)) {
@@ -1558,19 +1613,18 @@ void block_coefficients(double tau, int bb, std::vector<double>* coef, std::vect
   }
 }
 
-// Largest b whose accumulators fit in 80% of the free device memory (and <= 256, <= n_steps).
-int64_t block_cap(const Plan& pl, int64_t n_steps) {
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  const int64_t by_mem = (int64_t)std::max<double>(1.0, 0.8 * (double)free_b / (double)pl.state_bytes - 4.0 - 34.0);
+// Largest b (<= 256, <= n_steps) whose accumulators fit in 80% of the memory there is, beside 34 blocks for a
+// window of 32 terms and 4 for the recurrence; what is over goes to a longer window.
+int64_t block_cap(tbpm_ctx* ctx, const Plan& pl, int64_t n_steps) {
+  const double have = (double)(memory_left(ctx) + ctx->ws_acc.cap + ctx->ws_blk.cap);
+  const int64_t by_mem = (int64_t)std::max<double>(1.0, 0.8 * have / (double)pl.state_bytes - 4.0 - 34.0);
   return std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(by_mem, 256), n_steps));
 }
 
-// Slots of a window: at most n_terms and what a flush takes, and the buffer at most half the free memory.
-int window_slots(const Plan& pl, int64_t n_terms) {
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  const int64_t fit = (int64_t)(0.5 * (double)free_b / (double)pl.state_bytes) - 2;
+// Slots of a window in the buffer b: at most n_terms and what a flush takes, and b at most half the memory it and
+// all further buffers can have.
+int window_slots(tbpm_ctx* ctx, const DevBuf& b, const Plan& pl, int64_t n_terms) {
+  const int64_t fit = (int64_t)(0.5 * (double)(memory_left(ctx) + b.cap) / (double)pl.state_bytes) - 2;
   const int64_t T = std::min<int64_t>(std::min<int64_t>(flush_max_terms(), fit), n_terms);
   return (int)(T >= 4 && T < n_terms ? T / 4 * 4 : T);  // a further window starts at a multiple of four terms
 }
@@ -1600,7 +1654,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
   g.r.prev_out = ctx->ws_phi[1].p;
   const bool sweep = sweep_ok(lat, pl);
   // terms per timed flush: enough that the accumulators' own traffic weighs little
-  const int Tm = ctx->buffer_blocks && k_acc >= 2 ? window_slots(pl, 24) : 0;
+  const int Tm = ctx->buffer_blocks && k_acc >= 2 ? window_slots(ctx, ctx->ws_blk, pl, 24) : 0;
   const bool buffered = Tm >= 4 && ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)Tm) == TBPM_OK &&
                         ensure(ctx, ctx->ws_blk_coef, sizeof(double) * (size_t)Tm * k_acc) == TBPM_OK;
   std::vector<std::function<int()>> pass;
@@ -1668,7 +1722,7 @@ int measure_pass_costs(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req
 // b_opt = argmin_b C(b) with measured costs (Sec. II.B), capped by memory.
 int choose_block(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan& pl, int64_t n_steps,
                  int64_t* b, double* t_amxsy, double* t_axpy) {
-  int64_t cap = block_cap(pl, n_steps);
+  int64_t cap = block_cap(ctx, pl, n_steps);
   // buffered blocks: one flush serves 16 accumulators per pass over the buffer; past that every
   // further 16 re-read the buffer, which the linear cost model does not see
   if (ctx->buffer_blocks) cap = std::min<int64_t>(cap, 16);
@@ -1794,7 +1848,7 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   // sequential form keeps its fused one-accumulator pass.
   int T = 0;
   if (ctx->buffer_blocks && (b >= 2 || sweep_ok(lat, pl)))
-    T = window_slots(pl, *std::max_element(nper_full.begin(), nper_full.end()));
+    T = window_slots(ctx, ctx->ws_blk, pl, *std::max_element(nper_full.begin(), nper_full.end()));
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
     // amplitudes, full block then last block
@@ -1867,12 +1921,14 @@ int run_blocks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const 
   return turn();
 }
 
-// Time blocks, quasi-eigenstates and the conductivity of a vacancy lattice take the full layout where
-// the masked sweep applies and the buffer's window fits.
-int take_full_layout(tbpm_ctx* ctx, tbpm_lattice* lat, Plan* pl) {
-  if (!ctx->buffer_blocks || !masked_sweep_ok(lat, *pl)) return TBPM_OK;
+// Time blocks, quasi-eigenstates and the conductivity of a vacancy lattice take the full layout where the masked
+// sweep applies and memory is ample: `blocks` state blocks of the request, six of the propagation (16-fold
+// roundings of the allocations included), and twice a window of eight terms, all of them for every site.
+int take_full_layout(tbpm_ctx* ctx, tbpm_lattice* lat, Plan* pl, int64_t blocks) {
+  if (!ctx->buffer_blocks || ctx->lean || !masked_sweep_ok(lat, *pl)) return TBPM_OK;
   set_layout(lat, pl, true);
-  if (window_slots(*pl, flush_max_terms()) < 8) set_layout(lat, pl, false);
+  const double have = (double)(memory_left(ctx) + kept_bytes(ctx));
+  if (((double)blocks + 6.0) * 1.07 + 20.0 > have / (double)pl->state_bytes) set_layout(lat, pl, false);
   return pl->full ? ensure_dfull(lat) : TBPM_OK;
 }
 
@@ -1901,7 +1957,7 @@ int run_correlation(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, c
                                       lat->H0 / lat->half, pl.tau, d_C));
     return TBPM_OK;
   }
-  TBPM_TRY(take_full_layout(ctx, lat, &pl));
+  TBPM_TRY(take_full_layout(ctx, lat, &pl, std::max<int64_t>(16, req->time_block)));
   if (req->form == TBPM_SEQUENTIAL) return run_blocks(ctx, lat, req, pl, n_steps, 1, d_C);
   if (req->form == TBPM_CONCURRENT_S) {
     int64_t b = req->time_block;
@@ -1936,7 +1992,7 @@ int run_qe(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     TBPM_TRY(launch_qe_coefficients(ctx, table, (int)n_steps, (int)need, d_E, nE, lat->H0, tphys, phase, coef));
     // buffered accumulation: the recurrence fills a window of T slots, and every T terms one flush
     // adds sum_t C_t(E) phi_t to all N_E accumulators
-    const int T = window_slots(pl, need);
+    const int T = window_slots(ctx, ctx->ws_acc, pl, need);
     if (T >= 4) {
       TBPM_TRY(ensure(ctx, ctx->ws_acc, pl.state_bytes * (size_t)(T + 2)));
       char* const terms = (char*)ctx->ws_acc.p + 2 * pl.state_bytes;
@@ -2079,7 +2135,7 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
   tbpm_request qreq = *req;
   qreq.form = nE <= 200 ? TBPM_CONCURRENT_E : TBPM_CONCURRENT_S;
   qreq.time_block = 0;
-  TBPM_TRY(take_full_layout(ctx, lat, &pl));
+  TBPM_TRY(take_full_layout(ctx, lat, &pl, nE + std::max<int64_t>(16, req->time_block)));
   TBPM_TRY(run_qe(ctx, lat, &qreq, pl, d_E, nE));
   const int rows = pl.Spad * nE;
   const int64_t W = n_steps + 1;
@@ -2117,9 +2173,9 @@ int run_ec(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, const Plan
     TBPM_TRY(base_args(ctx, lat, pl, &g.r, 3));
     g.b = 0;
     g.j_done = -1;
-    // buffered: the recurrence fills a window of up to 32 slots and one block inner product
+    // buffered: the recurrence fills a window of slots and one block inner product
     // gives the window's moments against all kets (each ket read once per window, not per term)
-    const int T = ctx->buffer_blocks ? window_slots(pl, Nn) : 0;
+    const int T = ctx->buffer_blocks ? window_slots(ctx, ctx->ws_blk, pl, Nn) : 0;
     if (T >= 4) {
       TBPM_TRY(ensure(ctx, ctx->ws_blk, pl.state_bytes * (size_t)(T + 2)));
       char* const terms = (char*)ctx->ws_blk.p + 2 * pl.state_bytes;
@@ -2196,12 +2252,12 @@ int fermi_series(tbpm_ctx* ctx, const tbpm_lattice* lat, double mu, double kT, i
 }
 
 // Workspaces of the response drivers are given back between their phases only where memory is short
-// (a block above an eighth of the free memory): freeing and allocating them again on every call cost
+// (a block above an eighth of what is left): freeing and allocating them again on every call cost
 // 7 of 85 ms of the optical conductivity of 2.1M sites.
 void release_if_tight(tbpm_ctx* ctx, DevBuf& b) {
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  if (b.cap > free_b / 8) release(ctx, b);
+  if (b.cap <= memory_left(ctx) / 8) return;
+  release(ctx, b);
+  cudaStreamSynchronize(ctx->stream);  // the pool counts the block as idle from here on
 }
 
 // out = sum_{n < n_terms} coef_n T_n(H~) X for one state block of plan pc.  The recurrence runs
@@ -2216,9 +2272,9 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
   g.b = 1;
   g.j_lo = 0;
   g.j_done = -1;
-  // buffered: terms go into a window of up to 32 slots and one flush adds sum_n a_n T_n phi to
+  // buffered: terms go into a window of slots and one flush adds sum_n a_n T_n phi to
   // the output per window (as the buffered time blocks)
-  const int T = ctx->buffer_blocks ? window_slots(pc, n_terms) : 0;
+  const int T = ctx->buffer_blocks ? window_slots(ctx, ctx->ws_blk, pc, n_terms) : 0;
   if (T >= 4) {
     TBPM_TRY(ensure(ctx, ctx->ws_blk, pc.state_bytes * (size_t)(T + 2)));
     char* const terms = (char*)ctx->ws_blk.p + 2 * pc.state_bytes;
@@ -2242,12 +2298,11 @@ int apply_series_bufs(tbpm_ctx* ctx, tbpm_lattice* lat, const Plan& pc, void* b0
 }
 
 // Largest power-of-two number of states per pass (<= cap) for which `blocks` state blocks of
-// that width fit in 85% of the free device memory; 0 when not even one state fits.
-int states_per_pass(const tbpm_lattice* lat, size_t elem, int cap, double blocks) {
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
+// that width fit in 85% of the memory there is, kept workspaces included; 0 when not even one state fits.
+int states_per_pass(tbpm_ctx* ctx, const tbpm_lattice* lat, size_t elem, int cap, double blocks) {
+  const double have = (double)(memory_left(ctx) + kept_bytes(ctx));
   int k = cap;
-  while (k >= 1 && blocks * (double)lat->n_sites * k * elem > 0.85 * (double)free_b) k >>= 1;
+  while (k >= 1 && blocks * (double)lat->n_sites * k * elem > 0.85 * have) k >>= 1;
   return k;
 }
 
@@ -2457,10 +2512,12 @@ int tbpm_moments_device(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
   const int64_t M = req->n_moments;
-  if (pl.Spad == pl.S) return run_moments(ctx, lat, req, pl, M, d_mu);
-  TBPM_TRY(ensure(ctx, ctx->ws_mu, sizeof(double) * 2 * (size_t)std::max<int64_t>(M, 2) * pl.Spad));
-  TBPM_TRY(run_moments(ctx, lat, req, pl, M, (double*)ctx->ws_mu.p));
-  return copy_rows(ctx, d_mu, (double*)ctx->ws_mu.p, pl.S, 2 * (size_t)M, cudaMemcpyDeviceToDevice);
+  return with_memory(ctx, [&]() -> int {
+    if (pl.Spad == pl.S) return run_moments(ctx, lat, req, pl, M, d_mu);
+    TBPM_TRY(ensure(ctx, ctx->ws_mu, sizeof(double) * 2 * (size_t)std::max<int64_t>(M, 2) * pl.Spad));
+    TBPM_TRY(run_moments(ctx, lat, req, pl, M, (double*)ctx->ws_mu.p));
+    return copy_rows(ctx, d_mu, (double*)ctx->ws_mu.p, pl.S, 2 * (size_t)M, cudaMemcpyDeviceToDevice);
+  });
 }
 
 int tbpm_moments(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, double* mu) {
@@ -2475,8 +2532,10 @@ int tbpm_moments(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* r
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
   const int64_t M = req->n_moments;
-  TBPM_TRY(ensure(ctx, ctx->ws_mu, sizeof(double) * 2 * (size_t)std::max<int64_t>(M, 2) * pl.Spad));
-  TBPM_TRY(run_moments(ctx, lat, req, pl, M, (double*)ctx->ws_mu.p));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    TBPM_TRY(ensure(ctx, ctx->ws_mu, sizeof(double) * 2 * (size_t)std::max<int64_t>(M, 2) * pl.Spad));
+    return run_moments(ctx, lat, req, pl, M, (double*)ctx->ws_mu.p);
+  }));
   TBPM_TRY(copy_rows(ctx, mu, (double*)ctx->ws_mu.p, pl.S, 2 * (size_t)M, cudaMemcpyDeviceToHost));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
   return sweep_status(ctx);
@@ -2494,10 +2553,13 @@ int tbpm_correlation_device(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
   const size_t row = 2 * (size_t)(req->n_steps + 1);
-  if (pl.Spad == pl.S) return run_correlation(ctx, lat, req, pl, d_C);
-  TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * row * pl.Spad));
-  TBPM_TRY(run_correlation(ctx, lat, req, pl, (double*)ctx->ws_out.p));
-  return copy_rows(ctx, d_C, (double*)ctx->ws_out.p, pl.S, row, cudaMemcpyDeviceToDevice);
+  TBPM_TRY(fresh_workspaces(ctx));
+  return with_memory(ctx, [&]() -> int {
+    if (pl.Spad == pl.S) return run_correlation(ctx, lat, req, pl, d_C);
+    TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * row * pl.Spad));
+    TBPM_TRY(run_correlation(ctx, lat, req, pl, (double*)ctx->ws_out.p));
+    return copy_rows(ctx, d_C, (double*)ctx->ws_out.p, pl.S, row, cudaMemcpyDeviceToDevice);
+  });
 }
 
 int tbpm_correlation(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, double* C) {
@@ -2516,8 +2578,11 @@ int tbpm_correlation(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_reques
     return TBPM_EINVAL;
   }
   const size_t row = 2 * (size_t)(req->n_steps + 1);
-  TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * row * pl.Spad));
-  TBPM_TRY(run_correlation(ctx, lat, req, pl, (double*)ctx->ws_out.p));
+  TBPM_TRY(fresh_workspaces(ctx));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    TBPM_TRY(ensure(ctx, ctx->ws_out, sizeof(double) * row * pl.Spad));
+    return run_correlation(ctx, lat, req, pl, (double*)ctx->ws_out.p);
+  }));
   TBPM_TRY(copy_rows(ctx, C, (double*)ctx->ws_out.p, pl.S, row, cudaMemcpyDeviceToHost));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
   return sweep_status(ctx);
@@ -2535,7 +2600,8 @@ int tbpm_dos_device(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request
   Plan pl;
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
-  return run_dos(ctx, lat, req, pl, d_E, nE, d_D);
+  if (req->dos_method != TBPM_DOS_JACKSON) TBPM_TRY(fresh_workspaces(ctx));
+  return with_memory(ctx, [&]() -> int { return run_dos(ctx, lat, req, pl, d_E, nE, d_D); });
 }
 
 int tbpm_dos(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, const double* energies,
@@ -2554,11 +2620,15 @@ int tbpm_dos(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_request* req, 
     set_error("n_energies must be >= 1");
     return TBPM_EINVAL;
   }
-  TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE * (1 + pl.S)));
-  double* dE = (double*)ctx->ws_energies.p;
-  double* dD = dE + nE;
-  TBPM_CK(cudaMemcpyAsync(dE, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
-  TBPM_TRY(run_dos(ctx, lat, req, pl, dE, nE, dD));
+  if (req->dos_method != TBPM_DOS_JACKSON) TBPM_TRY(fresh_workspaces(ctx));
+  double* dD = nullptr;
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE * (1 + pl.S)));
+    double* dE = (double*)ctx->ws_energies.p;
+    dD = dE + nE;
+    TBPM_CK(cudaMemcpyAsync(dE, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
+    return run_dos(ctx, lat, req, pl, dE, nE, dD);
+  }));
   TBPM_CK(cudaMemcpyAsync(D, dD, sizeof(double) * nE * pl.S, cudaMemcpyDeviceToHost, ctx->stream));
   TBPM_CK(cudaStreamSynchronize(ctx->stream));
   return sweep_status(ctx);
@@ -2621,8 +2691,12 @@ int tbpm_block_autotune(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_req
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
   double ta = 0, tx = 0;
-  TBPM_TRY(take_full_layout(ctx, lat, &pl));
-  TBPM_TRY(choose_block(ctx, lat, req, pl, n_steps, b_opt, &ta, &tx));
+  TBPM_TRY(fresh_workspaces(ctx));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    set_layout(lat, &pl, false);
+    TBPM_TRY(take_full_layout(ctx, lat, &pl, 16));
+    return choose_block(ctx, lat, req, pl, n_steps, b_opt, &ta, &tx);
+  }));
   if (times_ms) {
     times_ms[0] = ta;
     times_ms[1] = tx;
@@ -2642,15 +2716,19 @@ int tbpm_quasi_eigenstates(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_
   Plan pl;
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
-  TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE));
-  TBPM_CK(cudaMemcpyAsync(ctx->ws_energies.p, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
-  TBPM_TRY(take_full_layout(ctx, lat, &pl));
-  TBPM_TRY(run_qe(ctx, lat, req, pl, (const double*)ctx->ws_energies.p, (int)nE));
+  TBPM_TRY(fresh_workspaces(ctx));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE));
+    TBPM_CK(cudaMemcpyAsync(ctx->ws_energies.p, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
+    set_layout(lat, &pl, false);
+    TBPM_TRY(take_full_layout(ctx, lat, &pl, nE + std::max<int64_t>(16, req->time_block)));
+    TBPM_TRY(run_qe(ctx, lat, req, pl, (const double*)ctx->ws_energies.p, (int)nE));
+    return pl.full ? ensure(ctx, ctx->ws_phi[0], pl.state_bytes) : TBPM_OK;
+  }));
   const int64_t n = lat->n_sites;
   for (int64_t k = 0; k < nE; ++k) {
     const char* block = (const char*)ctx->ws_qe.p + (size_t)k * pl.state_bytes;
     if (pl.full) {  // back to the compact order of the active sites
-      TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
       const int nb = grid_for(ctx, n * pl.P, kT);
       if (pl.spt == 2)
         k_compact_states<<<nb, kT, 0, ctx->stream>>>(n, pl.P, lat->full_of, (const float4*)block,
@@ -2687,10 +2765,13 @@ int tbpm_conductivity_overlap(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tb
   Plan pl;
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
-  TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE));
-  TBPM_CK(cudaMemcpyAsync(ctx->ws_energies.p, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
   double *d_C = nullptr, *d_sigma = nullptr;
-  TBPM_TRY(run_ec(ctx, lat, req, pl, (const double*)ctx->ws_energies.p, (int)nE, direction, &d_C, &d_sigma));
+  TBPM_TRY(fresh_workspaces(ctx));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    TBPM_TRY(ensure(ctx, ctx->ws_energies, sizeof(double) * (size_t)nE));
+    TBPM_CK(cudaMemcpyAsync(ctx->ws_energies.p, energies, sizeof(double) * nE, cudaMemcpyHostToDevice, ctx->stream));
+    return run_ec(ctx, lat, req, pl, (const double*)ctx->ws_energies.p, (int)nE, direction, &d_C, &d_sigma);
+  }));
   // rows s*nE + k of the first S states are contiguous
   const size_t rows = (size_t)pl.S * nE;
   if (C)
@@ -2716,14 +2797,17 @@ int tbpm_fermi_apply(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_reques
   Plan pl;
   TBPM_TRY(make_plan(lat, req, &pl));
   TBPM_CK(cudaSetDevice(ctx->device));
-  const double* coef = nullptr;
-  int nf = 0;
-  TBPM_TRY(fermi_series(ctx, lat, mu, kT, sqrt_f ? 1 : 0, &coef, &nf));
-  TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
-  TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
-  TBPM_TRY(ensure(ctx, ctx->ws_phi2[0], pl.state_bytes));
-  TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
-  TBPM_TRY(apply_series_bufs(ctx, lat, pl, ctx->ws_phi[0].p, ctx->ws_phi[1].p, ctx->ws_phi2[0].p, coef, nf));
+  TBPM_TRY(fresh_workspaces(ctx));
+  TBPM_TRY(with_memory(ctx, [&]() -> int {
+    const double* coef = nullptr;
+    int nf = 0;
+    TBPM_TRY(fermi_series(ctx, lat, mu, kT, sqrt_f ? 1 : 0, &coef, &nf));
+    TBPM_TRY(ensure(ctx, ctx->ws_phi[0], pl.state_bytes));
+    TBPM_TRY(ensure(ctx, ctx->ws_phi[1], pl.state_bytes));
+    TBPM_TRY(ensure(ctx, ctx->ws_phi2[0], pl.state_bytes));
+    TBPM_TRY(init_states(ctx, lat, req, pl, ctx->ws_phi[0].p, nullptr));
+    return apply_series_bufs(ctx, lat, pl, ctx->ws_phi[0].p, ctx->ws_phi[1].p, ctx->ws_phi2[0].p, coef, nf);
+  }));
   const int64_t n = lat->n_sites;
   for (int s = 0; s < pl.S; ++s)
     TBPM_CK(cudaMemcpy2DAsync((char*)out + (size_t)s * n * pl.elem, pl.elem,
@@ -2751,7 +2835,8 @@ int response_chunks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, i
   int cap = std::min(pl.Spad, 16);
   if (ctx->max_pass_states > 0)
     while (cap > ctx->max_pass_states) cap >>= 1;
-  const int k = states_per_pass(lat, pl.elem, cap, pair_blocks);
+  TBPM_TRY(fresh_workspaces(ctx));
+  const int k = states_per_pass(ctx, lat, pl.elem, cap, pair_blocks);
   if (k < 1) {
     set_error("not enough device memory for one state of %lld sites", (long long)lat->n_sites);
     return TBPM_ENOMEM;
@@ -2763,7 +2848,7 @@ int response_chunks(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, i
     Plan pk;
     TBPM_TRY(make_plan(lat, &rq, &pk));
     pk.s0 = s0;
-    TBPM_TRY(pass(&rq, pk));
+    TBPM_TRY(with_memory(ctx, [&]() -> int { return pass(&rq, pk); }));
   }
   return TBPM_OK;
 }

@@ -218,6 +218,7 @@ struct tbpm_ctx {
   tbpm::DevBuf ws_packets;
   size_t packet_cap = 0;
   int64_t packet_tag = 0;
+  bool lean = false;  // a request that ran out of memory is run again with the fewest state blocks
   int max_pass_states = 0;  // cap on states per pass of the OC, DP and CD drivers (0 = by memory)
   double* pinned = nullptr;
   size_t pinned_cap = 0;
