@@ -178,13 +178,17 @@ int64_t tbpm_launch_count(const tbpm_ctx* ctx);
  * register-resident sweep (each thread keeps the recurrence levels of its cell in registers and
  * exchanges only the x-neighbours through shared memory, one barrier per row; rows of phi_n and
  * phi_{n-1} arrive by TMA bulk copies; 128-, 192- and 256-thread CTAs; a lattice narrower than
- * one band takes mode 5).  Default 8; until a
- * mode has been chosen by this call, moment requests on small matrix-free lattices (two state blocks within
- * the SMs' shared memory, up to about 2M complex64 site-states) run all their steps in one resident launch,
- * and afterwards those that no fused pass of the chosen mode takes (mode 0: none).  -1 = the fastest of modes 0, 4, 5 and 8 timed on the
+ * one band takes mode 5).  Default 8.  A mode chosen by this call, 8 included, names the passes of every
+ * request: small lattices then take it too instead of the resident recurrence (tbpm_set_resident).  -1 = the fastest of modes 0, 4, 5 and 8 timed on the
  * request's lattice shape.  Results of different modes agree within the complex64 tolerance, not
  * bit for bit; each mode is deterministic.  Modes outside -1..10 are rejected with TBPM_EINVAL. */
 int tbpm_set_fusion(tbpm_ctx* ctx, int mode);
+/* Resident recurrence (default on): moment requests on small matrix-free lattices (two state blocks within the
+ * SMs' shared memory; honeycomb state pairs up to 70,000 site-states) run all their steps in one cooperative
+ * launch.  tbpm_set_fusion switches it off; enable = 1 after it brings the default back, for small lattices
+ * whatever the mode; enable = 0 alone keeps the mode and leaves small lattices to it.  Its results agree with
+ * those of other passes within the tolerance, not bit for bit. */
+int tbpm_set_resident(tbpm_ctx* ctx, int enable);
 /* mode -1 = autotuned: the first moment request on a lattice shape (kind, sizes, boundaries,
  * path, padded S, precision, disorder) with at least 128 moments times 24 steps of each of modes
  * 0, 4, 5 and 8 on scratch buffers and keeps the fastest for that shape in the context.  Results
@@ -253,6 +257,7 @@ int tbpm_lattice_taps(const tbpm_lattice* lat, int32_t* offsets, double* t);
  *   TBPM_PASS_SWEEP    four-step register sweep (fusion modes 8-10; k_sweep_moments)
  *   TBPM_PASS_ROWS     row-sweep fused pass with shared-memory level rings (modes 3-7)
  *   TBPM_PASS_TILES    2-D tile fused pass (modes 1, 2)
+ *   TBPM_PASS_RESIDENT all steps of a small lattice in one launch (k_resident)
  * Under fusion mode -1 a fused lattice reports TBPM_PASS_STENCIL (the mode is chosen by timing
  * at the first request).  Errors: TBPM_EINVAL for NULL arguments or an invalid request. */
 /* Index checks of a debug build (libtbpm_debug.so, compiled with TBPM_DEBUG; the paper has no
@@ -285,7 +290,7 @@ int tbpm_wait_probe(tbpm_ctx* ctx, int arrive, double budget_s);
 int tbpm_fp32_fma_peak(tbpm_ctx* ctx, double* tflops_scalar, double* tflops_packed);
 
 enum { TBPM_PASS_STENCIL = 0, TBPM_PASS_ELL = 1, TBPM_PASS_TAPS = 2, TBPM_PASS_SWEEP = 3, TBPM_PASS_ROWS = 4,
-       TBPM_PASS_TILES = 5 };
+       TBPM_PASS_TILES = 5, TBPM_PASS_RESIDENT = 6 };
 int tbpm_moment_pass_kind(tbpm_ctx* ctx, const tbpm_lattice* lat, const tbpm_request* req, int* kind);
 
 /* ---------------------------------------------------------------- states */

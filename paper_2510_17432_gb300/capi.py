@@ -98,6 +98,7 @@ def _bind(lib):
         "tbpm_launch_count": (C.c_int64, [_P]),
         "tbpm_profile": (C.c_int, [_P, C.c_int]),
         "tbpm_set_fusion": (C.c_int, [_P, C.c_int]),
+        "tbpm_set_resident": (C.c_int, [_P, C.c_int]),
         "tbpm_profile_read": (C.c_int, [_P, C.POINTER(C.c_double)]),
         "tbpm_lattice_create": (C.c_int, [_P, C.POINTER(LatticeDesc), C.POINTER(_P)]),
         "tbpm_lattice_destroy": (C.c_int, [_P]),
@@ -154,7 +155,7 @@ def _bind(lib):
 def exported_symbols():
     """Names of every entry point this binding wraps (all declared in include/tbpm.h)."""
     return ["tbpm_create", "tbpm_destroy", "tbpm_last_error", "tbpm_stream", "tbpm_sync",
-            "tbpm_launch_count", "tbpm_set_fusion", "tbpm_profile", "tbpm_profile_read", "tbpm_lattice_create", "tbpm_lattice_destroy", "tbpm_lattice_info",
+            "tbpm_launch_count", "tbpm_set_fusion", "tbpm_set_resident", "tbpm_profile", "tbpm_profile_read", "tbpm_lattice_create", "tbpm_lattice_destroy", "tbpm_lattice_info",
             "tbpm_lattice_export", "tbpm_lattice_taps", "tbpm_moment_pass_kind", "tbpm_fp32_fma_peak", "tbpm_debug_status", "tbpm_wait_probe", "tbpm_states_export", "tbpm_apply_hopping", "tbpm_moments",
             "tbpm_moments_device", "tbpm_correlation", "tbpm_correlation_device", "tbpm_dos",
             "tbpm_dos_device", "tbpm_quasi_eigenstates", "tbpm_conductivity", "tbpm_conductivity_overlap",
@@ -223,6 +224,11 @@ def tbpm_launch_count(ctx) -> int:
 def tbpm_set_fusion(ctx, mode: int):
     """0 = one step per pass, 1..3 = fused variants (see include/tbpm.h)."""
     _check(load().tbpm_set_fusion(ctx, int(mode)))
+
+
+def tbpm_set_resident(ctx, enable: bool):
+    """Small lattices in one resident launch: the default until tbpm_set_fusion names the passes."""
+    _check(load().tbpm_set_resident(ctx, int(bool(enable))))
 
 
 def tbpm_profile(ctx, enable: bool):
@@ -361,7 +367,7 @@ def tbpm_conductivity(ctx, lat, req: Request, direction: int, energies: np.ndarr
                                     _host_ptr(C_out), _host_ptr(sigma)))
 
 
-PASS_STENCIL, PASS_ELL, PASS_TAPS, PASS_SWEEP, PASS_ROWS, PASS_TILES = 0, 1, 2, 3, 4, 5
+PASS_STENCIL, PASS_ELL, PASS_TAPS, PASS_SWEEP, PASS_ROWS, PASS_TILES, PASS_RESIDENT = 0, 1, 2, 3, 4, 5, 6
 DEBUG_KERNELS = {1: "stencil units", 2: "ELL neighbour index", 3: "sweep store", 4: "sweep row copy",
                  5: "serving units"}
 

@@ -617,7 +617,17 @@ int tbpm_set_fusion(tbpm_ctx* ctx, int enable) {
     return TBPM_EINVAL;
   }
   ctx->fusion = enable;
-  ctx->fusion_set = true;
+  ctx->resident = false;  // a chosen mode names the passes
+  return TBPM_OK;
+}
+
+int tbpm_set_resident(tbpm_ctx* ctx, int enable) {
+  clear_error();
+  if (!ctx) {
+    set_error("tbpm_set_resident: ctx is NULL");
+    return TBPM_EINVAL;
+  }
+  ctx->resident = enable != 0;
   return TBPM_OK;
 }
 
@@ -1402,8 +1412,8 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
   ctx->queue_live[k] = true;
 }
 
-// Whether the resident kernel runs this moment request: a small lattice, unless a chosen fusion mode names
-// another pass that takes it (mode 0: one step per launch).  Where the register sweep takes the lattice as
+// Whether the resident kernel runs this moment request: a small lattice, unless a fusion mode has been chosen
+// since (tbpm_set_resident).  Where the register sweep takes the lattice as
 // well, the resident kernel is faster alone, but its grid must be resident as a whole: requests of several
 // contexts overlap only as far as several grids fit, while sweeps and one-step passes fill each other's gaps.
 // Requests of 512 moments a second from one and from eight contexts, one-step or sweep before -> resident:
@@ -1416,10 +1426,7 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
 // reads half empty and stop where the sweep is as fast alone (us per step, resident / sweep: two states
 // 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1 / 2.9).
 bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
-  if (ctx->lean) return false;
-  if (ctx->fusion_set && (ctx->fusion == 0 || fused_applicable(lat, pl.precision, pl.Spad) ||
-                          (ctx->fusion >= 8 && sweep_ok(lat, pl))))
-    return false;
+  if (ctx->lean || !ctx->resident) return false;
   if (fused_applicable(lat, pl.precision, pl.Spad) && pl.n * pl.Spad > 70000) return false;
   if (pl.precision == TBPM_C128 && lat->geom.kind == TBPM_HONEYCOMB && pl.Spad >= 4 && pl.n * pl.Spad > 90000) return false;
   if (pl.Spad <= 2 && pl.n * pl.Spad > (pl.Spad == 1 ? 200000 : 1000000) && sweep_ok(lat, pl)) return false;
@@ -2482,7 +2489,7 @@ int tbpm_moment_pass_kind(tbpm_ctx* ctx, const tbpm_lattice* lat_c, const tbpm_r
   const int m = ctx->fusion;  // -1: autotuned on first use, reported as the mode it would time first
   const int64_t M = req->n_moments > 0 ? req->n_moments : truncation_order_host(req->n_steps * pl.tau);
   if (use_resident(ctx, lat, pl, M / 2)) {
-    *kind = TBPM_PASS_STENCIL;
+    *kind = TBPM_PASS_RESIDENT;
     return TBPM_OK;
   }
   if (m > 0 && fused_applicable(lat, pl.precision, pl.Spad) && M / 2 - 1 >= fused_steps(m)) {

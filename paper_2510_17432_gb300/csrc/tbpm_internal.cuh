@@ -200,7 +200,7 @@ struct tbpm_ctx {
   // time blocks buffer up to 32 Chebyshev vectors and flush them into the accumulators at once
   bool buffer_blocks = true;
   int fusion = 8;  // temporal-fusion mode of the moment pass (8 = four-step register sweep; -1 = autotuned)
-  bool fusion_set = false;  // chosen by tbpm_set_fusion: a lattice a mode's fused pass takes then runs that pass
+  bool resident = true;  // small lattices in one resident launch, until a mode is chosen (tbpm_set_resident)
   // autotuned fusion modes: key (kind, Lx, Ly, Lz, pbc bits, path, Spad, precision, disorder) -> mode
   std::vector<std::pair<std::vector<int64_t>, int>> fusion_choice;
   std::vector<std::pair<int, double>> fusion_timings;  // last autotune: (mode, ms per step)

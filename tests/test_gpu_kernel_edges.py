@@ -205,6 +205,49 @@ def test_resident_recurrence_matches_the_oracle(capi, name, spec, S, prec, M):
         capi.tbpm_destroy(ctx)
 
 
+def test_the_reported_pass_is_the_one_that_runs(capi):
+    """By default, under each mode set (the documented default 8 as well), and with the default brought back: the
+    reported kind, and the launches of the request (resident: states, recurrence, sums; else one a pass or step)."""
+    M = 64
+    cases = [  # lattice, states, precision; kinds by default, in mode 8, in mode 0
+        (dict(kind=1, L=(100, 64), t=-2.7, W=1.0), 4, 0, "RESIDENT", "SWEEP", "STENCIL"),
+        (dict(kind=1, L=(100, 64), t=-2.7, W=1.0), 1, 0, "RESIDENT", "STENCIL", "STENCIL"),
+        (dict(kind=1, L=(200, 180), t=-2.7, W=1.0), 4, 0, "SWEEP", "SWEEP", "STENCIL"),
+        (dict(kind=0, L=(64, 64), t=1.0, W=1.0), 1, 1, "RESIDENT", "STENCIL", "STENCIL"),
+        (dict(kind=0, L=(128, 96), t=1.0, W=1.0), 4, 0, "RESIDENT", "SWEEP", "STENCIL"),
+        (dict(kind=2, L=(9, 8, 7), t=1.0, W=1.0), 2, 0, "RESIDENT", "STENCIL", "STENCIL"),
+    ]
+    launches = {"RESIDENT": 3, "SWEEP": 1 + M // 8, "STENCIL": 1 + M // 2}
+    ctx = capi.tbpm_create(0)
+    try:
+        capi.tbpm_set_graphs(ctx, False)
+        for spec, S, prec, *kinds in cases:
+            lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(seed=3, **spec))
+            req = capi.request(n_states=S, precision=prec, n_moments=M, state_seed=3)
+            for mode, want in zip((None, 8, 0, None), kinds + [kinds[0]]):
+                if mode is None:  # the default, by the call that brings it back
+                    capi.tbpm_set_fusion(ctx, 8)
+                    capi.tbpm_set_resident(ctx, True)
+                else:
+                    capi.tbpm_set_fusion(ctx, mode)
+                assert capi.tbpm_moment_pass_kind(ctx, lat, req) == getattr(capi, "PASS_" + want), (spec, mode)
+                mu = np.zeros((S, M, 2))
+                capi.tbpm_moments(ctx, lat, req, mu)
+                n = capi.tbpm_launch_count(ctx)
+                capi.tbpm_moments(ctx, lat, req, mu)
+                assert capi.tbpm_launch_count(ctx) - n == launches[want], (spec, mode, want)
+            capi.tbpm_lattice_destroy(lat)
+    finally:
+        capi.tbpm_destroy(ctx)
+    ctx = capi.tbpm_create(0)  # and without any call
+    try:
+        lat = capi.tbpm_lattice_create(ctx, capi.lattice_desc(1, (100, 64), t=-2.7, W=1.0, seed=3))
+        assert capi.tbpm_moment_pass_kind(ctx, lat, capi.request(n_states=4, n_moments=M)) == capi.PASS_RESIDENT
+        capi.tbpm_lattice_destroy(lat)
+    finally:
+        capi.tbpm_destroy(ctx)
+
+
 # The cubic march: tiles cut at every edge, lattices of one tile and less, one and two planes, every number of
 # state pairs per CTA, segments of planes, open boundaries, both precisions.
 MARCH = [
