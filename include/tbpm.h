@@ -262,11 +262,13 @@ int tbpm_lattice_taps(const tbpm_lattice* lat, int32_t* offsets, double* t);
  * at the first request).  Errors: TBPM_EINVAL for NULL arguments or an invalid request. */
 /* Index checks of a debug build (libtbpm_debug.so, compiled with TBPM_DEBUG; the paper has no
  * counterpart).  There the hot kernels (stencil, ELL and serving passes, the register sweep's
- * stores and row copies) skip any global-memory access whose index falls outside its buffer and
+ * stores and row copies, the resident recurrence, the cubic march, the tap kernel and the flush of the time
+ * blocks) skip any global-memory access whose index falls outside its buffer and
  * record the first such index per source unit; they never trap, so the context stays usable.
- * words[k] (k = 0: recurrence passes, 1: register sweep, 2: serving) = (kernel id << 48) |
+ * words[k] (k = 0: recurrence passes and the flush, 1: register sweep, 2: serving) = (kernel id << 48) |
  * (index & 0xFFFFFFFFFFFF), 0 when no check failed; kernel ids: 1 stencil units, 2 ELL
- * neighbour index, 3 sweep store, 4 sweep row copy, 5 serving units.  Reading clears the words
+ * neighbour index, 3 sweep store, 4 sweep row copy, 5 serving units, 6 resident units, 7 cubic march
+ * units, 8 flush units, 9 tap kernel units.  Reading clears the words
  * and synchronises the device.  The regular library returns TBPM_EUNSUPPORTED and zero words. */
 int tbpm_debug_status(tbpm_ctx* ctx, uint64_t words[3]);
 

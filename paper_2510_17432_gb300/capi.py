@@ -369,7 +369,7 @@ def tbpm_conductivity(ctx, lat, req: Request, direction: int, energies: np.ndarr
 
 PASS_STENCIL, PASS_ELL, PASS_TAPS, PASS_SWEEP, PASS_ROWS, PASS_TILES, PASS_RESIDENT = 0, 1, 2, 3, 4, 5, 6
 DEBUG_KERNELS = {1: "stencil units", 2: "ELL neighbour index", 3: "sweep store", 4: "sweep row copy",
-                 5: "serving units"}
+                 5: "serving units", 6: "resident units", 7: "cubic march units", 8: "flush units", 9: "tap kernel units"}
 
 
 def tbpm_debug_status(ctx, lib=None) -> list:

@@ -1119,7 +1119,10 @@ int tbpm_debug_status(tbpm_ctx* ctx, uint64_t words[3]) {
 #ifdef TBPM_DEBUG
   TBPM_CK(cudaSetDevice(ctx->device));
   TBPM_CK(cudaDeviceSynchronize());
-  words[0] = debug_take_cheb();
+  words[0] = 0;
+  for (const unsigned long long w : {debug_take_cheb(), debug_take_resident(), debug_take_march(), debug_take_flush(),
+                                     debug_take_taps()})  // every unit's word is cleared, the first one reported
+    if (words[0] == 0) words[0] = w;
   words[1] = debug_take_sweep();
   words[2] = debug_take_serve();
   return TBPM_OK;

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, EB >= 16 ? 2 : 3) k_flush(FlushArgs 
 #pragma unroll
     for (int e = 0; e < EB; ++e) {
       U q{};
-      if (!f.init && e < ne) q = __ldcs(Q + (int64_t)(e0 + e) * f.stride + u);
+      if (!f.init && e < ne && TBPM_DBG_OK((int64_t)(e0 + e) * f.stride + u, f.nb * f.stride, TBPM_DBG_FLUSH)) q = __ldcs(Q + (int64_t)(e0 + e) * f.stride + u);
 #pragma unroll
       for (int k = 0; k < C; ++k) ac[e][k] = part(q, k);
     }
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, EB >= 16 ? 2 : 3) k_flush(FlushArgs 
       U x[TB];
 #pragma unroll
       for (int j = 0; j < TB; ++j) {
-        if (t0 + j < f.T) x[j] = __ldg(Phi + (int64_t)(t0 + j) * f.stride + u);
+        if (t0 + j < f.T && TBPM_DBG_OK((int64_t)(t0 + j) * f.stride + u, f.T * f.stride, TBPM_DBG_FLUSH)) x[j] = __ldg(Phi + (int64_t)(t0 + j) * f.stride + u);
         else x[j] = U{};
       }
 #pragma unroll
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, EB >= 16 ? 2 : 3) k_flush(FlushArgs 
     }
 #pragma unroll
     for (int e = 0; e < EB; ++e) {
-      if (e < ne) {
+      if (e < ne && TBPM_DBG_OK((int64_t)(e0 + e) * f.stride + u, f.nb * f.stride, TBPM_DBG_FLUSH)) {
         __stcs(Q + (int64_t)(e0 + e) * f.stride + u, join(ac[e]));
       }
     }
@@ -195,3 +195,5 @@ int launch_flush(tbpm_ctx* ctx, int precision, int64_t n_numbers, const void* ph
 }
 
 }  // namespace tbpm
+
+TBPM_DEBUG_UNIT(flush)

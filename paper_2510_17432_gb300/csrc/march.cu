@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_cubic_march(MarchArgs a) {
   const int p = tid & (PC - 1), x = (tid >> logPC) & (TX - 1), y = tid >> (logPC + a.logTX);
   const bool own = x < w && y < h;
   const int64_t pstride = a.Lx * a.Ly * a.P;  // units per plane
+  const int64_t n_units = a.Lz * pstride;     // debug build: every unit's index is checked against it
   const int64_t site = (y0 + y) * a.Lx + x0 + x;  // within a plane
   const int64_t oo = site * a.P + (chunk << logPC) + p;
   const int so = ((y + 1) * (TX + 2) + x + 1) * PC + p;
@@ -139,14 +140,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_cubic_march(MarchArgs a) {
       src_rim -= a.Lz * pstride;
       if (!a.pbc_z) n_own = n_rim = 0;
     }
-    if (own) copy_async<sizeof(PK)>(d_own + slot * slice_bytes, src_own, n_own);
-    if (rim) copy_async<sizeof(PK)>(d_rim + slot * slice_bytes, src_rim, n_rim);
+    if (own && (n_own == 0 || TBPM_DBG_OK(src_own - cur, n_units, TBPM_DBG_MARCH)))
+      copy_async<sizeof(PK)>(d_own + slot * slice_bytes, src_own, n_own);
+    if (rim && (n_rim == 0 || TBPM_DBG_OK(src_rim - cur, n_units, TBPM_DBG_MARCH)))
+      copy_async<sizeof(PK)>(d_rim + slot * slice_bytes, src_rim, n_rim);
     src_own += pstride;
     src_rim += pstride;
     ++zc;
   };
   PK m1{}, c0{};
-  if (own && (z0 > 0 || a.pbc_z)) m1 = cur[oo + (z0 > 0 ? z0 - 1 : Lz - 1) * pstride];
+  if (own && (z0 > 0 || a.pbc_z) && TBPM_DBG_OK(oo + (z0 > 0 ? z0 - 1 : Lz - 1) * pstride, n_units, TBPM_DBG_MARCH)) m1 = cur[oo + (z0 > 0 ? z0 - 1 : Lz - 1) * pstride];
   // phi_{n-1} and D of plane zo: each thread its own
   const PK* pp = prev + (own ? oo : 0) + z0 * pstride;
   const R* dp = diag ? diag + (own ? site : 0) + z0 * (a.Lx * a.Ly) : nullptr;
@@ -154,8 +157,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_cubic_march(MarchArgs a) {
   int zo = z0;
   auto copy_own = [&](int slot) {
     if (own && zo < z1) {
-      if (!FIRST) copy_async<sizeof(PK)>(d_prev + slot * (uint32_t)(kThreads * sizeof(PK)), pp, sizeof(PK));
-      if (diag) copy_async<sizeof(R)>(d_d + slot * (uint32_t)(kThreads * sizeof(R)), dp, sizeof(R));
+      if (!FIRST && TBPM_DBG_OK(pp - prev, n_units, TBPM_DBG_MARCH)) copy_async<sizeof(PK)>(d_prev + slot * (uint32_t)(kThreads * sizeof(PK)), pp, sizeof(PK));
+      if (diag && TBPM_DBG_OK(dp - diag, a.Lz * a.Lx * a.Ly, TBPM_DBG_MARCH)) copy_async<sizeof(R)>(d_d + slot * (uint32_t)(kThreads * sizeof(R)), dp, sizeof(R));
     }
     pp += pstride;
     dp += a.Lx * a.Ly;
@@ -223,8 +226,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_cubic_march(MarchArgs a) {
             acc[2 * q + 1] = fma2(o.c[q], c0.c[q], acc[2 * q + 1]);
           }
         }
-        if constexpr (sizeof(PK) == 16 && sizeof(R) == 4) __stcs(reinterpret_cast<float4*>(dst), *reinterpret_cast<const float4*>(&o));
-        else __stcs(reinterpret_cast<V2*>(dst), o.c[0]);
+        if (TBPM_DBG_OK(dst - out, n_units, TBPM_DBG_MARCH)) {
+          if constexpr (sizeof(PK) == 16 && sizeof(R) == 4) __stcs(reinterpret_cast<float4*>(dst), *reinterpret_cast<const float4*>(&o));
+          else __stcs(reinterpret_cast<V2*>(dst), o.c[0]);
+        }
         m1 = c0;
         c0 = p1;
       }
@@ -373,3 +378,5 @@ int launch_cubic_march(tbpm_ctx* ctx, const RecurrenceArgs& ra, int precision, b
 }
 
 }  // namespace tbpm
+
+TBPM_DEBUG_UNIT(march)

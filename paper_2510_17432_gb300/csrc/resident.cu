@@ -173,10 +173,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == kResThreads ? 2 : 1) k_resident(
     pub[li] = out;
   }
   const PK* x0 = reinterpret_cast<const PK*>(a.x0) + l0 * upr;
-  for (int u = tid; u < nu; u += NT) sA[u] = x0[u];
+  for (int u = tid; u < nu; u += NT)
+    if (TBPM_DBG_OK(l0 * upr + u, a.n_units, TBPM_DBG_RESIDENT)) sA[u] = x0[u];
   if (has_diag)
     for (int i = tid; i < (nu >> logP); i += NT)
-      sD[i] = reinterpret_cast<const R*>(a.diag)[(l0 * upr >> logP) + i];
+      if (TBPM_DBG_OK((l0 * upr >> logP) + i, g.n_full, TBPM_DBG_RESIDENT))
+        sD[i] = reinterpret_cast<const R*>(a.diag)[(l0 * upr >> logP) + i];
   __syncthreads();
   PK* cur = sA;
   PK* prv = sB;
@@ -212,6 +214,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == kResThreads ? 2 : 1) k_resident(
         if (t >= 0) take(cur[(int)t + off]);
         else if (t != -1) {
           const int64_t r = -(t + 2) + off;
+          if (!TBPM_DBG_OK(r, a.n_units, TBPM_DBG_RESIDENT)) return;
           if (first) take(reinterpret_cast<const PK*>(a.x0)[r]);
           else take(receive_or_zero<R, SPT>(pr_in + r * NP, tag, kResWaitNs, failed));
         }
@@ -254,7 +257,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == kResThreads ? 2 : 1) k_resident(
         for (int w = 0; w < 2 * SPT; ++w) o.v[w] = fma(d, ph.v[w], fma(th, h.v[w], -pv.v[w]));
       }
       prv[u] = o;
-      if (pub[li]) publish<R, SPT>(pr_out + (int64_t)u * NP, o, tag + 1);
+      if (pub[li] && TBPM_DBG_OK(l0 * upr + u, a.n_units, TBPM_DBG_RESIDENT))
+        publish<R, SPT>(pr_out + (int64_t)u * NP, o, tag + 1);
 #pragma unroll
       for (int k = 0; k < SPT; ++k) {
         const R pr = ph.v[2 * k], pi = ph.v[2 * k + 1];
@@ -420,3 +424,5 @@ int launch_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const RecurrenceArgs
 }
 
 }  // namespace tbpm
+
+TBPM_DEBUG_UNIT(resident)

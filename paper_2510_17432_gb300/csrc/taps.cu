@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kTapThreads, 2) k_taps_moment(RecurrenceArgs a
     const float4* src = colsrc + gy * rstride;
     unsigned dst = (unsigned)__cvta_generic_to_shared(tile + ty0 * RS + (c & 1) * TW + (c >> 1));
     for (int i = 0; i < ty1 - ty0; ++i, dst += (unsigned)(RS * sizeof(float4))) {
-      const bool ok = okx && i >= first && i < last;
+      const bool ok = okx && i >= first && i < last && TBPM_DBG_OK(src - cur, Ly * rstride, TBPM_DBG_TAPS);
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(ok ? src : cur), "r"(ok ? 16 : 0)
                    : "memory");
       src += rstride;
@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(kTapThreads, 2) k_taps_moment(RecurrenceArgs a
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
-        const bool in = o2 + i < ny && s < nx;
+        const bool in = o2 + i < ny && s < nx &&
+                        TBPM_DBG_OK(prev + (o2 + i) * rstep + s * P - po, Ly * rstep, TBPM_DBG_TAPS);
         pv[i][s] = !FIRST && in ? __ldcs(prev + (o2 + i) * rstep + s * P) : make_float4(0.f, 0.f, 0.f, 0.f);
         dd[i][s] = diag && in ? __ldg(diag + (o2 + i) * LS + s) : 0.f;
       }
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(kTapThreads, 2) k_taps_moment(RecurrenceArgs a
             out.z -= pv[i][s].z;
             out.w -= pv[i][s].w;
           }
-          next[o * rstep + s * P] = out;
+          if (TBPM_DBG_OK(prev + o * rstep + s * P - po, Ly * rstep, TBPM_DBG_TAPS)) next[o * rstep + s * P] = out;
           if constexpr (MOM) {
             t.x += ph.x * ph.x + ph.y * ph.y;
             t.y += out.x * ph.x + out.y * ph.y;
@@ -342,3 +343,5 @@ int build_tap_table(tbpm_lattice* lat) {
 }
 
 }  // namespace tbpm
+
+TBPM_DEBUG_UNIT(taps)

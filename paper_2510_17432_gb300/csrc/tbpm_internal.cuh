@@ -31,7 +31,11 @@ enum {
   TBPM_DBG_ELL = 2,         // ELL neighbour index against the site count
   TBPM_DBG_SWEEP_STORE = 3, // k_sweep_moments: output units
   TBPM_DBG_SWEEP_ROW = 4,   // k_sweep_moments: source range of a row copy
-  TBPM_DBG_SERVE = 5        // k_serve_step: neighbour units
+  TBPM_DBG_SERVE = 5,       // k_serve_step: neighbour units
+  TBPM_DBG_RESIDENT = 6,    // k_resident: own units, units and packets of other CTAs
+  TBPM_DBG_MARCH = 7,       // k_cubic_march: copied and stored units
+  TBPM_DBG_FLUSH = 8,       // k_flush: units of vectors and accumulators
+  TBPM_DBG_TAPS = 9         // k_taps_moment: staged and stored units
 };
 #ifdef TBPM_DEBUG
 static __device__ unsigned long long g_tbpm_dbg;
@@ -62,6 +66,10 @@ namespace tbpm {
 unsigned long long debug_take_cheb();
 unsigned long long debug_take_sweep();
 unsigned long long debug_take_serve();
+unsigned long long debug_take_resident();
+unsigned long long debug_take_march();
+unsigned long long debug_take_flush();
+unsigned long long debug_take_taps();
 #endif
 
 // ------------------------------------------------------------------ error reporting
