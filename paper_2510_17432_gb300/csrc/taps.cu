@@ -184,7 +184,6 @@ __global__ void __launch_bounds__(kTapThreads, 2) k_taps_moment(RecurrenceArgs a
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int o = o2 + i;
-      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);  // the row's |phi|^2 and Re <out|phi>, per state
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
         if (o < ny && s < nx) {
@@ -204,18 +203,12 @@ __global__ void __launch_bounds__(kTapThreads, 2) k_taps_moment(RecurrenceArgs a
           }
           if (TBPM_DBG_OK(prev + o * rstep + s * P - po, Ly * rstep, TBPM_DBG_TAPS)) next[o * rstep + s * P] = out;
           if constexpr (MOM) {
-            t.x += ph.x * ph.x + ph.y * ph.y;
-            t.y += out.x * ph.x + out.y * ph.y;
-            t.z += ph.z * ph.z + ph.w * ph.w;
-            t.w += out.z * ph.z + out.w * ph.w;
+            v[0] = add(v[0], sum_of(ph.x * ph.x + ph.y * ph.y));
+            v[1] = add(v[1], sum_of(out.x * ph.x + out.y * ph.y));
+            v[2] = add(v[2], sum_of(ph.z * ph.z + ph.w * ph.w));
+            v[3] = add(v[3], sum_of(out.z * ph.z + out.w * ph.w));
           }
         }
-      }
-      if constexpr (MOM) {
-        v[0] = add(v[0], sum_of(t.x));
-        v[1] = add(v[1], sum_of(t.y));
-        v[2] = add(v[2], sum_of(t.z));
-        v[3] = add(v[3], sum_of(t.w));
       }
     }
   }

@@ -361,7 +361,7 @@ struct AccumArgs {
   RecurrenceArgs r;     // recurrence part (cur, prev_out, lattice, reduction buffers)
   void* acc;            // accumulators [b][n_sites][S]
   int64_t acc_stride;   // elements (complex) between accumulators
-  const double* coef;   // [n_terms][b] complex (re, im) incl. the exp(-i H0 t) phase
+  const double* coef;   // [n_terms][b] complex (re, im)
   int b;
   int j_lo;             // first accumulator still active at this term
   int j_done;           // accumulator whose last term this is, or -1
