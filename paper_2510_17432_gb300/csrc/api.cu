@@ -415,11 +415,13 @@ __global__ void k_make_diag(int64_t n, const double* v64, double H0, double half
 }
 
 // ------------------------------------------------------------------ initial states
-// exp(2 pi i u / 2^32) * (sh + sl) in FP32 with an error below 0.5 ulp + 2^-10 ulp: the draw is reduced
-// exactly to a quarter turn (an integer below 2^29, split exactly into two floats), sin and cos
-// of the remainder |x| <= 1/4 (in units of pi) come from their Taylor series, whose first three
-// (sine) and four (cosine) terms are summed in float pairs (h + l) and the rest in FP32, where their
-// weight keeps the error below 2^-36, and the scale is applied to the pair before the one rounding.
+// exp(2 pi i u / 2^32) * (sh + sl) in FP32, and whether each part is surely the correctly rounded one.  The pair it
+// is rounded from is within 2^-14 ulp of the exact value (6e-5 over all 2^32 draws and ten scales), so it is unless
+// the pair lies within 2^-13 ulp of the middle between two floats.  The draw is reduced exactly to a quarter turn
+// (an integer below 2^29, split exactly into two floats), sin and cos of the remainder |x| <= 1/4 (in units of pi)
+// come from their Taylor series, whose first three (sine) and four (cosine) terms are summed in float pairs
+// (h + l) and the rest in FP32, where their weight keeps the error below 2^-36, and the scale is applied to the
+// pair before the one rounding.
 struct F2 {
   float h, l;
 };
@@ -430,7 +432,22 @@ __host__ __device__ __forceinline__ F2 pair_step(F2 c, F2 z, F2 s) {
   const float h = c.h + p;
   return {h, (c.h - h) + p + (c.l + e)};
 }
-__host__ __device__ __forceinline__ float2 unit_phase(uint32_t u, float sh, float sl) {
+// c scaled by sh + sl and rounded; *sure is cleared next to a tie (and for zero and powers of two, whose
+// neighbours are not symmetric)
+__host__ __device__ __forceinline__ float scaled(F2 c, float sh, float sl, bool* sure) {
+  const float lo = fmaf(c.h, sl, c.l * sh);
+  const float v = fmaf(c.h, sh, lo);
+  const float p = c.h * sh;
+  const float r = (p - v) + (fmaf(c.h, sh, -p) + lo);  // what the rounding left, at most half an ulp
+  uint32_t b;
+  memcpy(&b, &v, 4);
+  const uint32_t e = b & 0x7f800000u, half_bits = e - (24u << 23);
+  float half;
+  memcpy(&half, &half_bits, 4);
+  if ((b & 0x007fffffu) == 0 || e < (64u << 23) || fabsf(r) > half * (1.f - 0x1p-12f)) *sure = false;
+  return v;
+}
+__host__ __device__ __forceinline__ float2 unit_phase(uint32_t u, float sh, float sl, bool* sure) {
   const uint32_t q = (u + 0x20000000u) >> 30;
   const int r = (int)(u - (q << 30));  // [-2^29, 2^29)
   const float xi = (float)r;
@@ -455,15 +472,16 @@ __host__ __device__ __forceinline__ float2 unit_phase(uint32_t u, float sh, floa
   c = pair_step({4.05871201f, 1.20801531e-07f}, z, c);
   c = pair_step({-4.93480206f, -1.45185794e-07f}, z, c);
   c = pair_step({1.f, 0.f}, z, c);
-  const float cs = fmaf(c.h, sh, fmaf(c.h, sl, c.l * sh));
-  const float sn = fmaf(s.h, sh, fmaf(s.h, sl, s.l * sh));
+  const float cs = scaled(c, sh, sl, sure);
+  const float sn = scaled(s, sh, sl, sure);
   const float a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;  // quarter turns: (c, s), (-s, c), (-c, -s), (s, -c)
   return make_float2((q == 1 || q == 2) ? -a : a, q >= 2 && q < 4 ? -b : b);
 }
 
 // Random phases psi_i = exp(2 pi i u / 2^32) / sqrt(N), u = Philox(state_seed; i, 2, s).
-// complex64 is bound by the draw (integer multiplies) and FP32 issue: 537M states take 3.2 ms against 31.1 ms
-// with FP64 sincospi (GB300 issues two FP64 operations per clock and SM), which complex128 keeps.
+// complex64 is bound by the draw (integer multiplies) and FP32 issue: 537M states take 3.5 ms against 31.1 ms
+// with FP64 sincospi (GB300 issues two FP64 operations per clock and SM), which complex128 keeps and which settles
+// the one draw in 2000 that lies next to a tie, so that every state is the FP64 one rounded once.
 template <typename R>
 __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint64_t seed, const int64_t* full_of,
                               const float* masked, double inv_sqrt_n, R* out, uint32_t* draws) {
@@ -478,9 +496,16 @@ __global__ void k_init_random(int64_t n, int Spad, int logS, int S, int s0, uint
       const int64_t f = full_of ? full_of[k] : k;
       const uint32_t u = draw_u32(seed, (uint64_t)f, STREAM_PHASE, (uint32_t)(s0 + s));
       if constexpr (sizeof(R) == 4) {
-        const float2 v = unit_phase(u, sh, sl);
+        bool sure = true;
+        const float2 v = unit_phase(u, sh, sl, &sure);
         re = v.x;
         im = v.y;
+        if (!sure) {
+          double sn, cs;
+          sincospi((double)u * 0x1p-31, &sn, &cs);
+          re = (R)(cs * inv_sqrt_n);
+          im = (R)(sn * inv_sqrt_n);
+        }
       } else {
         double sn, cs;
         sincospi((double)u * 0x1p-31, &sn, &cs);
