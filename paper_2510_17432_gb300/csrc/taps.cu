@@ -51,7 +51,7 @@ constexpr int kTapRB = 4;                        // row blocks per tile
 constexpr int kTapTY = kTapWin * kTapRB;         // rows per tile
 constexpr int kTapTX = 64;                       // cells per tile along x (two warps)
 constexpr int kTapThreads = kTapTX * kTapRB;
-constexpr int kTapMaxSmem = 227 * 1024;
+constexpr int kTapMaxSmem = 226 * 1024;         // beside the sums' static shared memory
 constexpr int kTapStage = 5;                     // groups of rows the staging is split into
 
 __device__ __forceinline__ int64_t tap_wrap(int64_t v, int64_t L, int periodic, bool* ok) {
@@ -269,7 +269,8 @@ static int launch_taps(tbpm_ctx* ctx, const RecurrenceArgs& a, bool first, bool 
   }
   void* fn = first ? (mom ? (void*)k_taps_moment<true, true> : (void*)k_taps_moment<true, false>)
                    : (mom ? (void*)k_taps_moment<false, true> : (void*)k_taps_moment<false, false>);
-  TBPM_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit is the kernel's, not the launch's: another thread's smaller lattice must not lower it in between
+  TBPM_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTapMaxSmem));
   RecurrenceArgs aa = a;
   void* args[] = {&aa, const_cast<TapTable*>(a.taps)};
   const cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTapThreads), args, smem, ctx->stream);

@@ -377,3 +377,36 @@ def test_fp32_fma_peak_is_a_plausible_device_rate(capi, ctx):
     scalar, packed = capi.tbpm_fp32_fma_peak(ctx)
     bound = sms * 128 * 2 * 3.0e9 / 1e12
     assert 0.0 < scalar < bound and 0.0 < packed < 2 * bound, (scalar, packed, bound)
+
+
+def test_two_contexts_with_different_tiles_at_once(capi):
+    """Two threads, a context each, tiles of 107 KB and 33 KB: the kernel's shared-memory limit is the device's, so
+    neither lattice's launches lower it under the other's."""
+    import threading
+    out, failed = {}, []
+
+    def work(name, cutoff):
+        try:
+            h = capi.tbpm_create(0)
+            lat = capi.tbpm_lattice_create(h, capi.lattice_desc(1, (70, 36), t=-2.7, cutoff=cutoff, decay=0.3187))
+            capi.tbpm_set_graphs(h, False)
+            req = capi.request(n_states=2, n_moments=400, state_seed=3)
+            runs = []
+            for _ in range(6):
+                mu = np.zeros((2, 400, 2))
+                capi.tbpm_moments(h, lat, req, mu)
+                runs.append(mu)
+            out[name] = runs
+            capi.tbpm_lattice_destroy(lat)
+            capi.tbpm_destroy(h)
+        except Exception as e:  # reported by the main thread
+            failed.append((name, str(e)))
+
+    threads = [threading.Thread(target=work, args=a) for a in (("wide", 9.7), ("narrow", 1.8))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    for runs in out.values():
+        assert all(np.array_equal(r, runs[0]) for r in runs)
