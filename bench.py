@@ -595,8 +595,8 @@ def run_gpu(args, work):
                      np.max(np.abs(res["sequential"][2])))
         block = float(info.n_sites) * S * elem
         fused = args.fusion in FUSION_STEPS and FUSION_STEPS[args.fusion] == 4 and spec.kind == wl.HONEYCOMB
-        conc_blocks = concurrent_m_blocks(Mtot, fused)
-        seq_blocks = Nt * sequential_step_blocks(Ntrunc, fused)
+        conc_blocks = sweep_moment_blocks(Mtot) if fused else concurrent_m_blocks(Mtot, False)
+        seq_blocks = Nt * (sweep_step_blocks(Ntrunc) if fused else sequential_step_blocks(Ntrunc, False))
         peak, _ = measured_hbm_peak()
         out["sequential"] = {
             "n_steps": Nt, "tau": "pi", "dos": "Hann-windowed Fourier DOS on 512 energies",
@@ -610,9 +610,9 @@ def run_gpu(args, work):
             "hbm_frac_concurrent": conc_blocks * block / res["concurrent_m"][0] / 1e9 / peak,
             "hbm_frac_sequential": seq_blocks * block / res["sequential"][0] / 1e9 / peak,
             "bytes_model": "state blocks of N x S x 8 B crossing HBM: concurrent = moment passes (4 per "
-                           "four-step pass, 3 per one-step pass); sequential = per time step the buffered "
-                           "time block of the library (copy, first step, four-term window passes writing 4 "
-                           "slots, one-step passes, one flush reading every term, <psi|psi(t)>, carry)",
+                           "four-step pass, the first reads and the last writes fewer); sequential = per time "
+                           "step the buffered time block of the library (copy into the first slot, four-term "
+                           "window passes, one flush reading every term and writing the state, <psi|psi(t)>)",
             "site_updates_per_s_sequential": seq_su / res["sequential"][0],
             "site_updates_per_s_concurrent": conc_su / res["concurrent_m"][0],
             "max_rel_dos_difference": diff}
@@ -671,7 +671,7 @@ def concurrent_m_blocks(n_moments: int, fused: bool) -> float:
 
 
 def sequential_step_blocks(n_terms: int, fused: bool) -> float:
-    """State-block crossings of one sequential time step as the library buffers it (b = 1):
+    """State-block crossings of one sequential time step, the buffered form in single steps (b = 1):
     clear the accumulator, copy psi(t) into the first slot, the first term H~ phi_0, four-term
     window passes (read 2, write 4) while four terms fit, one-step passes (read 2, write 1) for
     the rest, one flush (read every term, read and write the accumulator), <psi|psi(t)> (2) and
@@ -684,6 +684,23 @@ def sequential_step_blocks(n_terms: int, fused: bool) -> float:
             n += 4
     blocks += 3 * (n_terms - n)
     return blocks + n_terms + 2 + 2 + 2
+
+
+def sweep_moment_blocks(n_moments: int) -> float:
+    """The same where the register sweep takes every step: initialisation writes phi_0, the first
+    pass reads it alone and writes two blocks, the passes between read two and write two, the last
+    one stores no state."""
+    steps = (n_moments + (n_moments & 1)) // 2
+    passes = (steps + 3) // 4
+    return 1 + (1 if passes == 1 else 3 + 4 * (passes - 2) + 2)
+
+
+def sweep_step_blocks(n_terms: int) -> float:
+    """State-block crossings of one sequential time step (b = 1) where the register sweep applies:
+    copy of psi(t) into the first slot (2), window passes of up to four terms (read two, the first
+    one; write each term), one flush (read every term, write the state), <psi|psi(t)> (2)."""
+    passes = (n_terms - 1 + 3) // 4
+    return 2 + 2 * passes - 1 + (n_terms - 1) + n_terms + 1 + 2
 
 
 # ---------------------------------------------------------------- state-based correlation (vacancy lattices)

@@ -1,5 +1,6 @@
 // Resident moment recurrence: every Chebyshev step of a request in one cooperative launch, for lattices
-// whose two state blocks fit in the SMs' shared memory (up to about 15 MB a block, 2M complex64 site-states).
+// whose two state blocks fit in the SMs' shared memory (up to about 15 MB a block, 2M complex64 site-states;
+// use_resident says which of them).
 //
 // One launch per step costs 6 to 8 us on a small lattice (launch, cold L1, the grid reduction's tail),
 // whatever its size.  Here a CTA owns a run of lattice lines (x-lines of the [row][site][state] layout) for
@@ -23,7 +24,7 @@
 // Bound: the exchange latency per step (a packet's way through L2 to the polling thread) for small lattices; shared-memory
 // bandwidth (complex64) or FP64 issue (complex128) when the blocks are large.  Measured, us per step, one
 // launch per step -> resident: 64 x 64 square, complex128, one state 6.6 -> 2.1; 45 x 47 honeycomb, 4 states
-// 8.1 -> 2.0; 40^3 cubic, 8 states 23.8 -> 7.5; 300 x 300 honeycomb, 8 states 25.8 -> 8.8.
+// 8.1 -> 2.0; 40^3 cubic, 8 states 23.8 -> 7.5.
 #include <cuda_runtime.h>
 #include <string.h>
 

@@ -42,8 +42,12 @@ constexpr int kServeTU = 16 * kThreads;  // largest tile (16 units per thread, F
 constexpr int kItemCache = 128;
 constexpr int64_t kLaneSiteStates = 1 << 21;  // full sites x padded states of a direct-lane request
 
-// Units per tile of a request with `units` thread units: 16 per thread (the per-tile reduction
-// and bookkeeping amortised; 32 left the last of two waves of tiles nearly empty) unless the request would get fewer than 64 tiles, then fewer.
+// Units per tile of a request with `units` thread units: 16 per thread, fewer where the request would get fewer
+// than 64 tiles.  Fewer units mean more of the per-tile reduction and bookkeeping, more units emptier last waves,
+// and how full those are depends on the mix: eight drawn mixes of 3 to 16 requests took (ms, 8 / 16 / 32 units)
+// 35.8 / 35.2 / 39.3, 24.8 / 20.3 / 15.7, 15.3 / 13.8 / 14.0, 17.6 / 17.7 / 19.4, 29.2 / 25.6 / 23.4,
+// 37.7 / 32.7 / 35.6, 29.2 / 27.2 / 30.5 and 6.3 / 6.2 / 6.3; 16 is the best of three on five of them and 1.4 %
+// ahead of 32 in the geometric mean (the version before the deferred sums: 48.4, 26.8, 21.1, 27.3, 35.6, 59.4, 46, 8.4).
 // Depends only on the request, so its partial sums (and results) are the same alone and in any mix.
 __host__ __device__ inline int serve_tile_units(int64_t units) {
   int upt = 1;
@@ -185,7 +189,7 @@ __device__ void serve_tile(const ServeItem* itp, int64_t lt, int step, double (*
     }
   }
 
-  // tile partial sums: FP32 (at most 32 units per thread), compensated over the lanes, FP64 over the warps
+  // tile partial sums: FP32 (at most kServeTU / kThreads units per thread), compensated over the lanes, FP64 over the warps
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   decltype(sum_of(R(0))) v[2 * SPT];
 #pragma unroll

@@ -205,7 +205,7 @@ struct tbpm_ctx {
   // cached workspaces (grow-only, stream-ordered allocations)
   tbpm::DevBuf ws_phi[2], ws_psi, ws_acc, ws_partials, ws_counter, ws_mu, ws_table, ws_aux, ws_out,
       ws_energies, ws_recon, ws_phi2[2], ws_fused_partials, ws_qe, ws_qe_coef, ws_xdot, ws_jpsi, ws_ec, ws_fermi, ws_blk, ws_blk_coef;
-  // time blocks buffer up to 32 Chebyshev vectors and flush them into the accumulators at once
+  // time blocks buffer up to flush_max_terms() Chebyshev vectors and flush them into the accumulators at once
   bool buffer_blocks = true;
   int fusion = 8;  // temporal-fusion mode of the moment pass (8 = four-step register sweep; -1 = autotuned)
   bool resident = true;  // small lattices in one resident launch, until a mode is chosen (tbpm_set_resident)

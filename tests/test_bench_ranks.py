@@ -100,3 +100,13 @@ def test_byte_models_of_the_two_forms():
     assert n_pi == 20
     assert bench.concurrent_m_blocks(4096, True) == 2056
     assert 1254 * bench.sequential_step_blocks(n_pi, True) == 76494
+
+
+def test_sweep_byte_models():
+    """The register sweep's own counts: 627 steps (157 passes) of the benchmark's Fourier DOS, and a sequential step
+    of N(pi) = 20 terms through five window passes: 2 + 9 + 19 + 20 + 1 + 2."""
+    import bench
+    assert bench.sweep_moment_blocks(8) == 1 + 1
+    assert bench.sweep_moment_blocks(1254) == 1 + 3 + 4 * 155 + 2
+    assert bench.sweep_step_blocks(20) == 53
+    assert bench.sweep_step_blocks(5) == 2 + 1 + 4 + 5 + 1 + 2
