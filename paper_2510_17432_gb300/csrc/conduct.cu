@@ -116,7 +116,8 @@ struct XdotArgs {
 // A product conj(a) b is two packed f32x2 FMAs, (ar, ai) (br, bi) and (ar, ai) (bi, -br), whose halves are
 // added at the fold.  Every 16 units the 32 sums are reduce-scattered over the lanes of a state pair
 // (31 shuffles instead of 160 for a tree per sum) and each lane adds the ones it keeps in FP64.
-// Bound: L1 and FP32 issue for many pairs, HBM for one block against a few.  On 2.1M sites 16 x 64 blocks
+// Bound: the latency of the 8- and 16-byte loads at 16 warps an SM for many pairs (long scoreboard 11.7 cycles per
+// instruction, L1 at 21 %, FMA pipe at 26 %), HBM for one block against a few.  On 2.1M sites 16 x 64 blocks
 // took 3320 us with a shuffle tree per sum and scalar FMAs, now 1206 us.
 struct XTile {
   int at, bt;   // tiles along A and B
