@@ -1440,19 +1440,19 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
   ctx->queue_live[k] = true;
 }
 
-// Whether the resident kernel runs this moment request: a small lattice, unless a fusion mode has been chosen
-// since (tbpm_set_resident).  Where the register sweep takes the lattice as
-// well, the resident kernel is faster alone, but its grid must be resident as a whole: requests of several
-// contexts overlap only as far as several grids fit, while sweeps and one-step passes fill each other's gaps.
-// Requests of 512 moments a second from one and from eight contexts, one-step or sweep before -> resident:
-// honeycomb pairs 64 x 64 x 8 states 506 / 3591 -> 1292 / 3962, 100 x 100 x 4 693 / 4737 -> 1379 / 3225,
-// 250 x 250 x 8 247 / 849 -> 493 / 503 (sweep now 302 / 998).  So honeycomb pairs, which had the sweep, go
-// resident up to 70,000 site-states, where no number of contexts is slower; other kinds gained at both
-// ends (300 x 300 square, 8 states 156 / 361 -> 566 / 812) but for complex128 honeycombs, whose FP64 time does not
-// overlap: 160 x 160 x 4 states 160 / 340 -> 216 / 260, so four states and more stop at 90,000 (below it, two
-// states on 110 x 110 cells 438 / 1294 -> 951 / 1043; four contexts 960 -> 1036).  Blocks of one or two states leave the shared-memory
-// reads half empty and stop where the sweep is as fast alone (us per step, resident / sweep: two states
-// 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1 / 2.9).
+// Whether the resident kernel runs this moment request: a small lattice, unless a fusion mode has been chosen since
+// (tbpm_set_resident).  Where the register sweep takes the lattice as well, the resident kernel is faster alone,
+// but its grid must be resident as a whole: requests of several contexts overlap only as far as several grids fit,
+// while sweeps and one-step passes fill each other's gaps. Requests of 512 moments a second from one and from eight
+// contexts, one-step or sweep before -> resident: honeycomb pairs 64 x 64 x 8 states 506 / 3591 -> 1292 / 3962, 100
+// x 100 x 4 693 / 4737 -> 1379 / 3225, 250 x 250 x 8 247 / 849 -> 493 / 503 (sweep now 302 / 998).  So honeycomb
+// pairs, which had the sweep, go resident up to 70,000 site-states, where no number of contexts is slower; other
+// kinds gained at both ends (300 x 300 square, 8 states 156 / 361 -> 566 / 812) but for complex128 honeycombs,
+// whose FP64 time does not overlap: 160 x 160 x 4 states 160 / 340 -> 216 / 260, so four states and more stop at
+// 90,000 (below it, two states on 110 x 110 cells 438 / 1294 -> 951 / 1043; four contexts 960 -> 1036).  Blocks of
+// one or two states leave the shared-memory reads half empty and stop where the sweep is as fast alone (us per
+// step, resident / sweep: two states 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1
+// / 2.9).
 bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
   if (ctx->lean || !ctx->resident) return false;
   if (fused_applicable(lat, pl.precision, pl.Spad) && pl.n * pl.Spad > 70000) return false;
@@ -1771,8 +1771,8 @@ int choose_block(tbpm_ctx* ctx, tbpm_lattice* lat, const tbpm_request* req, cons
 
 // State-based propagation in blocks of b steps; b = 1 is the sequential form.
 // d_C [Spad][n_steps+1][2].  The hook sees each finished time block: psi~(t_{start+1}) ..
-// psi~(t_{start+bb}) as bb consecutive state blocks, without the common factor: psi(t) = e^{-i H0 t} psi~(t).  init (device, optional) replaces the
-// request's initial states.
+// psi~(t_{start+bb}) as bb consecutive state blocks, without the common factor:
+// psi(t) = e^{-i H0 t} psi~(t).  init (device, optional) replaces the request's initial states.
 using BlockHook = std::function<int(int64_t /*start*/, int /*bb*/, const void* /*first state block*/)>;
 
 // The Chebyshev vectors phi_0 .. phi_{n_terms-1} in windows of T buffer slots: slot 2 holds phi_0 on

@@ -103,8 +103,8 @@ def test_byte_models_of_the_two_forms():
 
 
 def test_sweep_byte_models():
-    """The register sweep's own counts: 627 steps (157 passes) of the benchmark's Fourier DOS, and a sequential step
-    of N(pi) = 20 terms through five window passes: 2 + 9 + 19 + 20 + 1 + 2."""
+    """The register sweep's own counts: 1254 moments in 627 steps (157 passes), and a sequential step of N(pi) = 20
+    terms through five window passes: 2 + 9 + 19 + 20 + 1 + 2."""
     import bench
     assert bench.sweep_moment_blocks(8) == 1 + 1
     assert bench.sweep_moment_blocks(1254) == 1 + 3 + 4 * 155 + 2
