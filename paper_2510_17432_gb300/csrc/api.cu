@@ -1449,13 +1449,15 @@ void throttle_queue(tbpm_ctx* ctx, bool capturing) {
 // pairs, which had the sweep, go resident up to 70,000 site-states, where no number of contexts is slower; other
 // kinds gained at both ends (300 x 300 square, 8 states 156 / 361 -> 566 / 812) but for complex128 honeycombs,
 // whose FP64 time does not overlap: 160 x 160 x 4 states 160 / 340 -> 216 / 260, so four states and more stop at
-// 90,000 (below it, two states on 110 x 110 cells 438 / 1294 -> 951 / 1043; four contexts 960 -> 1036).  Blocks of
-// one or two states leave the shared-memory reads half empty and stop where the sweep is as fast alone (us per
-// step, resident / sweep: two states 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1
-// / 2.9).
+// 90,000 (below it, two states on 110 x 110 cells 438 / 1294 -> 951 / 1043; four contexts 960 -> 1036).  Cubic
+// lattices near the kernel's limit gain little alone and lose from eight contexts (60^3, 8 states: one step per
+// launch before 259 / 476, resident 377 / 399, march 322 / 767), so they stop at 1.5M. Blocks of one or two states
+// leave the shared-memory reads half empty and stop where the sweep is as fast alone (us per step, resident /
+// sweep: two states 819k site-states 5.5 / 6.1, 1.44M 7.5 / 7.0; one state 262k 4.5 / 4.3, 33k 2.1 / 2.9).
 bool use_resident(tbpm_ctx* ctx, const tbpm_lattice* lat, const Plan& pl, int64_t steps) {
   if (ctx->lean || !ctx->resident) return false;
   if (fused_applicable(lat, pl.precision, pl.Spad) && pl.n * pl.Spad > 70000) return false;
+  if (lat->geom.kind == TBPM_CUBIC && pl.n * pl.Spad > 1500000) return false;
   if (pl.precision == TBPM_C128 && lat->geom.kind == TBPM_HONEYCOMB && pl.Spad >= 4 && pl.n * pl.Spad > 90000) return false;
   if (pl.Spad <= 2 && pl.n * pl.Spad > (pl.Spad == 1 ? 200000 : 1000000) && sweep_ok(lat, pl)) return false;
   return resident_applicable(ctx, lat, pl.precision, pl.Spad, steps);
